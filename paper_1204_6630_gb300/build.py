@@ -1,6 +1,6 @@
 """Build the CUDA library ``libtpcf.so`` in-tree with nvcc for sm_103a.
 
-The translation units (the counting kernel, catalog preparation, host
+The translation units (the counting kernels, catalog preparation, host
 runtime, job server, the no-allocation entry point, the FP32 peak
 measurement) are compiled in
 parallel and linked into ``paper_1204_6630_gb300/_build/libtpcf.so``.  Host
@@ -20,7 +20,7 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(BUILD, "libtpcf.so")
-SOURCES = ["count.cu", "prep.cu", "runtime.cpp", "server.cpp", "noalloc.cu", "peak.cu"]
+SOURCES = ["count.cu", "count_tc.cu", "prep.cu", "runtime.cpp", "server.cpp", "noalloc.cu", "peak.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 
@@ -49,7 +49,7 @@ def _stale(out: str, deps: list[str]) -> bool:
 def build(force: bool = False, verbose: bool = False) -> str:
     """Compile (if any source changed) and return the path of libtpcf.so."""
     os.makedirs(BUILD, exist_ok=True)
-    headers = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".h")]
+    headers = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".h", ".cuh"))]
     headers.append(os.path.join(ROOT, "include", "tpcf.h"))
     srcs = [os.path.join(CSRC, s) for s in SOURCES]
     if not force and not _stale(LIB, srcs + headers + [__file__]):

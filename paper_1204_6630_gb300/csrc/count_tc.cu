@@ -1,0 +1,646 @@
+// CUDA counting kernel (sm_103a) whose screen runs on the tensor cores.
+//
+// Paper: Ponce et al., "Application of GPUs for the calculation of two point
+// correlation functions in cosmology", Section 3: the dot product of each
+// pair, its bin, partial histograms combined into one.  Here the dot products
+// of a block of pairs are one small matrix product, which serves only to
+// reject: a 32 x 32 block of pairs none of which can lie within the last edge
+// is overflow and needs nothing more.  Every other block is classified as in
+// count.cu: FP32 screen value, lookup table, chord refinement, binary64.
+//
+// The screen as a contraction.  The FP32 coordinates are split into two
+// binary16 values, a = a1 + a2 + r with |r| <= 2^-22 |a| + 2^-25, and a pair's
+// screen value is the K = 16 product
+//   D = sum_c a1 b1 + a2 b2 + a1 b2 + a2 b1,   c = x, y, z:
+// the i-side record is [X | X] and the j-side record [X | Y] with X = (x1, y1,
+// z1, x2, y2, z2, 0, 0) and Y = (x2, y2, z2, x1, y1, z1, 0, 0).  Products of
+// binary16 values are exact in binary32; with accumulation in at least single
+// precision D is within 44u of the binary64 dot d (u = 2^-24: 2u from the FP32
+// copies, 9.8u from the split, at most one unit 2u in the last place for each
+// of 16 additions of partial sums below 1.002).  A block is rejected when
+// every D < tc_thr = RD(C_B - 64u), which proves d < C_B for all its pairs.
+//
+// One CTA per SM, 21 warps:
+//   * warps 0..15, four groups of four: group g reads the accumulators of
+//     i-points 128 g .. 128 g + 127 of the CTA's 512 (tcgen05.ld with a maximum
+//     over 32 columns: one comparison per 32 x 32 pairs), releases them, and
+//     classifies the blocks it kept, one i-point per lane;
+//   * warps 16..19: group g's tcgen05.mma issuer (M 128 x N 128 x K 16);
+//   * warp 20: draws items (512 i-points x a j-chunk), finds the tiles and
+//     groups that can hold countable pairs, and copies operands with TMA.
+// The j-tiles (operand and FP32 coordinates, one bulk copy) are shared by the
+// four groups; a group that is busy classifying holds back its own
+// accumulators only, and the others run up to the ring's depth ahead.
+#include <stdint.h>
+
+#include "count_common.cuh"
+
+namespace tpcf {
+
+namespace {
+
+constexpr int kWorkWarps = 16;                    // classifying warps
+constexpr int kWorkThreads = 32 * kWorkWarps;
+constexpr int kGroups = 4;                        // groups of four warps: 128 i-points each
+constexpr int kIssueWarp = kWorkWarps;            // .. + kGroups - 1: the groups' mma issuers
+constexpr int kLoadWarp = kWorkWarps + kGroups;
+constexpr int kThreads = 32 * (kLoadWarp + 1);
+constexpr int kTmemCols = 512;                    // 128 columns per group
+constexpr uint32_t kABytes = 4 * kOpABlock;       // i-side operand of an item (512 points)
+constexpr int kQueueCodes = 64;                   // per-warp queue of unsettled pairs
+
+enum TcCtl { kTcAbort = 0, kTcTmem = 1, kTcTake = 2, kTcCtlWords = 32 };
+
+// A staged tile: first i of the item, first j of the tile, and what to do with it.
+struct TcMeta {
+    uint32_t i0, jbase;
+    uint32_t info;   // kInfo* below, sub-problem in bits 16..31
+    uint32_t pad;
+};
+enum : uint32_t {
+    kInfoGroups = 0xfu,   // groups with countable pairs in this tile
+    kInfoABuf = 0x10u,    // operand buffer of the item
+    kInfoNew = 0x20u,     // first tile of an item
+    kInfoLast = 0x40u,    // last tile of an item
+    kInfoStop = 0x80u,    // no tile: the launch's (or slice's) items are done
+};
+
+// Barriers (8 bytes each): full[S], empty[S], a_full[2], a_empty[2], d_full[4], d_free[4].
+__host__ __device__ constexpr uint32_t tc_bar_words(uint32_t S) { return 2 * S + 4 + 2 * kGroups; }
+
+struct TcLayout {
+    uint32_t ctl, bars, meta, atile, stage, hist, cos_thr, lo, hi, cos32, zlo, zhi, lut, queue, bwd, total;
+};
+
+__host__ __device__ inline TcLayout tc_layout(int S, int nedges) {
+    TcLayout L;
+    uint32_t off = 0;
+    L.ctl = off; off += kTcCtlWords * 4;
+    L.bars = off; off += tc_bar_words((uint32_t)S) * 8;
+    off = align_up(off, 16);
+    L.meta = off; off += (uint32_t)S * (uint32_t)sizeof(TcMeta);
+    off = align_up(off, 128);
+    L.atile = off; off += 2 * kABytes;
+    L.stage = off; off += (uint32_t)S * kOpBBlock;
+    L.hist = off; off += (uint32_t)(nedges + 1) * (uint32_t)(kWorkThreads / 2) * 4;
+    off = align_up(off, 16);
+    L.cos_thr = off; off += (uint32_t)nedges * 8;
+    L.lo = off; off += (uint32_t)nedges * 4;
+    L.hi = off; off += (uint32_t)nedges * 4;
+    L.cos32 = off; off += (uint32_t)nedges * 4;
+    L.zlo = off; off += (uint32_t)nedges * 4;
+    L.zhi = off; off += (uint32_t)nedges * 4;
+    off = align_up(off, 16);
+    L.lut = off; off += (uint32_t)kLutCells * 2;
+    off = align_up(off, 16);
+    L.queue = off; off += (uint32_t)kWorkWarps * kQueueCodes * 4;
+    off = align_up(off, 16);
+    L.bwd = off; off += (uint32_t)sizeof(WorkDesc);
+    L.total = align_up(off, 16);
+    return L;
+}
+
+// ============================================================== tcgen05 wrappers
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
+}
+
+__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+
+// Shared-memory matrix descriptor of a K-major operand without swizzle: rows
+// in groups of 8, a group's two 8 x 16-byte core matrices at `addr` + 0 and
+// + 2048 (the X and the second plane of 128 points), groups 128 bytes apart.
+__device__ __forceinline__ uint64_t op_desc(uint32_t addr) {
+    return (uint64_t)((addr >> 4) & 0x3fffu) | ((uint64_t)(2048u >> 4) << 16) | ((uint64_t)(128u >> 4) << 32) |
+           (1ull << 46);
+}
+
+// D (FP32, 128 x 128) = A B^T, K = 16, binary16 operands; issued by one thread.
+constexpr uint32_t kIdesc = (1u << 4) | ((128u >> 3) << 17) | ((128u >> 4) << 24);
+__device__ __forceinline__ void tc_mma(uint32_t d, uint64_t a, uint64_t b) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, 0, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+        "l"(a), "l"(b), "r"(kIdesc)
+        : "memory");
+}
+__device__ __forceinline__ void tc_commit(uint64_t* bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_addr(bar))
+                 : "memory");
+}
+
+// Maximum over 32 columns of the lane's accumulator row (the loaded values
+// themselves are not used).  The result is valid after tc_wait_ld.
+__device__ __forceinline__ float tc_row_max32(uint32_t addr) {
+    uint32_t r[32];
+    float m;
+    asm volatile(
+        "tcgen05.ld.red.sync.aligned.32x32b.x32.max.f32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
+        "%14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, %32, [%33];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
+          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31]),
+          "=f"(m)
+        : "r"(addr));
+    return m;
+}
+// Waits for the warp's tensor-memory loads; the operands tie the loaded maxima to the wait.
+__device__ __forceinline__ void tc_wait_ld(float& a, float& b) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;" : "+f"(a), "+f"(b)::"memory");
+}
+
+// Bounded wait of a whole warp for phase `parity` of `bar`: false (with the
+// block's abort word and the call's error word set) after limit_ns, and false
+// as soon as another warp has aborted.
+__device__ __noinline__ bool tc_wait_slow(uint64_t* bar, uint32_t parity, uint64_t limit_ns, volatile int* ctl,
+                                          unsigned long long* stats) {
+    const uint64_t t0 = global_ns();
+    bool ok = false;
+    while (true) {
+        ok = mbar_try_wait(bar, parity);
+        if (ok || ctl[kTcAbort]) break;
+        if (global_ns() - t0 > limit_ns) {
+            ctl[kTcAbort] = 1;
+            atomicOr(stats + kStatError, (unsigned long long)kErrWaitTimeout);
+            break;
+        }
+    }
+    return __all_sync(0xffffffffu, ok);
+}
+__device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity, uint64_t limit_ns, volatile int* ctl,
+                                        unsigned long long* stats) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    return tc_wait_slow(bar, parity, limit_ns, ctl, stats);
+}
+
+// ============================================================== classification of a kept block
+// One i-point per lane (as (a, a) pairs) against 32 staged j-points: FP32
+// screen value, LUT code, one counter increment per settled pair, as the slow
+// path of count.cu (the codes of a group of four j are read before the
+// increments of the group before it).  `valid` (MASKED) names the lane's pairs
+// that may be counted.  Returns the unsettled pairs: pair j at bit 31 - j.
+template <bool MASKED>
+__device__ __forceinline__ uint32_t tc_block(const WorkDesc& wd, u64 ax, u64 ay, u64 az, const float* sx,
+                                             uint32_t valid, const HistCol& hc) {
+    const uint32_t lut_adj = smem_addr(dyn_smem) + wd.off_lut - 0x4B000000u * 2u;
+    const u64 nt2 = wd.neg_fast_t2;
+    uint32_t ent[2][4];
+    uint32_t um = 0;
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        if (k < 8) {
+            const ulonglong2 bx = *reinterpret_cast<const ulonglong2*>(sx + 4 * k);
+            const ulonglong2 by = *reinterpret_cast<const ulonglong2*>(sx + kOpBlock + 4 * k);
+            const ulonglong2 bz = *reinterpret_cast<const ulonglong2*>(sx + 2 * kOpBlock + 4 * k);
+            const u64 v0 = ffma2(az, bz.x, ffma2(ay, by.x, ffma2(ax, bx.x, nt2)));
+            const u64 v1 = ffma2(az, bz.y, ffma2(ay, by.y, ffma2(ax, bx.y, nt2)));
+            const float e[4] = {lo_of(v0), hi_of(v0), lo_of(v1), hi_of(v1)};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float v = __saturatef(e[u] * wd.lut_scale);
+                const float f = fmaf(v, 16384.0f, 8388608.0f);
+                asm volatile("ld.shared.s16 %0, [%1];" : "=r"(ent[k & 1][u]) : "r"(__float_as_uint(f) * 2u + lut_adj));
+            }
+        }
+        if (k >= 1) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                uint32_t x = ent[(k - 1) & 1][u];
+                if constexpr (MASKED) x = ((valid >> (4 * (k - 1) + u)) & 1u) ? x : kLutSkip;
+                if (x < kLutRowLimit) red_add_shared(hc.addr + (x << row_shift<kWorkThreads>()), hc.inc);
+                um = __funnelshift_l(x, um, 1);
+            }
+        }
+    }
+    return um;
+}
+
+// Classifies the n <= 32 queued pairs at q, one per lane: code = lane holding
+// the i-point | j-offset from jq0 << 5.
+__device__ __forceinline__ void tc_drain(const WorkDesc& wd, const SubProblem& sp, const uint32_t* q, uint32_t n,
+                                         u64 ax, u64 ay, u64 az, uint32_t iw, uint32_t jq0, const HistCol& hc,
+                                         uint32_t& band, uint32_t& mism) {
+    const uint32_t lane = threadIdx.x & 31u;
+    const bool has = lane < n;
+    const uint32_t code = has ? q[lane] : 0u;
+    const int l = (int)(code & 31u);
+    const uint32_t jg = jq0 + (code >> 5);
+    const float x = __shfl_sync(0xffffffffu, lo_of(ax), l);
+    const float y = __shfl_sync(0xffffffffu, lo_of(ay), l);
+    const float z = __shfl_sync(0xffffffffu, lo_of(az), l);
+    if (has) {
+        const float4 b = __ldg(sp.b32 + jg);
+        hist_inc<kWorkThreads>(hc, classify_unsettled<false>(wd, sp, x, y, z, b.x, b.y, b.z, iw + (uint32_t)l, jg,
+                                                             band, mism));
+    }
+}
+
+// ============================================================== the kernel
+// PREEMPT: draws start at wd.pos_lo and stop once stats[kStatYield] is set
+// (the job server's steps of one large job).
+template <bool PREEMPT>
+__global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_constant__ WorkDesc wd) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const uint32_t S = wd.stages;
+    volatile int* ctl = sptr<volatile int>(wd.off_ctl);
+    uint64_t* bars = sptr<uint64_t>(wd.off_bars);
+    uint64_t* const full = bars;
+    uint64_t* const empty = bars + S;
+    uint64_t* const a_full = bars + 2 * S;
+    uint64_t* const a_empty = a_full + 2;
+    uint64_t* const d_full = a_full + 4;
+    uint64_t* const d_free = d_full + kGroups;
+    TcMeta* const meta = sptr<TcMeta>(wd.off_meta);
+    const bool check = (wd.flags & TPCF_F_CHECK_OVERFLOW) != 0;
+    const uint64_t limit = wd.wait_limit_ns;
+
+    // ---- set-up: control words, barriers, tensor memory, counters, bins
+    if (tid < kTcCtlWords) ctl[tid] = 0;
+    if (tid == 0) {
+        for (uint32_t s = 0; s < S; ++s) {
+            mbar_init(full + s, 1);
+            mbar_init(empty + s, kWorkWarps + kGroups);
+        }
+        for (int k = 0; k < 2; ++k) {
+            mbar_init(a_full + k, 1);
+            mbar_init(a_empty + k, kWorkWarps);
+        }
+        for (int g = 0; g < kGroups; ++g) {
+            mbar_init(d_full + g, 1);
+            mbar_init(d_free + g, 4);
+        }
+        fence_mbar_init();
+    }
+    __syncthreads();
+    if (warp == kIssueWarp) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
+                         smem_addr(sptr<uint32_t>(wd.off_ctl) + kTcTmem)),
+                     "r"((uint32_t)kTmemCols)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    }
+    {
+        uint32_t* hist = sptr<uint32_t>(wd.off_hist);
+        for (int k = tid; k < (wd.nedges_max + 1) * (kWorkThreads / 2); k += kThreads) hist[k] = 0;
+    }
+    load_bins<kThreads>(sub_of(wd, 0).bins, wd, false);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = (uint32_t)ctl[kTcTmem];
+
+    if (warp < kWorkWarps) {
+        // ================================================== classifying warps
+        const int g = warp >> 2;
+        const uint32_t d_addr = tmem + (uint32_t)(g * 128) + ((uint32_t)(warp & 3) << 21);  // lane (w % 4) * 32
+        const HistCol hc = hist_col<kWorkThreads>(wd);
+        uint32_t* const uq = sptr<uint32_t>(wd.off_queue) + (uint32_t)warp * kQueueCodes;
+        const float thr = wd.tc_thr;
+        uint32_t stage = 0, phase = 0, dphase = 0;
+        uint32_t iw = 0, qn = 0, jq0 = 0;  // first i of the warp, queue length, j origin of the queue's codes
+        uint32_t na = 0, nb = 0, rule = 0;
+        int cur_sub = -1;
+        unsigned long long* cur_hist = nullptr;
+        uint32_t inc_bound = 0, over = 0, band = 0, mism = 0;
+        u64 ax = 0, ay = 0, az = 0;
+        bool aborted = false;
+
+        auto flush = [&]() {
+            warp_flush_hist<kWorkThreads>(hc, wd.ne, check, cur_hist);
+            if (check) {
+                const unsigned long long o = warp_sum(over);
+                if (lane == 0 && o) atomicAdd(cur_hist + wd.ne, o);
+                over = 0;
+            }
+            inc_bound = 0;
+        };
+
+        while (true) {
+            if (!tc_wait(full + stage, phase, limit, ctl, wd.stats)) {
+                aborted = true;
+                break;
+            }
+            const volatile TcMeta* vm = meta + stage;
+            const uint32_t info = vm->info;
+            if (info & kInfoStop) {
+                __syncwarp();
+                if (lane == 0) mbar_arrive(empty + stage);
+                break;
+            }
+            const uint32_t jbase = vm->jbase;
+            if (info & kInfoNew) {
+                const int sub = (int)(info >> 16);
+                const uint32_t i0 = vm->i0;
+                const SubProblem& sp = sub_of(wd, sub);
+                iw = i0 + 32u * (uint32_t)warp;
+                jq0 = jbase;
+                unsigned long long* tgt = sp.hist;
+                if (sp.row_seg) tgt += (size_t)__ldg(sp.row_seg + iw / kSegAlign) * sp.row_stride;
+                if (cur_sub >= 0 && tgt != cur_hist) flush();
+                cur_sub = sub;
+                cur_hist = tgt;
+                na = sp.na;
+                nb = sp.nb;
+                rule = sp.auto_mode ? 1u : (sp.no_self ? 2u : 0u);
+                const float4 p = __ldg(sp.a32 + iw + (uint32_t)lane);
+                ax = pack2(p.x, p.x);
+                ay = pack2(p.y, p.y);
+                az = pack2(p.z, p.z);
+            }
+            uint32_t nbatch = 0, kept = 0;
+            // a lane's counter gains at most one per pair of the tile and one per queue batch
+            if (inc_bound + 2u * kOpBlock + 2u > 0xffffu || over > 0x40000000u) flush();
+            if ((info >> g) & 1u) {
+                // ---- the group's accumulators: one maximum per 32 x 32 pairs
+                if (!tc_wait(d_full + g, dphase, limit, ctl, wd.stats)) {
+                    aborted = true;
+                    break;
+                }
+                dphase ^= 1u;
+                tc_fence_after();
+                float m0 = tc_row_max32(d_addr), m1 = tc_row_max32(d_addr + 32u);
+                tc_wait_ld(m0, m1);
+                kept = __any_sync(0xffffffffu, m0 >= thr) ? 1u : 0u;
+                kept |= __any_sync(0xffffffffu, m1 >= thr) ? 2u : 0u;
+                float m2 = tc_row_max32(d_addr + 64u), m3 = tc_row_max32(d_addr + 96u);
+                tc_wait_ld(m2, m3);
+                tc_fence_before();
+                if (lane == 0) mbar_arrive(d_free + g);
+                kept |= __any_sync(0xffffffffu, m2 >= thr) ? 4u : 0u;
+                kept |= __any_sync(0xffffffffu, m3 >= thr) ? 8u : 0u;
+                const SubProblem& sp = sub_of(wd, cur_sub);
+                // blocks at or below the diagonal (j-block and i-block of 32 coincide or do not overlap)
+                uint32_t todo = check ? 0xfu : kept;
+                if (rule == 1u && jbase < iw) todo &= ~0u << ((iw - jbase) >> 5 < 4u ? (iw - jbase) >> 5 : 4u);
+                // (a counted block's overflow needs its pair mask; otherwise a mask is needed on the
+                // diagonal and, where padding could look in range, at the catalogs' ends)
+                const bool ends = (wd.need_idx || check) && (jbase + kOpBlock > nb || iw + 32u > na);
+                const float* sx = sptr<const float>(wd.off_stage + stage * kOpBBlock + kOpBCoord);
+                while (todo) {
+                    const uint32_t b = (uint32_t)__ffs((int)todo) - 1u;
+                    todo &= todo - 1u;
+                    const uint32_t jb = jbase + 32u * b;
+                    const bool diag = rule != 0u && jb == iw;
+                    uint32_t valid = ~0u;
+                    if (diag || ends) {
+                        const uint32_t left = nb > jb ? nb - jb : 0u;
+                        if (left < 32u) valid = (1u << left) - 1u;
+                        if (iw + (uint32_t)lane >= na) valid = 0u;
+                        if (diag) valid &= rule == 1u ? (0xfffffffeu << lane) : ~(1u << lane);
+                    }
+                    if (!((kept >> b) & 1u)) {  // (only with a counted overflow row)
+                        over += (uint32_t)__popc(valid);
+                        continue;
+                    }
+                    uint32_t um = (diag || ends) ? tc_block<true>(wd, ax, ay, az, sx + 32 * b, valid, hc)
+                                                 : tc_block<false>(wd, ax, ay, az, sx + 32 * b, valid, hc);
+                    // ---- queue the unsettled pairs; a full batch of 32 is classified at once
+                    uint32_t act = __ballot_sync(0xffffffffu, um != 0u);
+                    while (act) {
+                        if (um) {
+                            const int k = __clz((int)um);
+                            um &= ~(0x80000000u >> k);
+                            uq[qn + (uint32_t)__popc(act & ((1u << lane) - 1u))] =
+                                (uint32_t)lane | ((jb + (uint32_t)k - jq0) << 5);
+                        }
+                        qn += (uint32_t)__popc(act);
+                        if (qn >= 32u) {
+                            __syncwarp();
+                            qn -= 32u;
+                            tc_drain(wd, sp, uq + qn, 32u, ax, ay, az, iw, jq0, hc, band, mism);
+                            ++nbatch;
+                            __syncwarp();  // the batch is read before later codes overwrite it
+                        }
+                        act = __ballot_sync(0xffffffffu, um != 0u);
+                    }
+                }
+            }
+            if (info & kInfoLast) {
+                if (lane == 0) mbar_arrive(a_empty + ((info & kInfoABuf) ? 1 : 0));
+                if (qn) {
+                    __syncwarp();
+                    tc_drain(wd, sub_of(wd, cur_sub), uq, qn, ax, ay, az, iw, jq0, hc, band, mism);
+                    ++nbatch;
+                    qn = 0;
+                }
+            }
+            inc_bound += 32u * (uint32_t)__popc(kept) + nbatch;
+            __syncwarp();
+            if (lane == 0) mbar_arrive(empty + stage);
+            if (++stage == S) {
+                stage = 0;
+                phase ^= 1u;
+            }
+        }
+        if (!aborted && cur_sub >= 0) flush();
+        const unsigned long long b = warp_sum(band), mm = warp_sum(mism);
+        if (lane == 0) {
+            if (b) atomicAdd(wd.stats + kStatBand, b);
+            if (mm) atomicAdd(wd.stats + kStatMismatch, mm);
+        }
+    } else if (warp < kLoadWarp) {
+        // ================================================== mma issuers
+        const int g = warp - kIssueWarp;
+        uint32_t stage = 0, phase = 0, dphase = 0, acnt = 0;
+        bool any = false;
+        while (true) {
+            if (!tc_wait(full + stage, phase, limit, ctl, wd.stats)) break;
+            const volatile TcMeta* vm = meta + stage;
+            const uint32_t info = vm->info;
+            if (info & kInfoStop) {
+                __syncwarp();
+                if (lane == 0) mbar_arrive(empty + stage);
+                break;
+            }
+            const uint32_t buf = (info & kInfoABuf) ? 1u : 0u;
+            if (info & kInfoNew) {
+                if (!tc_wait(a_full + buf, (acnt >> 1) & 1u, limit, ctl, wd.stats)) break;
+                ++acnt;
+            }
+            if ((info >> g) & 1u) {
+                if (!tc_wait(d_free + g, dphase ^ 1u, limit, ctl, wd.stats)) break;
+                dphase ^= 1u;
+                tc_fence_after();
+                if (lane == 0) {
+                    tc_mma(tmem + (uint32_t)(g * 128),
+                           op_desc(smem_addr(dyn_smem) + wd.off_atile + buf * kABytes + (uint32_t)g * kOpABlock),
+                           op_desc(smem_addr(dyn_smem) + wd.off_stage + stage * kOpBBlock));
+                    tc_commit(d_full + g);
+                }
+                any = true;
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(empty + stage);
+            if (++stage == S) {
+                stage = 0;
+                phase ^= 1u;
+            }
+        }
+        // after an abort: the last product finishes before the tensor memory is given back
+        if (ctl[kTcAbort] && any) (void)mbar_wait_bounded(d_full + g, dphase ^ 1u, limit);
+    } else {
+        // ================================================== loader: items, tiles, copies
+        const bool hook = (wd.flags & TPCF_F_TEST_WAIT_TIMEOUT) != 0;
+        uint32_t stage = 0, phase = 0, acnt = 0, issued = 0;
+        unsigned long long pruned = 0;
+        bool ok = true;
+        const uint64_t n = wd.item_hi - wd.item_lo;
+        unsigned long long* const counter = wd.stats + kStatNextItem;
+        auto draw = [&]() -> unsigned long long {
+            unsigned long long p = ~0ull;
+            if (lane == 0) {
+                if constexpr (PREEMPT) {
+                    if (*reinterpret_cast<volatile unsigned long long*>(wd.stats + kStatYield) == 0ull)
+                        p = wd.pos_lo + atomicAdd(counter, 1ull);
+                } else {
+                    p = atomicAdd(counter, 1ull);
+                }
+            }
+            return __shfl_sync(0xffffffffu, p, 0);
+        };
+        while (ok) {
+            const unsigned long long p = draw();
+            if (p >= n || ctl[kTcAbort]) break;
+            Cursor c;
+            if (!load_item(wd, (uint32_t)(wd.item_lo + p), c)) continue;
+            const SubProblem& sp = sub_of(wd, c.sub);
+            if (lane == 0)
+                atomicAdd(wd.stats + kStatPairs,
+                          (unsigned long long)span_pairs(c.g.i0, wd.I, (uint64_t)c.g.j0 + (uint64_t)c.t * wd.J,
+                                                         (uint64_t)c.g.j0 + (uint64_t)c.g.t_end * wd.J, sp.na, sp.nb,
+                                                         sp.auto_mode != 0));
+            // lane t: the groups with countable pairs in the item's tile t_first + t (at most 32 tiles)
+            const uint32_t t = c.g.t_first + (uint32_t)lane;
+            const uint32_t jb = c.g.j0 + t * kOpBlock;
+            uint32_t groups = 0;
+            if (t < c.g.t_end) {
+                float4 jc = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (wd.prune) jc = __ldg(sp.b_caps + jb / kCapPoints);
+#pragma unroll
+                for (int gg = 0; gg < kGroups; ++gg) {
+                    const uint32_t ib = c.g.i0 + 128u * (uint32_t)gg;
+                    bool in = ib < sp.na && !(sp.auto_mode && jb < ib);
+                    if (in && wd.prune && prune_block(wd, __ldg(sp.a_caps + ib / kCapPoints), jc)) {
+                        in = false;
+                        pruned += (unsigned long long)kOpBlock * kOpBlock;
+                    }
+                    groups |= in ? 1u << gg : 0u;
+                }
+            }
+            uint32_t tiles = __ballot_sync(0xffffffffu, groups != 0u);
+            if (!tiles) continue;
+            // ---- the item's i-side operand
+            const uint32_t buf = acnt & 1u;
+            if (!tc_wait(a_empty + buf, ((acnt >> 1) & 1u) ^ 1u, limit, ctl, wd.stats)) break;
+            if (lane == 0) {
+                mbar_expect_tx(a_full + buf, kABytes);
+                bulk_copy_g2s(sptr<unsigned char>(wd.off_atile + buf * kABytes),
+                              sp.a_op + (size_t)(c.g.i0 / kOpBlock) * kOpABlock, kABytes, a_full + buf);
+            }
+            ++acnt;
+            // ---- its tiles
+            uint32_t first = kInfoNew;
+            while (tiles) {
+                const int k = __ffs((int)tiles) - 1;
+                tiles &= tiles - 1u;
+                const uint32_t gm = __shfl_sync(0xffffffffu, groups, k);
+                if (!tc_wait(empty + stage, phase ^ 1u, limit, ctl, wd.stats)) {
+                    ok = false;
+                    break;
+                }
+                if (lane == 0) {
+                    const uint32_t jt = c.g.j0 + (c.g.t_first + (uint32_t)k) * kOpBlock;
+                    volatile TcMeta* vm = meta + stage;
+                    vm->i0 = c.g.i0;
+                    vm->jbase = jt;
+                    vm->info = gm | (buf ? kInfoABuf : 0u) | first | (tiles ? 0u : kInfoLast) | ((uint32_t)c.sub << 16);
+                    fence_proxy_async_smem();  // the group's reads of the stage's previous tile come first
+                    if (!(hook && issued == 0)) {  // (test hook: the first copy is never issued)
+                        mbar_expect_tx(full + stage, kOpBBlock);
+                        bulk_copy_g2s(sptr<unsigned char>(wd.off_stage + stage * kOpBBlock),
+                                      sp.b_op + (size_t)(jt / kOpBlock) * kOpBBlock, kOpBBlock, full + stage);
+                    }
+                }
+                first = 0;
+                ++issued;
+                if (++stage == S) {
+                    stage = 0;
+                    phase ^= 1u;
+                }
+            }
+        }
+        if (ok && !ctl[kTcAbort] && tc_wait(empty + stage, phase ^ 1u, limit, ctl, wd.stats) && lane == 0) {
+            volatile TcMeta* vm = meta + stage;
+            vm->info = kInfoStop;
+            mbar_arrive(full + stage);
+        }
+        __syncwarp();
+        if (wd.prune) {
+            pruned = warp_sum(pruned);
+            if (lane == 0 && pruned) atomicAdd(wd.stats + kStatPruned, pruned);
+        }
+        // after an abort: copies still in flight land before the block leaves (bounded)
+        if (ctl[kTcAbort]) {
+            const uint32_t back = issued < S ? issued : S;
+            for (uint32_t k = issued - back; k < issued; ++k)
+                if (!(hook && k == 0)) (void)mbar_wait_bounded(full + k % S, (k / S) & 1u, limit);
+            for (uint32_t k = acnt < 2u ? 0u : acnt - 2u; k < acnt; ++k)
+                (void)mbar_wait_bounded(a_full + (k & 1u), (k >> 1) & 1u, limit);
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == kIssueWarp)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)kTmemCols));
+}
+
+template <bool PREEMPT>
+cudaError_t launch_tc_t(const WorkDesc& wd_in, const Shape& sh, cudaStream_t stream) {
+    WorkDesc wd = wd_in;
+    const TcLayout L = tc_layout((int)wd.stages, wd.nedges_max);
+    wd.off_ctl = L.ctl;
+    wd.off_bars = L.bars;
+    wd.off_meta = L.meta;
+    wd.off_atile = L.atile;
+    wd.off_stage = L.stage;
+    wd.off_hist = L.hist;
+    wd.off_cthr = L.cos_thr;
+    wd.off_lo = L.lo;
+    wd.off_hi = L.hi;
+    wd.off_c32 = L.cos32;
+    wd.off_zlo = L.zlo;
+    wd.off_zhi = L.zhi;
+    wd.off_lut = L.lut;
+    wd.off_queue = L.queue;
+    wd.off_bwd = L.bwd;
+    wd.stage_bytes = kOpBBlock;
+    if (L.total > sh.smem || wd.I != 128u * kGroups || wd.J != kOpBlock || wd.Jc > 32u * kOpBlock)
+        return cudaErrorInvalidValue;
+    count_tc_kernel<PREEMPT><<<sh.blocks, kThreads, sh.smem, stream>>>(wd);
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+size_t count_tc_smem_bytes(int stages, int nedges) { return tc_layout(stages, nedges).total; }
+
+cudaError_t count_tc_set_smem_limit() {
+    int dev = 0, optin = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    // (the opt-in maximum: the attribute belongs to the kernel, not to a launch)
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(count_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(count_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
+    return e;
+}
+
+cudaError_t launch_count_tc(const WorkDesc& wd, const Shape& sh, bool preempt, cudaStream_t stream) {
+    return preempt ? launch_tc_t<true>(wd, sh, stream) : launch_tc_t<false>(wd, sh, stream);
+}
+
+}  // namespace tpcf

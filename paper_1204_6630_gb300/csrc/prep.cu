@@ -7,6 +7,7 @@
 // correlation functions in cosmology", Section 3 (the pair angle follows from
 // the dot product of unit vectors; this file prepares those vectors once per
 // catalog so that the O(N^2) counting kernel reads compact, sorted copies).
+#include <cuda_fp16.h>
 #include <stdint.h>
 
 #include "tpcf.h"
@@ -193,6 +194,34 @@ __global__ void __launch_bounds__(1024) bitonic_local_kernel(unsigned long long*
     vals[base + t + 1024] = sv[t + 1024];
 }
 
+// The binary16 split of an FP32 coordinate: v = hi + lo + r, |r| <= 2^-22 |v| + 2^-25.
+__device__ __forceinline__ uint32_t split16(float v) {  // hi | lo << 16
+    const __half h = __float2half_rn(v), l = __float2half_rn(v - __half2float(h));
+    return (uint32_t)__half_as_ushort(h) | ((uint32_t)__half_as_ushort(l) << 16);
+}
+
+// Writes point q's records into the tensor-core operands (layout: tpcf_internal.h).
+__device__ __forceinline__ void put_operands(unsigned char* op_a, unsigned char* op_b, uint32_t q, float x, float y,
+                                             float z) {
+    const uint32_t sx = split16(x), sy = split16(y), sz = split16(z);
+    const uint32_t h01 = __byte_perm(sx, sy, 0x5410), l01 = __byte_perm(sx, sy, 0x7632);
+    const uint32_t h2 = sz & 0xffffu, l2 = sz >> 16;
+    const uint4 X = make_uint4(h01, h2 | (l01 << 16), (l01 >> 16) | (l2 << 16), 0u);
+    const uint4 Y = make_uint4(l01, l2 | (h01 << 16), (h01 >> 16) | (h2 << 16), 0u);
+    const uint32_t o = q % kOpBlock;
+    uint4* a = reinterpret_cast<uint4*>(op_a + (size_t)(q / kOpBlock) * kOpABlock);
+    unsigned char* bb = op_b + (size_t)(q / kOpBlock) * kOpBBlock;
+    uint4* b = reinterpret_cast<uint4*>(bb);
+    a[o] = X;
+    a[kOpBlock + o] = X;
+    b[o] = X;
+    b[kOpBlock + o] = Y;
+    float* f = reinterpret_cast<float*>(bb + kOpBCoord);
+    f[o] = x;
+    f[kOpBlock + o] = y;
+    f[2 * kOpBlock + o] = z;
+}
+
 // Gather points in sorted order into the binary64 and FP32 device copies (the
 // outputs are zeroed beforehand: padding and segment gaps hold zero vectors).
 // Sorted point p of segment s goes to position p + seg_delta[s] (segments of a
@@ -200,7 +229,7 @@ __global__ void __launch_bounds__(1024) bitonic_local_kernel(unsigned long long*
 __global__ void prep_gather_kernel(const double* __restrict__ xyz, uint32_t n,
                                    const uint32_t* __restrict__ order, const uint32_t* __restrict__ seg_of_point,
                                    const uint32_t* __restrict__ seg_delta, Point64* out64, float4* out32,
-                                   float* out_soa, uint32_t n_pad) {
+                                   float* out_soa, unsigned char* op_a, unsigned char* op_b, uint32_t n_pad) {
     const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
     const uint32_t s = order ? order[p] : p;
@@ -212,6 +241,7 @@ __global__ void prep_gather_kernel(const double* __restrict__ xyz, uint32_t n,
     out_soa[q] = fx;
     out_soa[(size_t)n_pad + q] = fy;
     out_soa[2ull * n_pad + q] = fz;
+    if (op_a) put_operands(op_a, op_b, q, fx, fy, fz);
 }
 
 // Padding of 3-D catalogs: (+inf, +inf, +inf).  A pair with a real point has
@@ -289,8 +319,8 @@ __global__ void prep_caps_kernel(const Point64* __restrict__ p64, uint32_t n_gro
 
 cudaError_t launch_prepare(const double* xyz_in, uint32_t n, const uint32_t* seg_of_point,
                            const uint32_t* seg_delta, int sort, int euclid, unsigned long long* bbox,
-                           Point64* out64, float4* out32, float* out_soa, float4* caps, uint32_t n_pad,
-                           unsigned long long* keys, uint32_t* vals, uint32_t n_pow2,
+                           Point64* out64, float4* out32, float* out_soa, unsigned char* op_a, unsigned char* op_b,
+                           float4* caps, uint32_t n_pad, unsigned long long* keys, uint32_t* vals, uint32_t n_pow2,
                            unsigned long long* err_word, unsigned long long* eps_word, cudaStream_t stream,
                            uint32_t* launches) {
     cudaError_t e;
@@ -334,10 +364,13 @@ cudaError_t launch_prepare(const double* xyz_in, uint32_t n, const uint32_t* seg
             (e = cudaMemsetAsync(out32, 0, (size_t)n_pad * sizeof(float4), stream)) != cudaSuccess ||
             (e = cudaMemsetAsync(out_soa, 0, (size_t)n_pad * 3 * sizeof(float), stream)) != cudaSuccess)
             return e;
+        if (op_a && ((e = cudaMemsetAsync(op_a, 0, (size_t)(n_pad / kOpBlock) * kOpABlock, stream)) != cudaSuccess ||
+                     (e = cudaMemsetAsync(op_b, 0, (size_t)(n_pad / kOpBlock) * kOpBBlock, stream)) != cudaSuccess))
+            return e;
     }
     if (n > 0) {
         prep_gather_kernel<<<(n + 255) / 256, 256, 0, stream>>>(xyz_in, n, do_sort ? vals : nullptr, seg_of_point,
-                                                               seg_delta, out64, out32, out_soa, n_pad);
+                                                               seg_delta, out64, out32, out_soa, op_a, op_b, n_pad);
         ++nl;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }

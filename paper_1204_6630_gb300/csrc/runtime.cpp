@@ -662,7 +662,8 @@ extern "C" int tpcf_bins_destroy(tpcf_bins* b) { return bins_destroy_impl(b); }
 // ====================================================================== catalogs
 size_t tpcf::catalog_bytes(uint64_t n) {
     const uint64_t n_pad = ((n + kPad - 1) / kPad + 1) * kPad;
-    return (size_t)n_pad * (sizeof(Point64) + sizeof(float4) + 3 * sizeof(float));
+    return (size_t)n_pad * (sizeof(Point64) + sizeof(float4) + 3 * sizeof(float)) +
+           (size_t)(n_pad / kOpBlock) * (kOpABlock + kOpBBlock);
 }
 
 int tpcf::catalog_create_impl(tpcf_ctx* ctx, const double* xyz, uint64_t n, int where, const uint64_t* offsets,
@@ -735,7 +736,9 @@ int tpcf::catalog_create_impl(tpcf_ctx* ctx, const double* xyz, uint64_t n, int 
     if (alloc((void**)&c->d64, (size_t)c->n_pad * sizeof(Point64)) != cudaSuccess ||
         alloc((void**)&c->d32, (size_t)c->n_pad * sizeof(float4)) != cudaSuccess ||
         alloc((void**)&c->soa, (size_t)c->n_pad * 3 * sizeof(float)) != cudaSuccess ||
-        alloc((void**)&c->caps, (size_t)(c->n_pad / kCapPoints) * sizeof(float4)) != cudaSuccess)
+        alloc((void**)&c->caps, (size_t)(c->n_pad / kCapPoints) * sizeof(float4)) != cudaSuccess ||
+        (!euclid && (alloc((void**)&c->op_a, (size_t)(c->n_pad / kOpBlock) * kOpABlock) != cudaSuccess ||
+                     alloc((void**)&c->op_b, (size_t)(c->n_pad / kOpBlock) * kOpBBlock) != cudaSuccess)))
         return fail_with(TPCF_ENOMEM, "device allocation failed");
     const double* in = xyz;
     if (n > 0 && where == TPCF_HOST) {
@@ -777,7 +780,7 @@ int tpcf::catalog_create_impl(tpcf_ctx* ctx, const double* xyz, uint64_t n, int 
     }
     uint32_t nl = 0;
     cudaError_t e = launch_prepare(in, (uint32_t)n, seg, seg_delta, sort ? 1 : 0, euclid ? 1 : 0, err + 2, c->d64,
-                                   c->d32, c->soa, c->caps, c->n_pad, keys, vals, n_pow2, err, err + 1, st, &nl);
+                                   c->d32, c->soa, c->op_a, c->op_b, c->caps, c->n_pad, keys, vals, n_pow2, err, err + 1, st, &nl);
     ctx->launches.fetch_add(nl);
     if (e != cudaSuccess) return fail_with(TPCF_ECUDA, cudaGetErrorString(e));
     unsigned long long hw[2] = {0, 0};
@@ -823,7 +826,7 @@ extern "C" int tpcf_catalog_create_3d(tpcf_ctx* ctx, const double* xyz, uint64_t
 int tpcf::catalog_destroy_impl(tpcf_catalog* c) {
     if (!c) return TPCF_EINVAL;
     cudaSetDevice(c->ctx->cfg.device);
-    void* bufs[5] = {c->d64, c->d32, c->soa, c->seg_of_block, c->caps};
+    void* bufs[7] = {c->d64, c->d32, c->soa, c->seg_of_block, c->caps, c->op_a, c->op_b};
     if (c->stream_ordered) {
         for (void* p : bufs)
             if (p) cudaFreeAsync(p, c->free_stream);
@@ -889,6 +892,30 @@ bool shape_for(tpcf_ctx* ctx, int mode, int nedges, int T, int R, int Jreq, int 
     sh->smem = smem;
     sh->blocks = ctx->num_sms;  // one persistent block per SM
     sh->jchunk = kChunk;
+    sh->tc = false;
+    return true;
+}
+
+// Shape of the tensor-core kernel (angular screen): 512 i-points x Jc j-points
+// per item.  Jc is the largest that leaves every SM kTcItemsPerSm items, so
+// that the launch's last items are a small part of it; a small problem is cut
+// down to one tile (512 x 128 pairs) per item.  False when the histograms do
+// not leave shared memory for a ring of four stages.
+bool tc_shape_for(tpcf_ctx* ctx, int nedges, uint64_t total_pairs, Shape* sh) {
+    constexpr uint64_t kTcItemsPerSm = 16;
+    int S = 8;
+    while (S >= 4 && count_tc_smem_bytes(S, nedges) > ctx->smem_optin) S -= 2;
+    if (S < 4) return false;
+    int Jc = 32 * (int)kOpBlock;
+    while (Jc > (int)kOpBlock && total_pairs / (512ull * (uint64_t)Jc) < kTcItemsPerSm * (uint64_t)ctx->num_sms) Jc /= 2;
+    sh->threads = 512;
+    sh->ipt = 16;
+    sh->jtile = (int)kOpBlock;
+    sh->jchunk = Jc;
+    sh->stages = S;
+    sh->blocks = ctx->num_sms;
+    sh->smem = count_tc_smem_bytes(S, nedges);
+    sh->tc = true;
     return true;
 }
 
@@ -898,6 +925,9 @@ bool choose_shape(tpcf_ctx* ctx, int mode, int nedges, uint64_t total_pairs, uin
     const tpcf_config& cfg = ctx->cfg;
     if (cfg.threads != 0 && cfg.ipt != 0)
         return shape_for(ctx, mode, nedges, cfg.threads, cfg.ipt, cfg.jtile, cfg.stages, sh);
+    if (mode == kModeScreenScalar && cfg.threads == 0 && cfg.ipt == 0 && cfg.jtile == 0 && cfg.stages == 0 &&
+        tc_shape_for(ctx, nedges, total_pairs, sh))
+        return true;
     const double per_sm = (double)total_pairs / std::max(1, ctx->num_sms);
     if (per_sm >= 4e7 && max_n >= 8192) {
         if (shape_for(ctx, mode, nedges, 512, 8, cfg.jtile, cfg.stages, sh)) return true;
@@ -946,6 +976,8 @@ uint64_t build_work(tpcf_ctx* ctx, const SubSpec* specs, int nsub, const BinsDev
         sp.b64 = p.b->d64 + p.b_off;
         sp.a_caps = p.a->caps + p.a_off / kCapPoints;  // sub-ranges start on kSegAlign boundaries
         sp.b_caps = p.b->caps + p.b_off / kCapPoints;
+        sp.a_op = p.a->op_a ? p.a->op_a + (size_t)(p.a_off / kOpBlock) * kOpABlock : nullptr;
+        sp.b_op = p.b->op_b ? p.b->op_b + (size_t)(p.b_off / kOpBlock) * kOpBBlock : nullptr;
         sp.na = p.na;
         sp.nb = p.nb;
         sp.n_iblk = (p.na + I - 1) / I;
@@ -990,6 +1022,7 @@ void fill_scalars(tpcf_ctx* ctx, const SubSpec* specs, int nsub, const BinsDev* 
         wd.neg_fast_t2 = ((unsigned long long)b << 32) | b;
     }
     wd.cos_last = bh->cos_last;
+    wd.tc_thr = bh->euclid ? 0.f : round_down_f32(bh->cos_last - kTcGuard);
     wd.zbits0 = bh->zbits0;
     wd.zshift = bh->zshift;
     // zero-vector padding has screen value e = -T: it can look in range only
@@ -1101,7 +1134,7 @@ int run_counts(tpcf_ctx* ctx, const SubSpec* specs, int nsub, const tpcf_bins* b
     if (!fits)
         return ctx->fail(TPCF_EINVAL, "no kernel shape fits (threads=%d ipt=%d jtile=%d)",
                          ctx->cfg.threads, ctx->cfg.ipt, ctx->cfg.jtile);
-    if (any_rows && 32u * (uint32_t)sh.ipt != kSegAlign)
+    if (any_rows && !sh.tc && 32u * (uint32_t)sh.ipt != kSegAlign)
         return ctx->fail(TPCF_EINVAL, "row-attributed counts need %u i-points per warp", kSegAlign);
 
     // ---- accumulators and statistics: a context slot for up to 3 histograms,
@@ -1176,16 +1209,19 @@ int run_counts(tpcf_ctx* ctx, const SubSpec* specs, int nsub, const tpcf_bins* b
         fill_scalars(ctx, specs, nsub, bh, mode, shp, force_idx, ne, wd);
         return TPCF_OK;
     };
+    auto smem_limit = [&](const Shape& shp) {
+        return shp.tc ? count_tc_set_smem_limit() : count_set_smem_limit(mode, shp.threads, shp.ipt, shp.smem);
+    };
     auto launch = [&](const Shape& shp) -> cudaError_t {
         if (wd.item_hi <= wd.item_lo) return cudaSuccess;
         Shape sl = shp;
         const uint64_t n_launch_items = wd.item_hi - wd.item_lo;
         if ((uint64_t)sl.blocks > n_launch_items) sl.blocks = (int)n_launch_items;
         if (!capture) {  // when capturing, set before the capture begins
-            cudaError_t e = count_set_smem_limit(mode, shp.threads, shp.ipt, shp.smem);
+            cudaError_t e = smem_limit(shp);
             if (e != cudaSuccess) return e;
         }
-        return launch_count(wd, sl, mode, ne, st);
+        return sl.tc ? launch_count_tc(wd, sl, false, st) : launch_count(wd, sl, mode, ne, st);
     };
 
     // ---- optional autotuning: time every fitting shape on a bounded window of the
@@ -1198,26 +1234,32 @@ int run_counts(tpcf_ctx* ctx, const SubSpec* specs, int nsub, const tpcf_bins* b
         if (it != ctx->tuned.end()) {
             sh = it->second;
         } else {
-            const int cand_t[3] = {128, 256, 512};
+            // (the FP32 kernel's nine shapes; the tensor-core kernel where it can run)
+            const int cand_t[4] = {128, 256, 512, 0};
             const int cand_j[3] = {128, 256, 512};
+            Shape tc_sh;
+            const bool tc_fits = sh.tc;
+            tc_sh = sh;
             double best = 1e300;
             Shape best_sh = sh;
             cudaEvent_t a0, a1;
             cudaEventCreate(&a0);
             cudaEventCreate(&a1);
-            for (int ti = 0; ti < 3; ++ti) {
+            for (int ti = 0; ti < 4; ++ti) {
                 for (int ji = 0; ji < 3; ++ji) {
-                    Shape c;
-                    if (!shape_for(ctx, mode, ne, cand_t[ti], 8, cand_j[ji], 0, &c)) continue;
+                    Shape c = tc_sh;
+                    if (cand_t[ti] == 0 ? (!tc_fits || ji > 0)
+                                        : !shape_for(ctx, mode, ne, cand_t[ti], 8, cand_j[ji], 0, &c))
+                        continue;
                     if (setup(c) != TPCF_OK) continue;
-                    const uint64_t window = (uint64_t)ctx->num_sms * (uint64_t)(c.threads / 32) * 4;
+                    const uint64_t window = (uint64_t)ctx->num_sms * (c.tc ? 1ull : (uint64_t)(c.threads / 32)) * 4;
                     if (wd.item_hi - wd.item_lo > window) wd.item_hi = wd.item_lo + window;
                     uint64_t wpairs = 0;
                     for (int s2 = 0; s2 < nsub; ++s2)
                         wpairs += range_pairs(subs[s2], wd.item_lo, wd.item_hi, wd.I, wd.Jc, wd.J);
                     if (wpairs == 0) continue;
                     cudaMemsetAsync(acc, 0, acc_words * 8, st);
-                    if (capture && count_set_smem_limit(mode, c.threads, c.ipt, c.smem) != cudaSuccess) continue;
+                    if (capture && smem_limit(c) != cudaSuccess) continue;
                     cudaEventRecord(a0, st);
                     if (launch(c) != cudaSuccess) continue;
                     cudaEventRecord(a1, st);
@@ -1250,8 +1292,7 @@ int run_counts(tpcf_ctx* ctx, const SubSpec* specs, int nsub, const tpcf_bins* b
         cudaMemcpyAsync(dev_totals, totals.data(), (size_t)H * 8, cudaMemcpyHostToDevice, st) != cudaSuccess)
         return release(ctx->fail(TPCF_ECUDA, "totals upload failed"));
     if (capture) {
-        if (count_set_smem_limit(mode, sh.threads, sh.ipt, sh.smem) != cudaSuccess ||
-            cudaStreamSynchronize(st) != cudaSuccess ||
+        if (smem_limit(sh) != cudaSuccess || cudaStreamSynchronize(st) != cudaSuccess ||
             cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal) != cudaSuccess)
             return release(ctx->fail(TPCF_ECUDA, "graph capture could not start"));
     }

@@ -18,6 +18,18 @@ constexpr uint32_t kSegAlign = 256;
 // Bounding spheres for spatial pruning: one per kCapPoints consecutive
 // points of a catalog's device layout.
 constexpr uint32_t kCapPoints = 128;
+// Operands of the tensor-core screen (count_tc.cu), in blocks of kOpBlock
+// points.  A point's binary16 split x = x1 + x2 (likewise y, z) gives the
+// 16-byte records X = (x1, y1, z1, x2, y2, z2, 0, 0) and Y = (x2, y2, z2, x1,
+// y1, z1, 0, 0).  i-side block: plane X, plane X (2 x 2048 bytes); j-side
+// block: plane X, plane Y, then the FP32 coordinates x | y | z (3 x 512 bytes).
+constexpr uint32_t kOpBlock = 128;
+constexpr uint32_t kOpABlock = 2 * kOpBlock * 16;
+constexpr uint32_t kOpBCoord = 2 * kOpBlock * 16;
+constexpr uint32_t kOpBBlock = kOpBCoord + kOpBlock * 12;
+// Bound on the distance of the tensor-core screen value from the binary64 dot
+// product (44u, derived in count_tc.cu) with a margin.
+constexpr double kTcGuard = 64.0 * 5.9604644775390625e-08;
 // 3-D catalogs store their spheres scaled by 2^-64 (exact), so that FP32
 // squares of separations up to 2e28 stay finite.
 constexpr double kCapScale3d = 5.421010862427522e-20;
@@ -93,6 +105,9 @@ struct SubProblem {
     // starting at the sub-range's first point (spatial pruning).
     const float4* a_caps;
     const float4* b_caps;
+    // Tensor-core operands of A (i-side) and B (j-side), the sub-range's first block.
+    const unsigned char* a_op;
+    const unsigned char* b_op;
 };
 
 constexpr int kMaxInlineSub = 3;
@@ -161,9 +176,10 @@ struct WorkDesc {
     float prune_thr;                 // sphere-gap threshold of the pruning test (see prune_block)
     float near_thr;                  // sphere gap below which two point groups may hold pairs in
                                      // range (the last edge's chord; scheduling only, see heavy_item)
+    float tc_thr;                    // tensor-core screen: blocks whose values are all below it are overflow
     // ... and the shared-memory layout of the shape (set by the launcher).
     uint32_t off_ctl, off_bars, off_meta, off_stage, off_hist, off_cthr, off_lo, off_hi, off_c32, off_zlo, off_zhi,
-        off_lut, off_queue, off_icap, off_bwd, off_counter;
+        off_lut, off_queue, off_icap, off_bwd, off_counter, off_atile;
     uint32_t stage_bytes;            // J * bytes per staged point
     uint32_t flush_limit;            // j-points between merges of the 16-bit counters
 };
@@ -177,6 +193,7 @@ struct Shape {
     int stages;    // S (per warp)
     int blocks;    // grid size
     size_t smem;   // dynamic shared memory bytes
+    bool tc;       // tensor-core kernel (T, R, J and the i-block are its own)
 };
 
 // Kernel variants (mode argument of the launchers): FP32 screen of angles,
@@ -193,6 +210,12 @@ cudaError_t launch_count_step(const WorkDesc& wd, const Shape& sh, cudaStream_t 
 // One serving step of a single job (FP32 screen of angles, shape 512 x 8): the
 // one-job kernel with preemptible draws (wd.pos_lo, stats[kStatYield]).
 cudaError_t launch_count_preemptible(const WorkDesc& wd, const Shape& sh, cudaStream_t stream);
+// The tensor-core counting kernel (count_tc.cu; FP32 screen of angles): items
+// of 512 i-points x Jc j-points in tiles of kOpBlock; preempt: draws from
+// wd.pos_lo on, stopping at the yield word.
+cudaError_t launch_count_tc(const WorkDesc& wd, const Shape& sh, bool preempt, cudaStream_t stream);
+size_t count_tc_smem_bytes(int stages, int nedges);
+cudaError_t count_tc_set_smem_limit();
 // count_over = 1: the kernel counted the overflow row (TPCF_F_CHECK_OVERFLOW);
 // the finalize then checks that the histogram sums to the pair total.
 cudaError_t launch_finalize(unsigned long long* acc, int nedges, unsigned long long* out,
@@ -203,7 +226,8 @@ cudaError_t launch_finalize_batch(const unsigned long long* acc, int acc_stride,
                                   int count, int count_over, unsigned long long* err_word, cudaStream_t stream);
 cudaError_t launch_prepare(const double* xyz_in, uint32_t n, const uint32_t* seg_of_point,
                            const uint32_t* seg_delta, int sort, int euclid, unsigned long long* bbox,
-                           Point64* out64, float4* out32, float* out_soa, float4* caps, uint32_t n_pad,
+                           Point64* out64, float4* out32, float* out_soa, unsigned char* op_a, unsigned char* op_b,
+                           float4* caps, uint32_t n_pad,
                            unsigned long long* key_scratch, uint32_t* val_scratch,
                            uint32_t n_pow2, unsigned long long* err_word, unsigned long long* eps_word,
                            cudaStream_t stream, uint32_t* launches);
