@@ -407,7 +407,7 @@ __device__ __forceinline__ uint32_t slow_group(const WorkDesc& wd, const u64 (&a
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const float v = __saturatef(e[r][u] * wd.lut_scale);
-                const float f = fmaf(v, 16384.0f, 8388608.0f);
+                const float f = fmaf(v, (float)(1 << kLutBits), 8388608.0f);
                 asm volatile("ld.shared.s16 %0, [%1];" : "=r"(ent[r & 1][u]) : "r"(__float_as_uint(f) * 2u + lut_adj));
             }
         }

@@ -372,7 +372,7 @@ __device__ __forceinline__ float screen_value(const WorkDesc& wd, const SubProbl
 // low bits of fma(v, 2^14, 2^23).
 __device__ __forceinline__ int lut_entry(const WorkDesc& wd, float e) {
     const float v = __saturatef(e * wd.lut_scale);
-    const float f = fmaf(v, 16384.0f, 8388608.0f);
+    const float f = fmaf(v, (float)(1 << kLutBits), 8388608.0f);
     return ld_shared_s16(smem_addr(dyn_smem) + wd.off_lut + (__float_as_uint(f) - 0x4B000000u) * 2u);
 }
 

@@ -49,7 +49,9 @@ constexpr int kTmemCols = 512;                    // 128 columns per group
 constexpr uint32_t kABytes = 4 * kOpABlock;       // i-side operand of an item (512 points)
 constexpr int kQueueCodes = 64;                   // per-warp queue of unsettled pairs
 
-enum TcCtl { kTcAbort = 0, kTcTmem = 1, kTcTake = 2, kTcCtlWords = 32 };
+// Control words.  kTcBeat changes with every batch of items the loader draws:
+// a wait is bounded by the time without progress.
+enum TcCtl { kTcAbort = 0, kTcTmem = 1, kTcBeat = 2, kTcCtlWords = 32 };
 
 // A staged tile: first i of the item, first j of the tile, and what to do with it.
 struct TcMeta {
@@ -58,11 +60,12 @@ struct TcMeta {
     uint32_t pad;
 };
 enum : uint32_t {
-    kInfoGroups = 0xfu,   // groups with countable pairs in this tile
+    kInfoGroups = 0xfu,   // groups of warps that work on this tile
     kInfoABuf = 0x10u,    // operand buffer of the item
     kInfoNew = 0x20u,     // first tile of an item
     kInfoLast = 0x40u,    // last tile of an item
     kInfoStop = 0x80u,    // no tile: the launch's (or slice's) items are done
+    // (PRUNE) bits 8 + 2 g, 9 + 2 g: which 128 i-points of the item group g takes
 };
 
 // Barriers (8 bytes each): full[S], empty[S], a_full[2], a_empty[2], d_full[4], d_free[4].
@@ -105,6 +108,15 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
 }
 
+// Allocation of the tensor memory (whole warp; the address goes to the shared word at `dst`).
+__device__ __forceinline__ void tc_alloc(uint32_t dst) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst), "r"((uint32_t)kTmemCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+}
+__device__ __forceinline__ void tc_dealloc(uint32_t tmem) {
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)kTmemCols));
+}
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 
@@ -133,7 +145,7 @@ __device__ __forceinline__ void tc_commit(uint64_t* bar) {
 // Maximum over 32 columns of the lane's accumulator row (the loaded values
 // themselves are not used).  The result is valid after tc_wait_ld.
 __device__ __forceinline__ float tc_row_max32(uint32_t addr) {
-    uint32_t r[32];
+    [[maybe_unused]] uint32_t r[32];
     float m;
     asm volatile(
         "tcgen05.ld.red.sync.aligned.32x32b.x32.max.f32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
@@ -152,16 +164,21 @@ __device__ __forceinline__ void tc_wait_ld(float& a, float& b) {
 }
 
 // Bounded wait of a whole warp for phase `parity` of `bar`: false (with the
-// block's abort word and the call's error word set) after limit_ns, and false
-// as soon as another warp has aborted.
+// block's abort word and the call's error word set) after limit_ns in which the
+// loader drew nothing, and false as soon as another warp has aborted.
 __device__ __noinline__ bool tc_wait_slow(uint64_t* bar, uint32_t parity, uint64_t limit_ns, volatile int* ctl,
                                           unsigned long long* stats) {
-    const uint64_t t0 = global_ns();
+    uint64_t t0 = global_ns();
+    int beat = ctl[kTcBeat];
     bool ok = false;
     while (true) {
         ok = mbar_try_wait(bar, parity);
         if (ok || ctl[kTcAbort]) break;
-        if (global_ns() - t0 > limit_ns) {
+        const int b = ctl[kTcBeat];
+        if (b != beat) {
+            beat = b;
+            t0 = global_ns();
+        } else if (global_ns() - t0 > limit_ns) {
             ctl[kTcAbort] = 1;
             atomicOr(stats + kStatError, (unsigned long long)kErrWaitTimeout);
             break;
@@ -173,6 +190,32 @@ __device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity, uint64_t
                                         unsigned long long* stats) {
     if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
     return tc_wait_slow(bar, parity, limit_ns, ctl, stats);
+}
+
+// A sphere that holds the (non-empty) spheres of an item's groups: centre the
+// FP32 mean of their centres, radius max |c - c_g| + r_g, enlarged by 2^-20.
+__device__ __forceinline__ float4 union_sphere(const float4 (&g)[kGroups]) {
+    float x = 0.f, y = 0.f, z = 0.f, n = 0.f;
+#pragma unroll
+    for (int k = 0; k < kGroups; ++k) {
+        if (g[k].w > -1e29f) {
+            x += g[k].x;
+            y += g[k].y;
+            z += g[k].z;
+            n += 1.f;
+        }
+    }
+    if (n == 0.f) return make_float4(0.f, 0.f, 0.f, -1e30f);
+    const float cx = x / n, cy = y / n, cz = z / n;
+    float r = 0.f;
+#pragma unroll
+    for (int k = 0; k < kGroups; ++k) {
+        if (g[k].w > -1e29f) {
+            const float dx = cx - g[k].x, dy = cy - g[k].y, dz = cz - g[k].z;
+            r = fmaxf(r, sqrtf(fmaf(dz, dz, fmaf(dy, dy, dx * dx))) + g[k].w);
+        }
+    }
+    return make_float4(cx, cy, cz, r * (1.0f + kPruneMargin));
 }
 
 // ============================================================== classification of a kept block
@@ -200,8 +243,8 @@ __device__ __forceinline__ uint32_t tc_block(const WorkDesc& wd, u64 ax, u64 ay,
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 const float v = __saturatef(e[u] * wd.lut_scale);
-                const float f = fmaf(v, 16384.0f, 8388608.0f);
-                asm volatile("ld.shared.s16 %0, [%1];" : "=r"(ent[k & 1][u]) : "r"(__float_as_uint(f) * 2u + lut_adj));
+                const float f = fmaf(v, (float)(1 << kLutBits), 8388608.0f);
+                ent[k & 1][u] = (uint32_t)ld_shared_s16(__float_as_uint(f) * 2u + lut_adj);
             }
         }
         if (k >= 1) {
@@ -239,8 +282,11 @@ __device__ __forceinline__ void tc_drain(const WorkDesc& wd, const SubProblem& s
 
 // ============================================================== the kernel
 // PREEMPT: draws start at wd.pos_lo and stop once stats[kStatYield] is set
-// (the job server's steps of one large job).
-template <bool PREEMPT>
+// (the job server's steps of one large job).  PRUNE: tiles and groups whose
+// bounding spheres are too far apart are left out, and a tile's i-groups go to
+// the groups of warps in turn (without pruning group g always takes i-points
+// 128 g .. of the item, and its loop is the shorter for it).
+template <bool PREEMPT, bool PRUNE>
 __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_constant__ WorkDesc wd) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t S = wd.stages;
@@ -275,11 +321,7 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
     }
     __syncthreads();
     if (warp == kIssueWarp) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
-                         smem_addr(sptr<uint32_t>(wd.off_ctl) + kTcTmem)),
-                     "r"((uint32_t)kTmemCols)
-                     : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+        tc_alloc(smem_addr(dyn_smem) + wd.off_ctl + 4u * kTcTmem);
     }
     {
         uint32_t* hist = sptr<uint32_t>(wd.off_hist);
@@ -301,6 +343,7 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
         uint32_t stage = 0, phase = 0, dphase = 0;
         uint32_t iw = 0, qn = 0, jq0 = 0;  // first i of the warp, queue length, j origin of the queue's codes
         uint32_t na = 0, nb = 0, rule = 0;
+        [[maybe_unused]] uint32_t cur_gi = 4u;  // which 128 of the item's i-points (4: none of this item yet)
         int cur_sub = -1;
         unsigned long long* cur_hist = nullptr;
         uint32_t inc_bound = 0, over = 0, band = 0, mism = 0;
@@ -330,11 +373,28 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                 break;
             }
             const uint32_t jbase = vm->jbase;
-            if (info & kInfoNew) {
+            // other i-points: a new item's, or (PRUNE) another 128 of the item's
+            bool turn = (info & kInfoNew) != 0u;
+            uint32_t gi = (uint32_t)g;
+            if constexpr (PRUNE) {
+                if (turn) cur_gi = 4u;
+                gi = (info >> (8 + 2 * g)) & 3u;
+                turn = ((info >> g) & 1u) && gi != cur_gi;
+            }
+            if (turn) {
+                if constexpr (PRUNE) {
+                    if (qn) {
+                        __syncwarp();
+                        tc_drain(wd, sub_of(wd, cur_sub), uq, qn, ax, ay, az, iw, jq0, hc, band, mism);
+                        ++inc_bound;
+                        qn = 0;
+                        __syncwarp();
+                    }
+                    cur_gi = gi;
+                }
                 const int sub = (int)(info >> 16);
-                const uint32_t i0 = vm->i0;
                 const SubProblem& sp = sub_of(wd, sub);
-                iw = i0 + 32u * (uint32_t)warp;
+                iw = vm->i0 + kOpBlock * gi + 32u * (uint32_t)(warp & 3);
                 jq0 = jbase;
                 unsigned long long* tgt = sp.hist;
                 if (sp.row_seg) tgt += (size_t)__ldg(sp.row_seg + iw / kSegAlign) * sp.row_stride;
@@ -465,7 +525,8 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                 tc_fence_after();
                 if (lane == 0) {
                     tc_mma(tmem + (uint32_t)(g * 128),
-                           op_desc(smem_addr(dyn_smem) + wd.off_atile + buf * kABytes + (uint32_t)g * kOpABlock),
+                           op_desc(smem_addr(dyn_smem) + wd.off_atile + buf * kABytes +
+                                   (PRUNE ? (info >> (8 + 2 * g)) & 3u : (uint32_t)g) * kOpABlock),
                            op_desc(smem_addr(dyn_smem) + wd.off_stage + stage * kOpBBlock));
                     tc_commit(d_full + g);
                 }
@@ -483,91 +544,146 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
     } else {
         // ================================================== loader: items, tiles, copies
         const bool hook = (wd.flags & TPCF_F_TEST_WAIT_TIMEOUT) != 0;
-        uint32_t stage = 0, phase = 0, acnt = 0, issued = 0;
+        uint32_t stage = 0, phase = 0, acnt = 0, issued = 0, turn = 0;
         unsigned long long pruned = 0;
         bool ok = true;
         const uint64_t n = wd.item_hi - wd.item_lo;
         unsigned long long* const counter = wd.stats + kStatNextItem;
-        auto draw = [&]() -> unsigned long long {
+        // Items are drawn wd.draw_batch at a time, one per lane: a lane finds its
+        // item's tiles and groups with countable pairs (bit t of gm[g]: tile t of the
+        // chunk for group g), so that a launch that prunes nearly everything spends a
+        // few instructions, not a draw, on an empty item.  A draw with its geometry
+        // takes about 6500 cycles for one item or for 32 (full sphere, 1.5M + 3M,
+        // 2 degrees: 145 ms with one item per draw, 40 ms with 32, 37 ms with the
+        // chunk spheres, 26 ms with tiles given to the groups of warps in turn).
+        const uint32_t batch = wd.draw_batch;
+        while (ok) {
             unsigned long long p = ~0ull;
             if (lane == 0) {
                 if constexpr (PREEMPT) {
                     if (*reinterpret_cast<volatile unsigned long long*>(wd.stats + kStatYield) == 0ull)
-                        p = wd.pos_lo + atomicAdd(counter, 1ull);
+                        p = wd.pos_lo + atomicAdd(counter, (unsigned long long)batch);
                 } else {
-                    p = atomicAdd(counter, 1ull);
+                    p = atomicAdd(counter, (unsigned long long)batch);
                 }
+                ctl[kTcBeat] = ctl[kTcBeat] + 1;
             }
-            return __shfl_sync(0xffffffffu, p, 0);
-        };
-        while (ok) {
-            const unsigned long long p = draw();
+            p = __shfl_sync(0xffffffffu, p, 0);
             if (p >= n || ctl[kTcAbort]) break;
             Cursor c;
-            if (!load_item(wd, (uint32_t)(wd.item_lo + p), c)) continue;
-            const SubProblem& sp = sub_of(wd, c.sub);
-            if (lane == 0)
-                atomicAdd(wd.stats + kStatPairs,
-                          (unsigned long long)span_pairs(c.g.i0, wd.I, (uint64_t)c.g.j0 + (uint64_t)c.t * wd.J,
-                                                         (uint64_t)c.g.j0 + (uint64_t)c.g.t_end * wd.J, sp.na, sp.nb,
-                                                         sp.auto_mode != 0));
-            // lane t: the groups with countable pairs in the item's tile t_first + t (at most 32 tiles)
-            const uint32_t t = c.g.t_first + (uint32_t)lane;
-            const uint32_t jb = c.g.j0 + t * kOpBlock;
-            uint32_t groups = 0;
-            if (t < c.g.t_end) {
-                float4 jc = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (wd.prune) jc = __ldg(sp.b_caps + jb / kCapPoints);
+            c.sub = 0;
+            c.g = ItemGeom{0u, 0u, 0u, 0u};
+            uint32_t gm[kGroups] = {0u, 0u, 0u, 0u};
+            unsigned long long pairs = 0;
+            if ((uint32_t)lane < batch && p + (uint32_t)lane < n &&
+                load_item(wd, (uint32_t)(wd.item_lo + p + (uint32_t)lane), c)) {
+                const SubProblem& sp = sub_of(wd, c.sub);
+                pairs = span_pairs(c.g.i0, wd.I, (uint64_t)c.g.j0 + (uint64_t)c.t * wd.J,
+                                   (uint64_t)c.g.j0 + (uint64_t)c.g.t_end * wd.J, sp.na, sp.nb, sp.auto_mode != 0);
 #pragma unroll
                 for (int gg = 0; gg < kGroups; ++gg) {
-                    const uint32_t ib = c.g.i0 + 128u * (uint32_t)gg;
-                    bool in = ib < sp.na && !(sp.auto_mode && jb < ib);
-                    if (in && wd.prune && prune_block(wd, __ldg(sp.a_caps + ib / kCapPoints), jc)) {
-                        in = false;
-                        pruned += (unsigned long long)kOpBlock * kOpBlock;
+                    const uint32_t ib = c.g.i0 + kOpBlock * (uint32_t)gg;
+                    uint32_t t0 = c.g.t_first;  // (auto counts: tiles from the group's own on)
+                    if (sp.auto_mode && ib > c.g.j0) t0 = max(t0, (ib - c.g.j0) / kOpBlock);
+                    if (ib < sp.na && t0 < c.g.t_end) gm[gg] = (0xffffffffu >> (32u - (c.g.t_end - t0))) << t0;
+                }
+                if (PRUNE && sp.b_caps2) {
+                    // the item's i-points against the whole chunk
+                    float4 ic[kGroups];
+#pragma unroll
+                    for (int gg = 0; gg < kGroups; ++gg)
+                        ic[gg] = gm[gg] ? __ldg(sp.a_caps + c.g.i0 / kCapPoints + gg) : make_float4(0.f, 0.f, 0.f, -1e30f);
+                    if (prune_block(wd, union_sphere(ic), __ldg(sp.b_caps2 + c.g.j0 / kPad))) {
+#pragma unroll
+                        for (int gg = 0; gg < kGroups; ++gg) {
+                            pruned += (unsigned long long)__popc(gm[gg]) * (kOpBlock * kOpBlock);
+                            gm[gg] = 0u;
+                        }
                     }
-                    groups |= in ? 1u << gg : 0u;
                 }
             }
-            uint32_t tiles = __ballot_sync(0xffffffffu, groups != 0u);
-            if (!tiles) continue;
-            // ---- the item's i-side operand
-            const uint32_t buf = acnt & 1u;
-            if (!tc_wait(a_empty + buf, ((acnt >> 1) & 1u) ^ 1u, limit, ctl, wd.stats)) break;
-            if (lane == 0) {
-                mbar_expect_tx(a_full + buf, kABytes);
-                bulk_copy_g2s(sptr<unsigned char>(wd.off_atile + buf * kABytes),
-                              sp.a_op + (size_t)(c.g.i0 / kOpBlock) * kOpABlock, kABytes, a_full + buf);
-            }
-            ++acnt;
-            // ---- its tiles
-            uint32_t first = kInfoNew;
-            while (tiles) {
-                const int k = __ffs((int)tiles) - 1;
-                tiles &= tiles - 1u;
-                const uint32_t gm = __shfl_sync(0xffffffffu, groups, k);
-                if (!tc_wait(empty + stage, phase ^ 1u, limit, ctl, wd.stats)) {
+            pairs = warp_sum(pairs);
+            if (lane == 0) atomicAdd(wd.stats + kStatPairs, pairs);
+            uint32_t items = __ballot_sync(0xffffffffu, (gm[0] | gm[1] | gm[2] | gm[3]) != 0u);
+            while (ok && items) {
+                const int l = __ffs((int)items) - 1;
+                items &= items - 1u;
+                const int sub = __shfl_sync(0xffffffffu, c.sub, l);
+                const uint32_t i0 = __shfl_sync(0xffffffffu, c.g.i0, l), j0 = __shfl_sync(0xffffffffu, c.g.j0, l);
+                uint32_t g0 = __shfl_sync(0xffffffffu, gm[0], l), g1 = __shfl_sync(0xffffffffu, gm[1], l),
+                         g2 = __shfl_sync(0xffffffffu, gm[2], l), g3 = __shfl_sync(0xffffffffu, gm[3], l);
+                const SubProblem& sp = sub_of(wd, sub);
+                if constexpr (PRUNE) {
+                    // every tile against every group, a tile per lane
+                    const uint32_t has = ((g0 >> lane) & 1u) | (((g1 >> lane) & 1u) << 1) | (((g2 >> lane) & 1u) << 2) |
+                                         (((g3 >> lane) & 1u) << 3);
+                    uint32_t keep = 0;
+                    if (has) {
+                        const float4 jt = __ldg(sp.b_caps + j0 / kCapPoints + (uint32_t)lane);
+#pragma unroll
+                        for (int gg = 0; gg < kGroups; ++gg)
+                            if (((has >> gg) & 1u) && !prune_block(wd, __ldg(sp.a_caps + i0 / kCapPoints + gg), jt))
+                                keep |= 1u << gg;
+                    }
+                    pruned += (unsigned long long)__popc(has ^ keep) * (kOpBlock * kOpBlock);
+                    g0 = __ballot_sync(0xffffffffu, keep & 1u);
+                    g1 = __ballot_sync(0xffffffffu, keep & 2u);
+                    g2 = __ballot_sync(0xffffffffu, keep & 4u);
+                    g3 = __ballot_sync(0xffffffffu, keep & 8u);
+                    if ((g0 | g1 | g2 | g3) == 0u) continue;
+                }
+                // ---- the item's i-side operand
+                const uint32_t buf = acnt & 1u;
+                if (!tc_wait(a_empty + buf, ((acnt >> 1) & 1u) ^ 1u, limit, ctl, wd.stats)) {
                     ok = false;
                     break;
                 }
                 if (lane == 0) {
-                    const uint32_t jt = c.g.j0 + (c.g.t_first + (uint32_t)k) * kOpBlock;
-                    volatile TcMeta* vm = meta + stage;
-                    vm->i0 = c.g.i0;
-                    vm->jbase = jt;
-                    vm->info = gm | (buf ? kInfoABuf : 0u) | first | (tiles ? 0u : kInfoLast) | ((uint32_t)c.sub << 16);
-                    fence_proxy_async_smem();  // the group's reads of the stage's previous tile come first
-                    if (!(hook && issued == 0)) {  // (test hook: the first copy is never issued)
-                        mbar_expect_tx(full + stage, kOpBBlock);
-                        bulk_copy_g2s(sptr<unsigned char>(wd.off_stage + stage * kOpBBlock),
-                                      sp.b_op + (size_t)(jt / kOpBlock) * kOpBBlock, kOpBBlock, full + stage);
-                    }
+                    mbar_expect_tx(a_full + buf, kABytes);
+                    bulk_copy_g2s(sptr<unsigned char>(wd.off_atile + buf * kABytes),
+                                  sp.a_op + (size_t)(i0 / kOpBlock) * kOpABlock, kABytes, a_full + buf);
                 }
-                first = 0;
-                ++issued;
-                if (++stage == S) {
-                    stage = 0;
-                    phase ^= 1u;
+                ++acnt;
+                // ---- its tiles
+                uint32_t first = kInfoNew, tiles = g0 | g1 | g2 | g3;
+                while (tiles) {
+                    const uint32_t t = (uint32_t)__ffs((int)tiles) - 1u;
+                    tiles &= tiles - 1u;
+                    if (!tc_wait(empty + stage, phase ^ 1u, limit, ctl, wd.stats)) {
+                        ok = false;
+                        break;
+                    }
+                    // the tile's i-groups; PRUNE: given to the groups of warps in turn, so that all work
+                    const uint32_t gs = ((g0 >> t) & 1u) | (((g1 >> t) & 1u) << 1) | (((g2 >> t) & 1u) << 2) |
+                                        (((g3 >> t) & 1u) << 3);
+                    uint32_t who = gs;
+                    if constexpr (PRUNE) {
+                        who = 0u;
+                        for (uint32_t m = gs; m; m &= m - 1u) {
+                            who |= (1u << turn) | (((uint32_t)__ffs((int)m) - 1u) << (8u + 2u * turn));
+                            turn = (turn + 1u) & 3u;
+                        }
+                    }
+                    if (lane == 0) {
+                        const uint32_t jt = j0 + t * kOpBlock;
+                        volatile TcMeta* vm = meta + stage;
+                        vm->i0 = i0;
+                        vm->jbase = jt;
+                        vm->info = who | (buf ? kInfoABuf : 0u) | first | (tiles ? 0u : kInfoLast) |
+                                   ((uint32_t)sub << 16);
+                        fence_proxy_async_smem();  // the group's reads of the stage's previous tile come first
+                        if (!(hook && issued == 0)) {  // (test hook: the first copy is never issued)
+                            mbar_expect_tx(full + stage, kOpBBlock);
+                            bulk_copy_g2s(sptr<unsigned char>(wd.off_stage + stage * kOpBBlock),
+                                          sp.b_op + (size_t)(jt / kOpBlock) * kOpBBlock, kOpBBlock, full + stage);
+                        }
+                    }
+                    first = 0;
+                    ++issued;
+                    if (++stage == S) {
+                        stage = 0;
+                        phase ^= 1u;
+                    }
                 }
             }
         }
@@ -577,7 +693,7 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
             mbar_arrive(full + stage);
         }
         __syncwarp();
-        if (wd.prune) {
+        if constexpr (PRUNE) {
             pruned = warp_sum(pruned);
             if (lane == 0 && pruned) atomicAdd(wd.stats + kStatPruned, pruned);
         }
@@ -593,11 +709,10 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (warp == kIssueWarp)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)kTmemCols));
+    if (warp == kIssueWarp) tc_dealloc(tmem);
 }
 
-template <bool PREEMPT>
+template <bool PREEMPT, bool PRUNE>
 cudaError_t launch_tc_t(const WorkDesc& wd_in, const Shape& sh, cudaStream_t stream) {
     WorkDesc wd = wd_in;
     const TcLayout L = tc_layout((int)wd.stages, wd.nedges_max);
@@ -619,7 +734,7 @@ cudaError_t launch_tc_t(const WorkDesc& wd_in, const Shape& sh, cudaStream_t str
     wd.stage_bytes = kOpBBlock;
     if (L.total > sh.smem || wd.I != 128u * kGroups || wd.J != kOpBlock || wd.Jc > 32u * kOpBlock)
         return cudaErrorInvalidValue;
-    count_tc_kernel<PREEMPT><<<sh.blocks, kThreads, sh.smem, stream>>>(wd);
+    count_tc_kernel<PREEMPT, PRUNE><<<sh.blocks, kThreads, sh.smem, stream>>>(wd);
     return cudaGetLastError();
 }
 
@@ -632,15 +747,16 @@ cudaError_t count_tc_set_smem_limit() {
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     // (the opt-in maximum: the attribute belongs to the kernel, not to a launch)
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(count_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(count_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
+    const void* kernels[4] = {(const void*)count_tc_kernel<false, false>, (const void*)count_tc_kernel<true, false>,
+                              (const void*)count_tc_kernel<false, true>, (const void*)count_tc_kernel<true, true>};
+    for (const void* k : kernels)
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
     return e;
 }
 
 cudaError_t launch_count_tc(const WorkDesc& wd, const Shape& sh, bool preempt, cudaStream_t stream) {
-    return preempt ? launch_tc_t<true>(wd, sh, stream) : launch_tc_t<false>(wd, sh, stream);
+    if (wd.prune) return preempt ? launch_tc_t<true, true>(wd, sh, stream) : launch_tc_t<false, true>(wd, sh, stream);
+    return preempt ? launch_tc_t<true, false>(wd, sh, stream) : launch_tc_t<false, false>(wd, sh, stream);
 }
 
 }  // namespace tpcf

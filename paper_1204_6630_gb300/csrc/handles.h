@@ -70,6 +70,7 @@ struct tpcf_catalog {
     float4* d32 = nullptr;
     float* soa = nullptr;           // FP32 points as x | y | z arrays of n_pad floats (the staged j-tiles)
     unsigned char *op_a = nullptr, *op_b = nullptr;  // tensor-core operands (unit-vector catalogs)
+    float4* caps2 = nullptr;        // bounding sphere of each kPad-point block (in the allocation of caps)
     float4* caps = nullptr;         // bounding sphere of each kCapPoints-point group (spatial pruning)
     std::vector<uint64_t> offsets;  // segments (empty = one segment), input order
     std::vector<uint64_t> seg_start;  // device position of each segment's first point (multiples of

@@ -317,10 +317,38 @@ __global__ void prep_caps_kernel(const Point64* __restrict__ p64, uint32_t n_gro
     if (lane == 0) caps[grp] = make_float4(cx, cy, cz, __double2float_ru(r * (1.0 + 0x1p-20)));
 }
 
+// Bounding sphere of each kPad-point block from its groups' spheres (one warp
+// per block, a group per lane): centre the FP32 mean of the non-empty groups'
+// centres, radius the largest |c - c_g| + r_g, enlarged by 2^-20; an empty
+// block gets radius -1e30 like an empty group.
+__global__ void prep_caps2_kernel(const float4* __restrict__ caps, uint32_t n_blocks, float4* caps2) {
+    static_assert(kPad == 32 * kCapPoints, "one group per lane");
+    const uint32_t blk = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (blk >= n_blocks) return;  // warp-uniform
+    const float4 g = caps[(size_t)blk * 32u + (threadIdx.x & 31u)];
+    const bool real = g.w > -1e29f;
+    float x = real ? g.x : 0.f, y = real ? g.y : 0.f, z = real ? g.z : 0.f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        x += __shfl_xor_sync(0xffffffffu, x, o);
+        y += __shfl_xor_sync(0xffffffffu, y, o);
+        z += __shfl_xor_sync(0xffffffffu, z, o);
+    }
+    const int n = __popc(__ballot_sync(0xffffffffu, real));
+    const float inv = 1.0f / (float)max(n, 1);
+    const float cx = x * inv, cy = y * inv, cz = z * inv;
+    const float dx = cx - g.x, dy = cy - g.y, dz = cz - g.z;
+    float r = real ? sqrtf(fmaf(dz, dz, fmaf(dy, dy, dx * dx))) + g.w : 0.f;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) r = fmaxf(r, __shfl_xor_sync(0xffffffffu, r, o));
+    if ((threadIdx.x & 31u) == 0)
+        caps2[blk] = n ? make_float4(cx, cy, cz, r * (1.0f + 9.5367431640625e-07f)) : make_float4(0.f, 0.f, 0.f, -1e30f);
+}
+
 cudaError_t launch_prepare(const double* xyz_in, uint32_t n, const uint32_t* seg_of_point,
                            const uint32_t* seg_delta, int sort, int euclid, unsigned long long* bbox,
                            Point64* out64, float4* out32, float* out_soa, unsigned char* op_a, unsigned char* op_b,
-                           float4* caps, uint32_t n_pad, unsigned long long* keys, uint32_t* vals, uint32_t n_pow2,
+                           float4* caps, float4* caps2, uint32_t n_pad, unsigned long long* keys, uint32_t* vals, uint32_t n_pow2,
                            unsigned long long* err_word, unsigned long long* eps_word, cudaStream_t stream,
                            uint32_t* launches) {
     cudaError_t e;
@@ -378,6 +406,10 @@ cudaError_t launch_prepare(const double* xyz_in, uint32_t n, const uint32_t* seg
         const uint32_t groups = n_pad / kCapPoints;  // n_pad is a multiple of kPad
         prep_caps_kernel<<<(groups + 7) / 8, 256, 0, stream>>>(out64, groups, euclid,
                                                                euclid ? kCapScale3d : 1.0, caps);
+        ++nl;
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        const uint32_t blocks = n_pad / kPad;
+        prep_caps2_kernel<<<(blocks + 7) / 8, 256, 0, stream>>>(caps, blocks, caps2);
         ++nl;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }

@@ -736,10 +736,11 @@ int tpcf::catalog_create_impl(tpcf_ctx* ctx, const double* xyz, uint64_t n, int 
     if (alloc((void**)&c->d64, (size_t)c->n_pad * sizeof(Point64)) != cudaSuccess ||
         alloc((void**)&c->d32, (size_t)c->n_pad * sizeof(float4)) != cudaSuccess ||
         alloc((void**)&c->soa, (size_t)c->n_pad * 3 * sizeof(float)) != cudaSuccess ||
-        alloc((void**)&c->caps, (size_t)(c->n_pad / kCapPoints) * sizeof(float4)) != cudaSuccess ||
+        alloc((void**)&c->caps, (size_t)(c->n_pad / kCapPoints + c->n_pad / kPad) * sizeof(float4)) != cudaSuccess ||
         (!euclid && (alloc((void**)&c->op_a, (size_t)(c->n_pad / kOpBlock) * kOpABlock) != cudaSuccess ||
                      alloc((void**)&c->op_b, (size_t)(c->n_pad / kOpBlock) * kOpBBlock) != cudaSuccess)))
         return fail_with(TPCF_ENOMEM, "device allocation failed");
+    c->caps2 = c->caps + c->n_pad / kCapPoints;
     const double* in = xyz;
     if (n > 0 && where == TPCF_HOST) {
         if (cudaMallocAsync(&tmp_in, n * 24, st) != cudaSuccess)
@@ -780,7 +781,7 @@ int tpcf::catalog_create_impl(tpcf_ctx* ctx, const double* xyz, uint64_t n, int 
     }
     uint32_t nl = 0;
     cudaError_t e = launch_prepare(in, (uint32_t)n, seg, seg_delta, sort ? 1 : 0, euclid ? 1 : 0, err + 2, c->d64,
-                                   c->d32, c->soa, c->op_a, c->op_b, c->caps, c->n_pad, keys, vals, n_pow2, err, err + 1, st, &nl);
+                                   c->d32, c->soa, c->op_a, c->op_b, c->caps, c->caps2, c->n_pad, keys, vals, n_pow2, err, err + 1, st, &nl);
     ctx->launches.fetch_add(nl);
     if (e != cudaSuccess) return fail_with(TPCF_ECUDA, cudaGetErrorString(e));
     unsigned long long hw[2] = {0, 0};
@@ -976,6 +977,7 @@ uint64_t build_work(tpcf_ctx* ctx, const SubSpec* specs, int nsub, const BinsDev
         sp.b64 = p.b->d64 + p.b_off;
         sp.a_caps = p.a->caps + p.a_off / kCapPoints;  // sub-ranges start on kSegAlign boundaries
         sp.b_caps = p.b->caps + p.b_off / kCapPoints;
+        sp.b_caps2 = p.b_off % kPad == 0 ? p.b->caps2 + p.b_off / kPad : nullptr;
         sp.a_op = p.a->op_a ? p.a->op_a + (size_t)(p.a_off / kOpBlock) * kOpABlock : nullptr;
         sp.b_op = p.b->op_b ? p.b->op_b + (size_t)(p.b_off / kOpBlock) * kOpBBlock : nullptr;
         sp.na = p.na;
@@ -1207,6 +1209,12 @@ int run_counts(tpcf_ctx* ctx, const SubSpec* specs, int nsub, const tpcf_bins* b
         wd.stats = stat_w;
         wd.item_counter = stat_w + kStatNextItem;
         fill_scalars(ctx, specs, nsub, bh, mode, shp, force_idx, ne, wd);
+        // items per draw: one, unless most are pruned away (then up to 32, as long as
+        // every SM still draws some 16 times)
+        wd.draw_batch = 1;
+        if (wd.prune)
+            wd.draw_batch = (uint32_t)std::min<uint64_t>(
+                32, std::max<uint64_t>(1, (wd.item_hi - wd.item_lo) / (16ull * (uint64_t)ctx->num_sms)));
         return TPCF_OK;
     };
     auto smem_limit = [&](const Shape& shp) {

@@ -105,7 +105,8 @@ struct SubProblem {
     // starting at the sub-range's first point (spatial pruning).
     const float4* a_caps;
     const float4* b_caps;
-    // Tensor-core operands of A (i-side) and B (j-side), the sub-range's first block.
+    // Tensor-core kernel: operands of A (i-side) and B (j-side), the sub-range's first block.
+    const float4* b_caps2;       // spheres of B's kPad-point blocks; NULL: the sub-range does not start on one
     const unsigned char* a_op;
     const unsigned char* b_op;
 };
@@ -147,6 +148,7 @@ struct WorkDesc {
     // positions it took.
     uint64_t pos_lo;
     uint32_t draw_warps;
+    uint32_t draw_batch;             // tensor-core kernel: items per draw (1..32)
     // serving steps (the multi-job kernel): the step's slices, sorted by position,
     // and one item counter per slice (zeroed before the launch)
     const StepSlice* slices;
@@ -227,7 +229,7 @@ cudaError_t launch_finalize_batch(const unsigned long long* acc, int acc_stride,
 cudaError_t launch_prepare(const double* xyz_in, uint32_t n, const uint32_t* seg_of_point,
                            const uint32_t* seg_delta, int sort, int euclid, unsigned long long* bbox,
                            Point64* out64, float4* out32, float* out_soa, unsigned char* op_a, unsigned char* op_b,
-                           float4* caps, uint32_t n_pad,
+                           float4* caps, float4* caps2, uint32_t n_pad,
                            unsigned long long* key_scratch, uint32_t* val_scratch,
                            uint32_t n_pow2, unsigned long long* err_word, unsigned long long* eps_word,
                            cudaStream_t stream, uint32_t* launches);
