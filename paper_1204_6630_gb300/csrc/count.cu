@@ -229,7 +229,7 @@ __device__ __forceinline__ void advance(const WorkDesc& wd, Cursor& c, unsigned 
 template <int R>
 struct PairSource {
     float x[R], y[R], z[R];
-    const float *sx, *sy, *sz;
+    const float* tile;  // blocks of kBlk points, x | y | z each
     uint32_t i0, jbase;
 };
 
@@ -257,7 +257,8 @@ __device__ __forceinline__ void drain_batch(const WorkDesc& wd, const SubProblem
     }
     if (has) {
         const uint32_t ig = ps.i0 + (uint32_t)l + 32u * (uint32_t)r, jg = ps.jbase + jo;
-        hist_inc<T>(hc, classify_unsettled<EUCLID>(wd, sp, ax, ay, az, ps.sx[jo], ps.sy[jo], ps.sz[jo], ig, jg,
+        const float* b = ps.tile + (jo / kBlk) * (3 * kBlk) + jo % kBlk;
+        hist_inc<T>(hc, classify_unsettled<EUCLID>(wd, sp, ax, ay, az, b[0], b[kBlk], b[2 * kBlk], ig, jg,
                                                    band, mism));
     }
 }
@@ -599,10 +600,10 @@ __global__ void __launch_bounds__(T, 1) count_kernel(const __grid_constant__ Wor
         if constexpr (PLAIN) {
             bulk_copy_g2s(dst, sp.b64 + jbase, wd.stage_bytes, bar);
         } else {
-            const uint32_t plane = wd.J * 4u;  // x | y | z arrays of J floats
-            bulk_copy_g2s(dst, sp.b_soa + jbase, plane, bar);
-            bulk_copy_g2s(dst + plane, sp.b_soa + sp.b_soa_stride + jbase, plane, bar);
-            bulk_copy_g2s(dst + 2 * plane, sp.b_soa + 2ull * sp.b_soa_stride + jbase, plane, bar);
+            // the x | y | z arrays of the tile's blocks (J is a multiple of kBlk)
+            const unsigned char* src = sp.b_blk + (size_t)(jbase / kBlk) * kBlkBytes + kBlkX;
+            for (uint32_t o = 0; o < wd.stage_bytes; o += kBlk * 12u, src += kBlkBytes)
+                bulk_copy_g2s(dst + o, src, kBlk * 12u, bar);
         }
     };
 
@@ -685,7 +686,7 @@ __global__ void __launch_bounds__(T, 1) count_kernel(const __grid_constant__ Wor
                     dy[r] = p.y;
                     dz[r] = p.z;
                 } else {
-                    const float4 p = __ldg(sp.a32 + i);
+                    const float3 p = ldg_point32(sp.a_blk, i);
                     ax2[r] = pack2(p.x, p.x);
                     ay2[r] = pack2(p.y, p.y);
                     az2[r] = pack2(p.z, p.z);
@@ -770,9 +771,8 @@ __global__ void __launch_bounds__(T, 1) count_kernel(const __grid_constant__ Wor
             // lane may be in range (angles: some e >= 0; 3-D: some e' <= 0).  The loop
             // does not branch per group: after kMaskGroups groups one warp reduction
             // names the groups that take the slow path, which recomputes their values.
-            const float* sx = sptr<const float>(stage_off);
-            const float* sy = sx + J;
-            const float* sz = sy + J;
+            // (the tile: blocks of kBlk points, x | y | z each)
+            const float* const tile = sptr<const float>(stage_off);
             // angles: (-T, -T); 3-D: (-H, -H), read from the kernel parameter
             const u64 nt2 = wd.neg_fast_t2;
             constexpr int CH = kMaskGroups * U;                     // j-points per mask chunk
@@ -785,15 +785,18 @@ __global__ void __launch_bounds__(T, 1) count_kernel(const __grid_constant__ Wor
                 src.y[r] = lo_of(ay2[r]);
                 src.z[r] = lo_of(az2[r]);
             }
-            src.sx = sx;
-            src.sy = sy;
-            src.sz = sz;
+            src.tile = tile;
             src.i0 = g_i0;
             src.jbase = jbase;
             static_assert(kMaskGroups <= 32, "one mask bit per group");
 #pragma unroll 1
             for (int jc = 0; jc < J; jc += CH) {
                 if (wd.prune && prune_chunk(wd, jbase + (uint32_t)jc, IB * CH)) continue;
+                // a chunk lies in one block: its points j at sx[j], sy[j], sz[j] (j from the tile's first)
+                static_assert((int)kBlk % CH == 0, "a chunk lies in one block");
+                const float* const sx = tile + 2 * (jc & ~((int)kBlk - 1));
+                const float* const sy = sx + kBlk;
+                const float* const sz = sy + kBlk;
                 uint32_t lane_mask = 0;
 #pragma unroll 4
                 for (int gi = 0; gi < kMaskGroups; ++gi) {

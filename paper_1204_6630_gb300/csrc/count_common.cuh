@@ -361,11 +361,11 @@ __device__ __forceinline__ Resolved resolve_f32(const WorkDesc& wd, float c, int
     return Resolved{-1, nb_, na_, h};
 }
 
-// Screen value of pair (ig, jg) recomputed from the FP32 copies, bit-identical
-// to the kernel's (fma.rn.f32x2 rounds each half as fmaf does).
-__device__ __forceinline__ float screen_value(const WorkDesc& wd, const SubProblem& sp, uint32_t ig, uint32_t jg) {
-    const float4 a = __ldg(sp.a32 + ig), b = __ldg(sp.b32 + jg);
-    return fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, wd.neg_fast_t)));
+// FP32 coordinates of point i of a blocked catalog (lanes with consecutive
+// points read consecutive words).
+__device__ __forceinline__ float3 ldg_point32(const unsigned char* blk, uint32_t i) {
+    const float* p = reinterpret_cast<const float*>(blk + (size_t)(i / kBlk) * kBlkBytes + kBlkX) + i % kBlk;
+    return make_float3(__ldg(p), __ldg(p + kBlk), __ldg(p + 2 * kBlk));
 }
 
 // LUT entry of screen value e: cell k = rne(sat(e * 2^-q) * 2^14), read as the

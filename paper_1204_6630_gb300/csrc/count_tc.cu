@@ -12,7 +12,7 @@
 // binary16 values, a = a1 + a2 + r with |r| <= 2^-22 |a| + 2^-25, and a pair's
 // screen value is the K = 16 product
 //   D = sum_c a1 b1 + a2 b2 + a1 b2 + a2 b1,   c = x, y, z:
-// the i-side record is [X | X] and the j-side record [X | Y] with X = (x1, y1,
+// the j-side record is [X | X] and the i-side record [X | Y] with X = (x1, y1,
 // z1, x2, y2, z2, 0, 0) and Y = (x2, y2, z2, x1, y1, z1, 0, 0).  Products of
 // binary16 values are exact in binary32; with accumulation in at least single
 // precision D is within 44u of the binary64 dot d (u = 2^-24: 2u from the FP32
@@ -46,7 +46,10 @@ constexpr int kIssueWarp = kWorkWarps;            // .. + kGroups - 1: the group
 constexpr int kLoadWarp = kWorkWarps + kGroups;
 constexpr int kThreads = 32 * (kLoadWarp + 1);
 constexpr int kTmemCols = 512;                    // 128 columns per group
-constexpr uint32_t kABytes = 4 * kOpABlock;       // i-side operand of an item (512 points)
+constexpr uint32_t kABlock = 2 * kBlkX;            // i-side operand of 128 points: planes X and Y
+constexpr uint32_t kABytes = kGroups * kABlock;   // ... of an item
+constexpr uint32_t kStageX2 = kBlkBytes;          // a stage: the tile's block (X, x | y | z), then X once more
+constexpr uint32_t kStageBytes = kBlkBytes + kBlkX;
 constexpr int kQueueCodes = 64;                   // per-warp queue of unsettled pairs
 
 // Control words.  kTcBeat changes with every batch of items the loader draws:
@@ -84,7 +87,7 @@ __host__ __device__ inline TcLayout tc_layout(int S, int nedges) {
     L.meta = off; off += (uint32_t)S * (uint32_t)sizeof(TcMeta);
     off = align_up(off, 128);
     L.atile = off; off += 2 * kABytes;
-    L.stage = off; off += (uint32_t)S * kOpBBlock;
+    L.stage = off; off += (uint32_t)S * kStageBytes;
     L.hist = off; off += (uint32_t)(nedges + 1) * (uint32_t)(kWorkThreads / 2) * 4;
     off = align_up(off, 16);
     L.cos_thr = off; off += (uint32_t)nedges * 8;
@@ -122,9 +125,9 @@ __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence:
 
 // Shared-memory matrix descriptor of a K-major operand without swizzle: rows
 // in groups of 8, a group's two 8 x 16-byte core matrices at `addr` + 0 and
-// + 2048 (the X and the second plane of 128 points), groups 128 bytes apart.
-__device__ __forceinline__ uint64_t op_desc(uint32_t addr) {
-    return (uint64_t)((addr >> 4) & 0x3fffu) | ((uint64_t)(2048u >> 4) << 16) | ((uint64_t)(128u >> 4) << 32) |
+// + `second` (its rows of the two planes of 128 points), groups 128 bytes apart.
+__device__ __forceinline__ uint64_t op_desc(uint32_t addr, uint32_t second) {
+    return (uint64_t)((addr >> 4) & 0x3fffu) | ((uint64_t)(second >> 4) << 16) | ((uint64_t)(128u >> 4) << 32) |
            (1ull << 46);
 }
 
@@ -235,8 +238,8 @@ __device__ __forceinline__ uint32_t tc_block(const WorkDesc& wd, u64 ax, u64 ay,
     for (int k = 0; k < 9; ++k) {
         if (k < 8) {
             const ulonglong2 bx = *reinterpret_cast<const ulonglong2*>(sx + 4 * k);
-            const ulonglong2 by = *reinterpret_cast<const ulonglong2*>(sx + kOpBlock + 4 * k);
-            const ulonglong2 bz = *reinterpret_cast<const ulonglong2*>(sx + 2 * kOpBlock + 4 * k);
+            const ulonglong2 by = *reinterpret_cast<const ulonglong2*>(sx + kBlk + 4 * k);
+            const ulonglong2 bz = *reinterpret_cast<const ulonglong2*>(sx + 2 * kBlk + 4 * k);
             const u64 v0 = ffma2(az, bz.x, ffma2(ay, by.x, ffma2(ax, bx.x, nt2)));
             const u64 v1 = ffma2(az, bz.y, ffma2(ay, by.y, ffma2(ax, bx.y, nt2)));
             const float e[4] = {lo_of(v0), hi_of(v0), lo_of(v1), hi_of(v1)};
@@ -274,7 +277,7 @@ __device__ __forceinline__ void tc_drain(const WorkDesc& wd, const SubProblem& s
     const float y = __shfl_sync(0xffffffffu, lo_of(ay), l);
     const float z = __shfl_sync(0xffffffffu, lo_of(az), l);
     if (has) {
-        const float4 b = __ldg(sp.b32 + jg);
+        const float3 b = ldg_point32(sp.b_blk, jg);
         hist_inc<kWorkThreads>(hc, classify_unsettled<false>(wd, sp, x, y, z, b.x, b.y, b.z, iw + (uint32_t)l, jg,
                                                              band, mism));
     }
@@ -394,7 +397,7 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                 }
                 const int sub = (int)(info >> 16);
                 const SubProblem& sp = sub_of(wd, sub);
-                iw = vm->i0 + kOpBlock * gi + 32u * (uint32_t)(warp & 3);
+                iw = vm->i0 + kBlk * gi + 32u * (uint32_t)(warp & 3);
                 jq0 = jbase;
                 unsigned long long* tgt = sp.hist;
                 if (sp.row_seg) tgt += (size_t)__ldg(sp.row_seg + iw / kSegAlign) * sp.row_stride;
@@ -404,14 +407,14 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                 na = sp.na;
                 nb = sp.nb;
                 rule = sp.auto_mode ? 1u : (sp.no_self ? 2u : 0u);
-                const float4 p = __ldg(sp.a32 + iw + (uint32_t)lane);
+                const float3 p = ldg_point32(sp.a_blk, iw + (uint32_t)lane);
                 ax = pack2(p.x, p.x);
                 ay = pack2(p.y, p.y);
                 az = pack2(p.z, p.z);
             }
             uint32_t nbatch = 0, kept = 0;
             // a lane's counter gains at most one per pair of the tile and one per queue batch
-            if (inc_bound + 2u * kOpBlock + 2u > 0xffffu || over > 0x40000000u) flush();
+            if (inc_bound + 2u * kBlk + 2u > 0xffffu || over > 0x40000000u) flush();
             if ((info >> g) & 1u) {
                 // ---- the group's accumulators: one maximum per 32 x 32 pairs
                 if (!tc_wait(d_full + g, dphase, limit, ctl, wd.stats)) {
@@ -436,8 +439,8 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                 if (rule == 1u && jbase < iw) todo &= ~0u << ((iw - jbase) >> 5 < 4u ? (iw - jbase) >> 5 : 4u);
                 // (a counted block's overflow needs its pair mask; otherwise a mask is needed on the
                 // diagonal and, where padding could look in range, at the catalogs' ends)
-                const bool ends = (wd.need_idx || check) && (jbase + kOpBlock > nb || iw + 32u > na);
-                const float* sx = sptr<const float>(wd.off_stage + stage * kOpBBlock + kOpBCoord);
+                const bool ends = (wd.need_idx || check) && (jbase + kBlk > nb || iw + 32u > na);
+                const float* sx = sptr<const float>(wd.off_stage + stage * kStageBytes + kBlkX);
                 while (todo) {
                     const uint32_t b = (uint32_t)__ffs((int)todo) - 1u;
                     todo &= todo - 1u;
@@ -526,8 +529,8 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                 if (lane == 0) {
                     tc_mma(tmem + (uint32_t)(g * 128),
                            op_desc(smem_addr(dyn_smem) + wd.off_atile + buf * kABytes +
-                                   (PRUNE ? (info >> (8 + 2 * g)) & 3u : (uint32_t)g) * kOpABlock),
-                           op_desc(smem_addr(dyn_smem) + wd.off_stage + stage * kOpBBlock));
+                                   (PRUNE ? (info >> (8 + 2 * g)) & 3u : (uint32_t)g) * kABlock, kBlkX),
+                           op_desc(smem_addr(dyn_smem) + wd.off_stage + stage * kStageBytes, kStageX2));
                     tc_commit(d_full + g);
                 }
                 any = true;
@@ -582,9 +585,9 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                                    (uint64_t)c.g.j0 + (uint64_t)c.g.t_end * wd.J, sp.na, sp.nb, sp.auto_mode != 0);
 #pragma unroll
                 for (int gg = 0; gg < kGroups; ++gg) {
-                    const uint32_t ib = c.g.i0 + kOpBlock * (uint32_t)gg;
+                    const uint32_t ib = c.g.i0 + kBlk * (uint32_t)gg;
                     uint32_t t0 = c.g.t_first;  // (auto counts: tiles from the group's own on)
-                    if (sp.auto_mode && ib > c.g.j0) t0 = max(t0, (ib - c.g.j0) / kOpBlock);
+                    if (sp.auto_mode && ib > c.g.j0) t0 = max(t0, (ib - c.g.j0) / kBlk);
                     if (ib < sp.na && t0 < c.g.t_end) gm[gg] = (0xffffffffu >> (32u - (c.g.t_end - t0))) << t0;
                 }
                 if (PRUNE && sp.b_caps2) {
@@ -596,7 +599,7 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                     if (prune_block(wd, union_sphere(ic), __ldg(sp.b_caps2 + c.g.j0 / kPad))) {
 #pragma unroll
                         for (int gg = 0; gg < kGroups; ++gg) {
-                            pruned += (unsigned long long)__popc(gm[gg]) * (kOpBlock * kOpBlock);
+                            pruned += (unsigned long long)__popc(gm[gg]) * (kBlk * kBlk);
                             gm[gg] = 0u;
                         }
                     }
@@ -625,7 +628,7 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                             if (((has >> gg) & 1u) && !prune_block(wd, __ldg(sp.a_caps + i0 / kCapPoints + gg), jt))
                                 keep |= 1u << gg;
                     }
-                    pruned += (unsigned long long)__popc(has ^ keep) * (kOpBlock * kOpBlock);
+                    pruned += (unsigned long long)__popc(has ^ keep) * (kBlk * kBlk);
                     g0 = __ballot_sync(0xffffffffu, keep & 1u);
                     g1 = __ballot_sync(0xffffffffu, keep & 2u);
                     g2 = __ballot_sync(0xffffffffu, keep & 4u);
@@ -638,10 +641,27 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                     ok = false;
                     break;
                 }
-                if (lane == 0) {
-                    mbar_expect_tx(a_full + buf, kABytes);
-                    bulk_copy_g2s(sptr<unsigned char>(wd.off_atile + buf * kABytes),
-                                  sp.a_op + (size_t)(i0 / kOpBlock) * kOpABlock, kABytes, a_full + buf);
+                {
+                    const unsigned char* src = sp.a_blk + (size_t)(i0 / kBlk) * kBlkBytes;
+                    uint4* const dst = sptr<uint4>(wd.off_atile + buf * kABytes);
+#pragma unroll 2
+                    for (int gg = 0; gg < kGroups; ++gg) {
+                        uint4 x[4];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            x[k] = __ldg(reinterpret_cast<const uint4*>(src + (size_t)gg * kBlkBytes) + 32 * k + lane);
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            uint4* const p = dst + gg * (kABlock / 16) + 32 * k + lane;
+                            p[0] = x[k];
+                            // Y: the halves' two triples exchanged
+                            p[kBlk] = make_uint4((x[k].y >> 16) | (x[k].z << 16), (x[k].z >> 16) | (x[k].x << 16),
+                                                 (x[k].x >> 16) | (x[k].y << 16), 0u);
+                        }
+                    }
+                    fence_proxy_async_smem();  // the products read it through the asynchronous proxy
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(a_full + buf);
                 }
                 ++acnt;
                 // ---- its tiles
@@ -665,7 +685,7 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                         }
                     }
                     if (lane == 0) {
-                        const uint32_t jt = j0 + t * kOpBlock;
+                        const uint32_t jt = j0 + t * kBlk;
                         volatile TcMeta* vm = meta + stage;
                         vm->i0 = i0;
                         vm->jbase = jt;
@@ -673,9 +693,11 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                                    ((uint32_t)sub << 16);
                         fence_proxy_async_smem();  // the group's reads of the stage's previous tile come first
                         if (!(hook && issued == 0)) {  // (test hook: the first copy is never issued)
-                            mbar_expect_tx(full + stage, kOpBBlock);
-                            bulk_copy_g2s(sptr<unsigned char>(wd.off_stage + stage * kOpBBlock),
-                                          sp.b_op + (size_t)(jt / kOpBlock) * kOpBBlock, kOpBBlock, full + stage);
+                            const unsigned char* src = sp.b_blk + (size_t)(jt / kBlk) * kBlkBytes;
+                            unsigned char* const dst = sptr<unsigned char>(wd.off_stage + stage * kStageBytes);
+                            mbar_expect_tx(full + stage, kStageBytes);
+                            bulk_copy_g2s(dst, src, kBlkBytes, full + stage);
+                            bulk_copy_g2s(dst + kStageX2, src, kBlkX, full + stage);
                         }
                     }
                     first = 0;
@@ -702,8 +724,6 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
             const uint32_t back = issued < S ? issued : S;
             for (uint32_t k = issued - back; k < issued; ++k)
                 if (!(hook && k == 0)) (void)mbar_wait_bounded(full + k % S, (k / S) & 1u, limit);
-            for (uint32_t k = acnt < 2u ? 0u : acnt - 2u; k < acnt; ++k)
-                (void)mbar_wait_bounded(a_full + (k & 1u), (k >> 1) & 1u, limit);
         }
     }
     tc_fence_before();
@@ -731,8 +751,8 @@ cudaError_t launch_tc_t(const WorkDesc& wd_in, const Shape& sh, cudaStream_t str
     wd.off_lut = L.lut;
     wd.off_queue = L.queue;
     wd.off_bwd = L.bwd;
-    wd.stage_bytes = kOpBBlock;
-    if (L.total > sh.smem || wd.I != 128u * kGroups || wd.J != kOpBlock || wd.Jc > 32u * kOpBlock)
+    wd.stage_bytes = kStageBytes;
+    if (L.total > sh.smem || wd.I != 128u * kGroups || wd.J != kBlk || wd.Jc > 32u * kBlk)
         return cudaErrorInvalidValue;
     count_tc_kernel<PREEMPT, PRUNE><<<sh.blocks, kThreads, sh.smem, stream>>>(wd);
     return cudaGetLastError();

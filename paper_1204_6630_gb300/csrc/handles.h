@@ -67,9 +67,7 @@ struct tpcf_catalog {
     uint64_t n = 0;
     uint32_t n_pad = 0;
     tpcf::Point64* d64 = nullptr;
-    float4* d32 = nullptr;
-    float* soa = nullptr;           // FP32 points as x | y | z arrays of n_pad floats (the staged j-tiles)
-    unsigned char *op_a = nullptr, *op_b = nullptr;  // tensor-core operands (unit-vector catalogs)
+    unsigned char* blk = nullptr;   // FP32 points and tensor-core operands in blocks (see kBlk)
     float4* caps2 = nullptr;        // bounding sphere of each kPad-point block (in the allocation of caps)
     float4* caps = nullptr;         // bounding sphere of each kCapPoints-point group (spatial pruning)
     std::vector<uint64_t> offsets;  // segments (empty = one segment), input order

@@ -200,26 +200,19 @@ __device__ __forceinline__ uint32_t split16(float v) {  // hi | lo << 16
     return (uint32_t)__half_as_ushort(h) | ((uint32_t)__half_as_ushort(l) << 16);
 }
 
-// Writes point q's records into the tensor-core operands (layout: tpcf_internal.h).
-__device__ __forceinline__ void put_operands(unsigned char* op_a, unsigned char* op_b, uint32_t q, float x, float y,
-                                             float z) {
-    const uint32_t sx = split16(x), sy = split16(y), sz = split16(z);
-    const uint32_t h01 = __byte_perm(sx, sy, 0x5410), l01 = __byte_perm(sx, sy, 0x7632);
-    const uint32_t h2 = sz & 0xffffu, l2 = sz >> 16;
-    const uint4 X = make_uint4(h01, h2 | (l01 << 16), (l01 >> 16) | (l2 << 16), 0u);
-    const uint4 Y = make_uint4(l01, l2 | (h01 << 16), (h01 >> 16) | (h2 << 16), 0u);
-    const uint32_t o = q % kOpBlock;
-    uint4* a = reinterpret_cast<uint4*>(op_a + (size_t)(q / kOpBlock) * kOpABlock);
-    unsigned char* bb = op_b + (size_t)(q / kOpBlock) * kOpBBlock;
-    uint4* b = reinterpret_cast<uint4*>(bb);
-    a[o] = X;
-    a[kOpBlock + o] = X;
-    b[o] = X;
-    b[kOpBlock + o] = Y;
-    float* f = reinterpret_cast<float*>(bb + kOpBCoord);
+// Writes point q's FP32 coordinates and operand record into its block.
+__device__ __forceinline__ void put_block(unsigned char* blk, uint32_t q, float x, float y, float z, bool operand) {
+    unsigned char* b = blk + (size_t)(q / kBlk) * kBlkBytes;
+    const uint32_t o = q % kBlk;
+    if (operand) {
+        const uint32_t sx = split16(x), sy = split16(y), sz = split16(z);
+        reinterpret_cast<uint4*>(b)[o] =
+            make_uint4(__byte_perm(sx, sy, 0x5410), __byte_perm(sz, sx, 0x7610), __byte_perm(sy, sz, 0x7632), 0u);
+    }
+    float* f = reinterpret_cast<float*>(b + kBlkX);
     f[o] = x;
-    f[kOpBlock + o] = y;
-    f[2 * kOpBlock + o] = z;
+    f[kBlk + o] = y;
+    f[2 * kBlk + o] = z;
 }
 
 // Gather points in sorted order into the binary64 and FP32 device copies (the
@@ -228,8 +221,8 @@ __device__ __forceinline__ void put_operands(unsigned char* op_a, unsigned char*
 // segmented catalog start on aligned positions; seg_delta = NULL: no shift).
 __global__ void prep_gather_kernel(const double* __restrict__ xyz, uint32_t n,
                                    const uint32_t* __restrict__ order, const uint32_t* __restrict__ seg_of_point,
-                                   const uint32_t* __restrict__ seg_delta, Point64* out64, float4* out32,
-                                   float* out_soa, unsigned char* op_a, unsigned char* op_b, uint32_t n_pad) {
+                                   const uint32_t* __restrict__ seg_delta, Point64* out64,
+                                   unsigned char* blk, int euclid) {
     const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
     const uint32_t s = order ? order[p] : p;
@@ -237,11 +230,7 @@ __global__ void prep_gather_kernel(const double* __restrict__ xyz, uint32_t n,
     const double x = xyz[3ull * s], y = xyz[3ull * s + 1], z = xyz[3ull * s + 2];
     const float fx = __double2float_rn(x), fy = __double2float_rn(y), fz = __double2float_rn(z);
     out64[q] = Point64{x, y, z, 0.0};
-    out32[q] = make_float4(fx, fy, fz, 0.f);
-    out_soa[q] = fx;
-    out_soa[(size_t)n_pad + q] = fy;
-    out_soa[2ull * n_pad + q] = fz;
-    if (op_a) put_operands(op_a, op_b, q, fx, fy, fz);
+    put_block(blk, q, fx, fy, fz, !euclid);
 }
 
 // Padding of 3-D catalogs: (+inf, +inf, +inf).  A pair with a real point has
@@ -250,15 +239,12 @@ __global__ void prep_gather_kernel(const double* __restrict__ xyz, uint32_t n,
 // cannot settle them (coordinates so large that the FP32 bounds overflow) the
 // binary64 recheck maps the NaN distance to overflow, so padding is never
 // counted (unit-vector catalogs are padded with zero vectors instead).
-__global__ void prep_fill_kernel(Point64* out64, float4* out32, float* out_soa, uint32_t n_pad, double v) {
+__global__ void prep_fill_kernel(Point64* out64, unsigned char* blk, uint32_t n_pad, double v) {
     const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n_pad) return;
     const float f = (float)v;
     out64[p] = Point64{v, v, v, 0.0};
-    out32[p] = make_float4(f, f, f, 0.f);
-    out_soa[p] = f;
-    out_soa[(size_t)n_pad + p] = f;
-    out_soa[2ull * n_pad + p] = f;
+    put_block(blk, p, f, f, f, false);
 }
 
 // Bounding sphere of each kCapPoints-point group of a prepared catalog (one
@@ -347,8 +333,8 @@ __global__ void prep_caps2_kernel(const float4* __restrict__ caps, uint32_t n_bl
 
 cudaError_t launch_prepare(const double* xyz_in, uint32_t n, const uint32_t* seg_of_point,
                            const uint32_t* seg_delta, int sort, int euclid, unsigned long long* bbox,
-                           Point64* out64, float4* out32, float* out_soa, unsigned char* op_a, unsigned char* op_b,
-                           float4* caps, float4* caps2, uint32_t n_pad, unsigned long long* keys, uint32_t* vals, uint32_t n_pow2,
+                           Point64* out64, unsigned char* blk, float4* caps, float4* caps2, uint32_t n_pad,
+                           unsigned long long* keys, uint32_t* vals, uint32_t n_pow2,
                            unsigned long long* err_word, unsigned long long* eps_word, cudaStream_t stream,
                            uint32_t* launches) {
     cudaError_t e;
@@ -384,21 +370,17 @@ cudaError_t launch_prepare(const double* xyz_in, uint32_t n, const uint32_t* seg
         }
     }
     if (n_pad > 0 && euclid) {
-        prep_fill_kernel<<<(n_pad + 255) / 256, 256, 0, stream>>>(out64, out32, out_soa, n_pad, (double)INFINITY);
+        prep_fill_kernel<<<(n_pad + 255) / 256, 256, 0, stream>>>(out64, blk, n_pad, (double)INFINITY);
         ++nl;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     } else if (n_pad > 0) {
         if ((e = cudaMemsetAsync(out64, 0, (size_t)n_pad * sizeof(Point64), stream)) != cudaSuccess ||
-            (e = cudaMemsetAsync(out32, 0, (size_t)n_pad * sizeof(float4), stream)) != cudaSuccess ||
-            (e = cudaMemsetAsync(out_soa, 0, (size_t)n_pad * 3 * sizeof(float), stream)) != cudaSuccess)
-            return e;
-        if (op_a && ((e = cudaMemsetAsync(op_a, 0, (size_t)(n_pad / kOpBlock) * kOpABlock, stream)) != cudaSuccess ||
-                     (e = cudaMemsetAsync(op_b, 0, (size_t)(n_pad / kOpBlock) * kOpBBlock, stream)) != cudaSuccess))
+            (e = cudaMemsetAsync(blk, 0, (size_t)(n_pad / kBlk) * kBlkBytes, stream)) != cudaSuccess)
             return e;
     }
     if (n > 0) {
         prep_gather_kernel<<<(n + 255) / 256, 256, 0, stream>>>(xyz_in, n, do_sort ? vals : nullptr, seg_of_point,
-                                                               seg_delta, out64, out32, out_soa, op_a, op_b, n_pad);
+                                                               seg_delta, out64, blk, euclid);
         ++nl;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }

@@ -662,8 +662,7 @@ extern "C" int tpcf_bins_destroy(tpcf_bins* b) { return bins_destroy_impl(b); }
 // ====================================================================== catalogs
 size_t tpcf::catalog_bytes(uint64_t n) {
     const uint64_t n_pad = ((n + kPad - 1) / kPad + 1) * kPad;
-    return (size_t)n_pad * (sizeof(Point64) + sizeof(float4) + 3 * sizeof(float)) +
-           (size_t)(n_pad / kOpBlock) * (kOpABlock + kOpBBlock);
+    return (size_t)n_pad * sizeof(Point64) + (size_t)(n_pad / kBlk) * kBlkBytes;
 }
 
 int tpcf::catalog_create_impl(tpcf_ctx* ctx, const double* xyz, uint64_t n, int where, const uint64_t* offsets,
@@ -733,13 +732,13 @@ int tpcf::catalog_create_impl(tpcf_ctx* ctx, const double* xyz, uint64_t n, int 
     auto alloc = [&](void** p, size_t bytes) {
         return stream_ordered ? dev_malloc_async(p, bytes, st) : dev_malloc(p, bytes);
     };
-    if (alloc((void**)&c->d64, (size_t)c->n_pad * sizeof(Point64)) != cudaSuccess ||
-        alloc((void**)&c->d32, (size_t)c->n_pad * sizeof(float4)) != cudaSuccess ||
-        alloc((void**)&c->soa, (size_t)c->n_pad * 3 * sizeof(float)) != cudaSuccess ||
-        alloc((void**)&c->caps, (size_t)(c->n_pad / kCapPoints + c->n_pad / kPad) * sizeof(float4)) != cudaSuccess ||
-        (!euclid && (alloc((void**)&c->op_a, (size_t)(c->n_pad / kOpBlock) * kOpABlock) != cudaSuccess ||
-                     alloc((void**)&c->op_b, (size_t)(c->n_pad / kOpBlock) * kOpBBlock) != cudaSuccess)))
+    // one allocation: binary64 points, blocks, spheres
+    const size_t b64 = (size_t)c->n_pad * sizeof(Point64), bblk = (size_t)(c->n_pad / kBlk) * kBlkBytes;
+    if (alloc((void**)&c->d64, b64 + bblk + (size_t)(c->n_pad / kCapPoints + c->n_pad / kPad) * sizeof(float4)) !=
+        cudaSuccess)
         return fail_with(TPCF_ENOMEM, "device allocation failed");
+    c->blk = (unsigned char*)c->d64 + b64;
+    c->caps = (float4*)(c->blk + bblk);
     c->caps2 = c->caps + c->n_pad / kCapPoints;
     const double* in = xyz;
     if (n > 0 && where == TPCF_HOST) {
@@ -781,7 +780,7 @@ int tpcf::catalog_create_impl(tpcf_ctx* ctx, const double* xyz, uint64_t n, int 
     }
     uint32_t nl = 0;
     cudaError_t e = launch_prepare(in, (uint32_t)n, seg, seg_delta, sort ? 1 : 0, euclid ? 1 : 0, err + 2, c->d64,
-                                   c->d32, c->soa, c->op_a, c->op_b, c->caps, c->caps2, c->n_pad, keys, vals, n_pow2, err, err + 1, st, &nl);
+                                   c->blk, c->caps, c->caps2, c->n_pad, keys, vals, n_pow2, err, err + 1, st, &nl);
     ctx->launches.fetch_add(nl);
     if (e != cudaSuccess) return fail_with(TPCF_ECUDA, cudaGetErrorString(e));
     unsigned long long hw[2] = {0, 0};
@@ -827,7 +826,7 @@ extern "C" int tpcf_catalog_create_3d(tpcf_ctx* ctx, const double* xyz, uint64_t
 int tpcf::catalog_destroy_impl(tpcf_catalog* c) {
     if (!c) return TPCF_EINVAL;
     cudaSetDevice(c->ctx->cfg.device);
-    void* bufs[7] = {c->d64, c->d32, c->soa, c->seg_of_block, c->caps, c->op_a, c->op_b};
+    void* bufs[2] = {c->d64, c->seg_of_block};
     if (c->stream_ordered) {
         for (void* p : bufs)
             if (p) cudaFreeAsync(p, c->free_stream);
@@ -907,11 +906,11 @@ bool tc_shape_for(tpcf_ctx* ctx, int nedges, uint64_t total_pairs, Shape* sh) {
     int S = 8;
     while (S >= 4 && count_tc_smem_bytes(S, nedges) > ctx->smem_optin) S -= 2;
     if (S < 4) return false;
-    int Jc = 32 * (int)kOpBlock;
-    while (Jc > (int)kOpBlock && total_pairs / (512ull * (uint64_t)Jc) < kTcItemsPerSm * (uint64_t)ctx->num_sms) Jc /= 2;
+    int Jc = 32 * (int)kBlk;
+    while (Jc > (int)kBlk && total_pairs / (512ull * (uint64_t)Jc) < kTcItemsPerSm * (uint64_t)ctx->num_sms) Jc /= 2;
     sh->threads = 512;
     sh->ipt = 16;
-    sh->jtile = (int)kOpBlock;
+    sh->jtile = (int)kBlk;
     sh->jchunk = Jc;
     sh->stages = S;
     sh->blocks = ctx->num_sms;
@@ -969,17 +968,13 @@ uint64_t build_work(tpcf_ctx* ctx, const SubSpec* specs, int nsub, const BinsDev
         const SubSpec& p = specs[s];
         SubProblem& sp = subs[s];
         memset(&sp, 0, sizeof sp);
-        sp.a32 = p.a->d32 + p.a_off;
-        sp.b32 = p.b->d32 + p.b_off;
-        sp.b_soa = p.b->soa + p.b_off;
-        sp.b_soa_stride = p.b->n_pad;
+        sp.a_blk = p.a->blk + (size_t)(p.a_off / kBlk) * kBlkBytes;  // sub-ranges start on kSegAlign boundaries
+        sp.b_blk = p.b->blk + (size_t)(p.b_off / kBlk) * kBlkBytes;
         sp.a64 = p.a->d64 + p.a_off;
         sp.b64 = p.b->d64 + p.b_off;
         sp.a_caps = p.a->caps + p.a_off / kCapPoints;  // sub-ranges start on kSegAlign boundaries
         sp.b_caps = p.b->caps + p.b_off / kCapPoints;
         sp.b_caps2 = p.b_off % kPad == 0 ? p.b->caps2 + p.b_off / kPad : nullptr;
-        sp.a_op = p.a->op_a ? p.a->op_a + (size_t)(p.a_off / kOpBlock) * kOpABlock : nullptr;
-        sp.b_op = p.b->op_b ? p.b->op_b + (size_t)(p.b_off / kOpBlock) * kOpBBlock : nullptr;
         sp.na = p.na;
         sp.nb = p.nb;
         sp.n_iblk = (p.na + I - 1) / I;

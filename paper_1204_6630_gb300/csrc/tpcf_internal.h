@@ -18,15 +18,13 @@ constexpr uint32_t kSegAlign = 256;
 // Bounding spheres for spatial pruning: one per kCapPoints consecutive
 // points of a catalog's device layout.
 constexpr uint32_t kCapPoints = 128;
-// Operands of the tensor-core screen (count_tc.cu), in blocks of kOpBlock
-// points.  A point's binary16 split x = x1 + x2 (likewise y, z) gives the
-// 16-byte records X = (x1, y1, z1, x2, y2, z2, 0, 0) and Y = (x2, y2, z2, x1,
-// y1, z1, 0, 0).  i-side block: plane X, plane X (2 x 2048 bytes); j-side
-// block: plane X, plane Y, then the FP32 coordinates x | y | z (3 x 512 bytes).
-constexpr uint32_t kOpBlock = 128;
-constexpr uint32_t kOpABlock = 2 * kOpBlock * 16;
-constexpr uint32_t kOpBCoord = 2 * kOpBlock * 16;
-constexpr uint32_t kOpBBlock = kOpBCoord + kOpBlock * 12;
+// A catalog's FP32 points and tensor-core operands, in blocks of kBlk points:
+// plane X (16 bytes a point), then the FP32 coordinates as x | y | z arrays.
+// X = (x1, y1, z1, x2, y2, z2, 0, 0) is the binary16 split x = x1 + x2
+// (likewise y, z); zero in 3-D catalogs.
+constexpr uint32_t kBlk = 128;
+constexpr uint32_t kBlkX = kBlk * 16;
+constexpr uint32_t kBlkBytes = kBlkX + kBlk * 12;
 // Bound on the distance of the tensor-core screen value from the binary64 dot
 // product (44u, derived in count_tc.cu) with a margin.
 constexpr double kTcGuard = 64.0 * 5.9604644775390625e-08;
@@ -78,10 +76,8 @@ struct BinsDev {
 // cross count A x B (all pairs).  Work is cut into items: (i-block of I points)
 // x (j-chunk of Jc points); an item is processed in j-tiles of J points.
 struct SubProblem {
-    const float4* a32;    // FP32 screen copy of A (padded to kPad)
-    const float4* b32;
-    const float* b_soa;   // B's FP32 points as x | y | z arrays (the sub-range's first point)
-    uint32_t b_soa_stride;  // floats between B's x, y and z arrays (its padded size)
+    const unsigned char* a_blk;  // FP32 points and operands of A and B in blocks (see kBlk), the
+    const unsigned char* b_blk;  // sub-range's first block (catalogs are padded to kPad points)
     const Point64* a64;   // binary64 copy of A (padded)
     const Point64* b64;
     uint32_t na, nb;      // real point counts
@@ -105,10 +101,7 @@ struct SubProblem {
     // starting at the sub-range's first point (spatial pruning).
     const float4* a_caps;
     const float4* b_caps;
-    // Tensor-core kernel: operands of A (i-side) and B (j-side), the sub-range's first block.
-    const float4* b_caps2;       // spheres of B's kPad-point blocks; NULL: the sub-range does not start on one
-    const unsigned char* a_op;
-    const unsigned char* b_op;
+    const float4* b_caps2;  // spheres of B's kPad-point blocks; NULL: the sub-range does not start on one
 };
 
 constexpr int kMaxInlineSub = 3;
@@ -213,7 +206,7 @@ cudaError_t launch_count_step(const WorkDesc& wd, const Shape& sh, cudaStream_t 
 // one-job kernel with preemptible draws (wd.pos_lo, stats[kStatYield]).
 cudaError_t launch_count_preemptible(const WorkDesc& wd, const Shape& sh, cudaStream_t stream);
 // The tensor-core counting kernel (count_tc.cu; FP32 screen of angles): items
-// of 512 i-points x Jc j-points in tiles of kOpBlock; preempt: draws from
+// of 512 i-points x Jc j-points in tiles of kBlk; preempt: draws from
 // wd.pos_lo on, stopping at the yield word.
 cudaError_t launch_count_tc(const WorkDesc& wd, const Shape& sh, bool preempt, cudaStream_t stream);
 size_t count_tc_smem_bytes(int stages, int nedges);
@@ -228,8 +221,7 @@ cudaError_t launch_finalize_batch(const unsigned long long* acc, int acc_stride,
                                   int count, int count_over, unsigned long long* err_word, cudaStream_t stream);
 cudaError_t launch_prepare(const double* xyz_in, uint32_t n, const uint32_t* seg_of_point,
                            const uint32_t* seg_delta, int sort, int euclid, unsigned long long* bbox,
-                           Point64* out64, float4* out32, float* out_soa, unsigned char* op_a, unsigned char* op_b,
-                           float4* caps, float4* caps2, uint32_t n_pad,
+                           Point64* out64, unsigned char* blk, float4* caps, float4* caps2, uint32_t n_pad,
                            unsigned long long* key_scratch, uint32_t* val_scratch,
                            uint32_t n_pow2, unsigned long long* err_word, unsigned long long* eps_word,
                            cudaStream_t stream, uint32_t* launches);
