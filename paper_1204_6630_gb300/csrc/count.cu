@@ -29,8 +29,8 @@
 namespace tpcf {
 
 // ============================================================== shared-memory layout
-// Block-wide control words (int32): the abort flag and each warp's queue length.
-enum Ctl { kCtlAbort = 0, kCtlChunk = 1, kCtlQueue = 8, kCtlWords = 48 };
+// Block-wide control words (int32): the abort flag.
+enum Ctl { kCtlAbort = 0, kCtlWords = 32 };
 
 // Per-warp queue of unsettled pairs of the current tile (32-bit codes): at most
 // 31 left from earlier groups plus one per lane and round.
@@ -59,8 +59,6 @@ struct SmemLayout {
     uint32_t lut;       // kLutCells 16-bit entries (screen kernels)
     uint32_t queue;     // W * kUQueue unsettled-pair codes (uint32, screen kernels)
     uint32_t icap;      // W pruning slots: the warp's i-sphere, B's sphere array, pruned pair slots
-    uint32_t bwd;       // serving steps: the block's current job (WorkDesc) and its item counter
-    uint32_t counter;
     uint32_t total;
 };
 
@@ -93,10 +91,6 @@ __host__ __device__ inline SmemLayout smem_layout(int mode, int T, int J, int S,
     L.queue = off; off += plain ? 0u : W * kUQueue * 4;
     off = align_up(off, 16);
     L.icap = off; off += W * kPruneSlotBytes;
-    off = align_up(off, 16);
-    L.bwd = off; off += (uint32_t)sizeof(WorkDesc);
-    off = align_up(off, 8);
-    L.counter = off; off += 8;
     L.total = off;
     return L;
 }
@@ -546,15 +540,7 @@ __device__ __forceinline__ bool prune_chunk(const WorkDesc& wd, uint32_t jg0, ui
 // waits for another.  Every wait is bounded; a timeout sets the block's abort
 // word and the call's error word, after which no copy is issued, warps leave
 // their loops and each waits (bounded) for its own copies in flight.
-//
-// MULTI (serving): the launch is one step of the job server, a list of slices
-// of many jobs' item ranges (each job with its own catalogs, bins and
-// histograms).  Every block walks the slices in order, copying a slice's job
-// description into shared memory; its warps draw the slice's items from the
-// slice's counter, shared by all blocks.  When a block moves to another job,
-// its warps merge their counters into the previous job's histograms and the
-// block loads the new job's bins and LUT.
-template <int T, int R, int MODE, bool MULTI, bool PREEMPT>
+template <int T, int R, int MODE, bool PREEMPT>
 __global__ void __launch_bounds__(T, 1) count_kernel(const __grid_constant__ WorkDesc wd) {
     constexpr bool PLAIN = MODE == kModePlain;
     constexpr bool EUCLID = MODE == kModeEuclid;
@@ -573,7 +559,7 @@ __global__ void __launch_bounds__(T, 1) count_kernel(const __grid_constant__ Wor
         uint32_t* hist = sptr<uint32_t>(wd.off_hist);
         for (int k = tid; k < (wd.nedges_max + 1) * (T / 2); k += T) hist[k] = 0;
     }
-    if constexpr (!MULTI) load_bins<T>(sub_of(wd, 0).bins, wd, PLAIN);
+    load_bins<T>(sub_of(wd, 0).bins, wd, PLAIN);
     // the warp's S barriers, stage records and stages (recomputed where used: no registers held)
 #define TPCF_BARS (sptr<uint64_t>(wd.off_bars) + (uint32_t)warp * S)
 #define TPCF_META (sptr<TileMeta>(wd.off_meta) + (uint32_t)warp * S)
@@ -586,11 +572,11 @@ __global__ void __launch_bounds__(T, 1) count_kernel(const __grid_constant__ Wor
     const HistCol hc = hist_col<T>(wd);
 
     // Lane 0 copies the tile at cursor p into stage seq % S and records it there.
-    auto issue = [&](const WorkDesc& wdi, uint32_t seq, const Cursor& p) {
+    auto issue = [&](uint32_t seq, const Cursor& p) {
         if (lane != 0) return;
         if ((wd.flags & TPCF_F_TEST_WAIT_TIMEOUT) && seq == 0) return;  // test hook: never issued
         const uint32_t s = seq % S;
-        const SubProblem& sp = sub_of(wdi, p.sub);
+        const SubProblem& sp = sub_of(wd, p.sub);
         const uint32_t jbase = p.g.j0 + p.t * wd.J;
         TPCF_META[s] = TileMeta{p.q, p.t | ((uint32_t)p.sub << 16), p.g.i0, p.g.j0};
         unsigned char* dst = sptr<unsigned char>(TPCF_STAGE_BASE + s * wd.stage_bytes);
@@ -607,7 +593,7 @@ __global__ void __launch_bounds__(T, 1) count_kernel(const __grid_constant__ Wor
         }
     };
 
-    // ---- the warp's state (kept across the pieces of a multi-job launch)
+    // ---- the warp's state
     uint32_t seq = 0, issued = 0;  // tiles consumed / issued so far (tile k: stage k % S)
     int cur_sub = -1;
     uint32_t cur_q = 0xffffffffu;
@@ -620,18 +606,13 @@ __global__ void __launch_bounds__(T, 1) count_kernel(const __grid_constant__ Wor
     uint32_t band_cnt = 0, mism_cnt = 0;  // pairs rechecked in binary64 / whose FP32-only bin differed
     bool aborted = false;
 
-    // The warp's loop over the items of work description wd (this parameter
-    // shadows the launch's: it is the launch's own or a job's copy in shared
-    // memory): the first S tiles, then each tile in turn, its stage refilled with
-    // the tile S ahead; returns with every issued tile consumed (or after an abort).
-    auto run_items = [&](const WorkDesc& wd) {
-    if (aborted || ctl[kCtlAbort]) return;
-    // (single launches draw from the launch's statistics word: no pointer held in registers)
+    // ---- the warp's loop over its items: the first S tiles, then each tile in
+    // turn, its stage refilled with the tile S ahead
     Cursor prod;
-    draw_next<PREEMPT>(wd, prod, MULTI ? wd.item_counter : wd.stats + kStatNextItem);
+    draw_next<PREEMPT>(wd, prod, wd.stats + kStatNextItem);
     for (; issued < seq + S && prod.valid; ++issued) {
-        issue(wd, issued, prod);
-        advance<PREEMPT>(wd, prod, MULTI ? wd.item_counter : wd.stats + kStatNextItem);
+        issue(issued, prod);
+        advance<PREEMPT>(wd, prod, wd.stats + kStatNextItem);
     }
     for (; seq < issued; ++seq) {
         // ---- wait for tile seq
@@ -851,87 +832,14 @@ __global__ void __launch_bounds__(T, 1) count_kernel(const __grid_constant__ Wor
         // ---- refill this stage with tile seq + S
         __syncwarp();
         if (prod.valid && !ctl[kCtlAbort]) {
-            issue(wd, seq + S, prod);
+            issue(seq + S, prod);
             ++issued;
-            advance<PREEMPT>(wd, prod, MULTI ? wd.item_counter : wd.stats + kStatNextItem);
+            advance<PREEMPT>(wd, prod, wd.stats + kStatNextItem);
         }
     }
-    };
-
-    if constexpr (!MULTI) {
-        run_items(wd);
-    } else {
-        // ---- serving step: every block walks the step's slices in order; its warps
-        // draw the items of a slice from the slice's counter (shared by all blocks)
-        // until it is exhausted, so a block waits for its own warps only where it
-        // leaves a slice.  Slices that other blocks have already drained are
-        // skipped; the job's bins and LUT are loaded when the block changes job.
-        WorkDesc& bw = *sptr<WorkDesc>(wd.off_bwd);  // the block's current job
-        volatile uint32_t* take_word = sptr<volatile uint32_t>(wd.off_ctl) + kCtlChunk;
-        const WorkDesc* cur_job = nullptr;  // block-uniform
-        for (int si = 0; si < wd.nslices; ++si) {
-            const StepSlice sl = wd.slices[si];
-            const uint32_t n = sl.pos_end - sl.pos_begin;
-            __syncthreads();
-            if (tid == 0)
-                *take_word = (ctl[kCtlAbort] == 0 &&
-                              *reinterpret_cast<volatile unsigned long long*>(wd.slice_ctr + si) < n) ? 1u : 0u;
-            __syncthreads();
-            if (!*take_word) continue;  // block-uniform
-            if (sl.job != cur_job) {
-                // merge the counters into the previous job's histograms (its row count)
-                if (cur_sub >= 0) {
-                    warp_flush_hist<T>(hc, bw.ne, check, cur_hist);
-                    cur_sub = -1;
-                    cur_hist = nullptr;
-                    inc_bound = 0;
-                    cur_q = 0xffffffffu;
-                }
-                __syncthreads();
-                // the job's description, with this launch's layout, counters and limits
-                {
-                    const uint32_t* src = reinterpret_cast<const uint32_t*>(sl.job);
-                    uint32_t* dst = reinterpret_cast<uint32_t*>(&bw);
-                    for (int k = tid; k < (int)(sizeof(WorkDesc) / 4); k += T) dst[k] = src[k];
-                }
-                __syncthreads();
-                if (tid == 0) {
-                    bw.stats = wd.stats;
-                    bw.flags = wd.flags;
-                    bw.wait_limit_ns = wd.wait_limit_ns;
-                    bw.stages = wd.stages;
-                    bw.I = wd.I;
-                    bw.J = wd.J;
-                    bw.Jc = wd.Jc;
-                    bw.nedges_max = wd.nedges_max;
-                    bw.stage_bytes = wd.stage_bytes;
-                    bw.flush_limit = wd.flush_limit;
-                    bw.off_ctl = wd.off_ctl; bw.off_bars = wd.off_bars; bw.off_meta = wd.off_meta;
-                    bw.off_stage = wd.off_stage; bw.off_hist = wd.off_hist; bw.off_cthr = wd.off_cthr;
-                    bw.off_lo = wd.off_lo; bw.off_hi = wd.off_hi; bw.off_c32 = wd.off_c32; bw.off_zlo = wd.off_zlo;
-                    bw.off_zhi = wd.off_zhi; bw.off_lut = wd.off_lut; bw.off_queue = wd.off_queue;
-                    bw.off_icap = wd.off_icap; bw.off_bwd = wd.off_bwd; bw.off_counter = wd.off_counter;
-                }
-                __syncthreads();
-                load_bins<T>(sub_of(bw, 0).bins, bw, PLAIN);
-                cur_job = sl.job;
-            }
-            if (tid == 0) {
-                bw.item_lo = sl.q_begin;
-                bw.item_hi = (uint64_t)sl.q_begin + n;
-                bw.item_counter = wd.slice_ctr + si;
-                bw.pos_lo = 0;
-                bw.draw_warps = gridDim.x * (uint32_t)W;
-            }
-            __syncthreads();
-            run_items(bw);
-        }
-    }
-
     // ---- merge this warp's columns (skipped after an abort: outputs are invalid)
     if (!aborted && cur_sub >= 0) {
-        if constexpr (MULTI) warp_flush_hist<T>(hc, sptr<WorkDesc>(wd.off_bwd)->ne, check, cur_hist);
-        else warp_flush_hist<T>(hc, wd.ne, check, cur_hist);
+        warp_flush_hist<T>(hc, wd.ne, check, cur_hist);
     }
     if constexpr (!PLAIN) {
         const unsigned long long b = warp_sum(band_cnt), mm = warp_sum(mism_cnt);
@@ -1025,7 +933,7 @@ cudaError_t launch_finalize(unsigned long long* acc, int nedges, unsigned long l
 // ============================================================== launchers
 // Fills the block constants of the work description (shared-memory offsets of
 // the shape, merge interval) and launches.
-template <int T, int R, int MODE, bool MULTI = false, bool PREEMPT = false>
+template <int T, int R, int MODE, bool PREEMPT = false>
 static cudaError_t launch_t(const WorkDesc& wd_in, const Shape& sh, cudaStream_t stream) {
     WorkDesc wd = wd_in;
     const SmemLayout L = smem_layout(MODE, T, (int)wd.J, (int)wd.stages, wd.nedges_max);
@@ -1043,8 +951,6 @@ static cudaError_t launch_t(const WorkDesc& wd_in, const Shape& sh, cudaStream_t
     wd.off_lut = L.lut;
     wd.off_queue = L.queue;
     wd.off_icap = L.icap;
-    wd.off_bwd = L.bwd;
-    wd.off_counter = L.counter;
     wd.stage_bytes = wd.J * staged_point_bytes(MODE);
     // the 16-bit counters' merge interval is bounded in the kernel, per tile
     wd.flush_limit = 0xffffu;
@@ -1052,40 +958,33 @@ static cudaError_t launch_t(const WorkDesc& wd_in, const Shape& sh, cudaStream_t
     // the draw order is laid out for this launch's warps unless the caller fixed it
     // (continuations of a preempted launch keep the order of the first)
     if (wd.draw_warps == 0) wd.draw_warps = (uint32_t)sh.blocks * (uint32_t)(T / 32);
-    count_kernel<T, R, MODE, MULTI, PREEMPT><<<sh.blocks, T, sh.smem, stream>>>(wd);
+    count_kernel<T, R, MODE, PREEMPT><<<sh.blocks, T, sh.smem, stream>>>(wd);
     return cudaGetLastError();
 }
 
 // The limit is raised to the device's opt-in maximum rather than to `bytes`:
 // the attribute belongs to the kernel, not to a launch, so a smaller value set
 // by one host thread could otherwise undercut a concurrent launch of another.
-template <int T, int R, int MODE, bool MULTI = false, bool PREEMPT = false>
+template <int T, int R, int MODE, bool PREEMPT = false>
 static cudaError_t set_smem_t(size_t bytes) {
     int dev = 0, optin = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return e;
     if (bytes > (size_t)optin) return cudaErrorInvalidValue;
-    return cudaFuncSetAttribute(count_kernel<T, R, MODE, MULTI, PREEMPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    return cudaFuncSetAttribute(count_kernel<T, R, MODE, PREEMPT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 optin);
 }
 
-cudaError_t launch_count_step(const WorkDesc& wd, const Shape& sh, cudaStream_t stream) {
+// The job server's jobs whose histograms do not fit the tensor-core kernel: the 512 x 8 screen kernel with preemptible
+// draws (a start position and the yield word).
+cudaError_t launch_count_preemptible(const WorkDesc& wd, const Shape& sh, cudaStream_t stream) {
     if (sh.threads != 512 || sh.ipt != 8) return cudaErrorInvalidConfiguration;
     return launch_t<512, 8, kModeScreen, true>(wd, sh, stream);
 }
 
-cudaError_t count_step_set_smem_limit(size_t bytes) { return set_smem_t<512, 8, kModeScreen, true>(bytes); }
-
-// The job server's one-job steps: the 512 x 8 screen kernel with preemptible
-// draws (a start position and the yield word).
-cudaError_t launch_count_preemptible(const WorkDesc& wd, const Shape& sh, cudaStream_t stream) {
-    if (sh.threads != 512 || sh.ipt != 8) return cudaErrorInvalidConfiguration;
-    return launch_t<512, 8, kModeScreen, false, true>(wd, sh, stream);
-}
-
 cudaError_t count_preemptible_set_smem_limit(size_t bytes) {
-    return set_smem_t<512, 8, kModeScreen, false, true>(bytes);
+    return set_smem_t<512, 8, kModeScreen, true>(bytes);
 }
 
 #define TPCF_SHAPES(X) X(128, 8) X(256, 8) X(512, 8) X(256, 16)

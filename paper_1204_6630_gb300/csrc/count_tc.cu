@@ -75,7 +75,7 @@ enum : uint32_t {
 __host__ __device__ constexpr uint32_t tc_bar_words(uint32_t S) { return 2 * S + 4 + 2 * kGroups; }
 
 struct TcLayout {
-    uint32_t ctl, bars, meta, atile, stage, hist, cos_thr, lo, hi, cos32, zlo, zhi, lut, queue, bwd, total;
+    uint32_t ctl, bars, meta, atile, stage, hist, cos_thr, lo, hi, cos32, zlo, zhi, lut, queue, total;
 };
 
 __host__ __device__ inline TcLayout tc_layout(int S, int nedges) {
@@ -101,7 +101,6 @@ __host__ __device__ inline TcLayout tc_layout(int S, int nedges) {
     off = align_up(off, 16);
     L.queue = off; off += (uint32_t)kWorkWarps * kQueueCodes * 4;
     off = align_up(off, 16);
-    L.bwd = off; off += (uint32_t)sizeof(WorkDesc);
     L.total = align_up(off, 16);
     return L;
 }
@@ -750,7 +749,6 @@ cudaError_t launch_tc_t(const WorkDesc& wd_in, const Shape& sh, cudaStream_t str
     wd.off_zhi = L.zhi;
     wd.off_lut = L.lut;
     wd.off_queue = L.queue;
-    wd.off_bwd = L.bwd;
     wd.stage_bytes = kStageBytes;
     if (L.total > sh.smem || wd.I != 128u * kGroups || wd.J != kBlk || wd.Jc > 32u * kBlk)
         return cudaErrorInvalidValue;

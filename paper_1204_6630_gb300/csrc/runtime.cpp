@@ -919,6 +919,13 @@ bool tc_shape_for(tpcf_ctx* ctx, int nedges, uint64_t total_pairs, Shape* sh) {
     return true;
 }
 
+// Items per draw of the tensor-core kernel: one, unless most are pruned away
+// (then up to 32, as long as every SM still draws some 16 times).
+uint32_t tc_draw_batch(tpcf_ctx* ctx, bool prune, uint64_t items) {
+    if (!prune) return 1u;
+    return (uint32_t)std::min<uint64_t>(32, std::max<uint64_t>(1, items / (16ull * (uint64_t)ctx->num_sms)));
+}
+
 // Default shape: 512 x 8 for large problems, smaller i-blocks when the
 // catalogs (or sub-ranges) are small or the per-thread histograms do not fit.
 bool choose_shape(tpcf_ctx* ctx, int mode, int nedges, uint64_t total_pairs, uint64_t max_n, Shape* sh) {
@@ -1202,14 +1209,8 @@ int run_counts(tpcf_ctx* ctx, const SubSpec* specs, int nsub, const tpcf_bins* b
             wd.item_hi = items * (ctx->cfg.shard_index + 1) / ctx->cfg.shard_count;
         }
         wd.stats = stat_w;
-        wd.item_counter = stat_w + kStatNextItem;
         fill_scalars(ctx, specs, nsub, bh, mode, shp, force_idx, ne, wd);
-        // items per draw: one, unless most are pruned away (then up to 32, as long as
-        // every SM still draws some 16 times)
-        wd.draw_batch = 1;
-        if (wd.prune)
-            wd.draw_batch = (uint32_t)std::min<uint64_t>(
-                32, std::max<uint64_t>(1, (wd.item_hi - wd.item_lo) / (16ull * (uint64_t)ctx->num_sms)));
+        wd.draw_batch = tc_draw_batch(ctx, wd.prune != 0, wd.item_hi - wd.item_lo);
         return TPCF_OK;
     };
     auto smem_limit = [&](const Shape& shp) {
@@ -1393,14 +1394,14 @@ int run_counts(tpcf_ctx* ctx, const SubSpec* specs, int nsub, const tpcf_bins* b
 }  // namespace
 
 // ====================================================================== serving steps
-// Shape of a serving step (the multi-job kernel exists for 512 x 8): j-tiles of
-// 256 points, or 128 where the step's histograms need the shared memory;
-// false when neither fits.
-bool tpcf::serving_shape(tpcf_ctx* ctx, int nedges_max, Shape* sh) {
-    return shape_for(ctx, kModeScreenScalar, nedges_max, 512, 8, 0, 2, sh);
+// Shape of a served job: the tensor-core kernel's, or (histograms too large for
+// it) the FP32 kernel's 512 x 8; false when neither fits.
+bool tpcf::serving_shape(tpcf_ctx* ctx, int nedges, uint64_t pairs, Shape* sh) {
+    if (kernel_mode(ctx->cfg, false) == kModeScreenScalar && tc_shape_for(ctx, nedges, pairs, sh)) return true;
+    return shape_for(ctx, kModeScreenScalar, nedges, 512, 8, 0, 2, sh);
 }
 
-// Work description of one served job for the serving-step kernel: the
+// Work description of one served job: the
 // sub-problems RR, DR and DD of catalogs (d, r) with bins b, accumulating
 // into three histograms of ne + 1 words at acc (in that order); also the
 // job's item count and the three histograms' pair totals.
@@ -1428,43 +1429,12 @@ int tpcf::serving_job_desc(tpcf_ctx* ctx, const tpcf_catalog* d, const tpcf_cata
     return TPCF_OK;
 }
 
-// One serving step: slices (device, sorted by position) of `positions` work
-// items in all, into the jobs' own accumulators; slice_ctr: one device counter
-// per slice and stats: kStatWords device words, all zeroed by the caller.
-int tpcf::serving_launch(tpcf_ctx* ctx, const Shape& sh, int nedges_max, const StepSlice* slices, int nslices,
-                         unsigned long long* slice_ctr, uint32_t positions, unsigned long long* stats,
-                         cudaStream_t st) {
-    WorkDesc wd;
-    memset(&wd, 0, sizeof wd);
-    wd.stats = stats;
-    wd.item_counter = stats + kStatNextItem;
-    wd.slices = slices;
-    wd.slice_ctr = slice_ctr;
-    wd.nslices = nslices;
-    wd.step_positions = positions;
-    wd.I = 32u * (uint32_t)sh.ipt;
-    wd.J = (uint32_t)sh.jtile;
-    wd.Jc = (uint32_t)sh.jchunk;
-    wd.stages = (uint32_t)sh.stages;
-    wd.flags = ctx->cfg.flags;
-    wd.nedges_max = nedges_max;
-    wd.wait_limit_ns = (uint64_t)ctx->cfg.wait_timeout_us * 1000ull;
-    Shape s2 = sh;  // (no more blocks than the step has items for their warps)
-    const uint64_t warps = (uint64_t)sh.threads / 32;
-    const uint64_t need = ((uint64_t)positions + warps - 1) / warps;
-    if ((uint64_t)s2.blocks > need) s2.blocks = (int)std::max<uint64_t>(1, need);
-    if (count_step_set_smem_limit(sh.smem) != cudaSuccess) return TPCF_ECUDA;
-    if (launch_count_step(wd, s2, st) != cudaSuccess) return TPCF_ECUDA;
-    ctx->launches.fetch_add(1);
-    return TPCF_OK;
-}
-
-// One serving step that holds a single job (job: its work description from
-// serving_job_desc): the one-job kernel, which reads the description from its
-// parameter, over the items [q_begin, q_begin + n), drawing their order's
-// positions from pos_lo on (the order laid out for draw_warps warps; 0: this
-// launch's) until it ends or stats[kStatYield] is set; stats: kStatWords
-// device words zeroed by the caller (its item counter included).
+// Counts a served job's items [q_begin, q_begin + n) (job: its work description
+// from serving_job_desc for shape sh): one launch, which draws the items'
+// order from position pos_lo on (FP32 kernel: the order laid out for
+// draw_warps warps; 0: this launch's) until it ends or stats[kStatYield] is
+// set; stats: kStatWords device words zeroed by the caller (its item counter
+// included).
 int tpcf::serving_launch_one(tpcf_ctx* ctx, const Shape& sh, const WorkDesc& job, uint32_t q_begin, uint32_t n,
                              uint64_t pos_lo, uint32_t draw_warps, unsigned long long* stats, cudaStream_t st) {
     WorkDesc wd = job;
@@ -1473,11 +1443,15 @@ int tpcf::serving_launch_one(tpcf_ctx* ctx, const Shape& sh, const WorkDesc& job
     wd.pos_lo = pos_lo;
     wd.draw_warps = draw_warps;
     wd.stats = stats;
-    wd.item_counter = stats + kStatNextItem;
-    wd.slices = nullptr;
-    wd.slice_ctr = nullptr;
-    wd.nslices = 0;
     Shape s2 = sh;
+    if (sh.tc) {
+        wd.draw_batch = tc_draw_batch(ctx, wd.prune != 0, n);
+        if ((uint64_t)s2.blocks > (uint64_t)n) s2.blocks = (int)std::max<uint32_t>(1, n);
+        if (count_tc_set_smem_limit() != cudaSuccess || launch_count_tc(wd, s2, true, st) != cudaSuccess)
+            return TPCF_ECUDA;
+        ctx->launches.fetch_add(1);
+        return TPCF_OK;
+    }
     const uint64_t warps = (uint64_t)sh.threads / 32;
     const uint64_t need = ((uint64_t)n + warps - 1) / warps;
     if ((uint64_t)s2.blocks > need) s2.blocks = (int)std::max<uint64_t>(1, need);
@@ -1487,7 +1461,9 @@ int tpcf::serving_launch_one(tpcf_ctx* ctx, const Shape& sh, const WorkDesc& job
     return TPCF_OK;
 }
 
-uint64_t tpcf::serving_positions(uint64_t n, uint32_t warps) { return draw_positions(n, warps); }
+uint64_t tpcf::serving_positions(const Shape& sh, uint64_t n, uint32_t warps) {
+    return sh.tc ? n : draw_positions(n, warps);
+}
 
 // ====================================================================== counting ABI
 extern "C" int tpcf_count_auto(tpcf_ctx* ctx, const tpcf_catalog* cat, const tpcf_bins* bins,

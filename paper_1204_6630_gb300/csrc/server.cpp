@@ -10,18 +10,18 @@
 // accumulators in device memory, which stay resident until the job completes.
 //
 // One scheduler thread runs the counting work of all admitted jobs as a
-// sequence of steps.  A step is one launch of the serving-step kernel over
-// slices of many jobs' item ranges, each job with its own bins and
-// histograms: a step gives every job with little work left all of it, then
-// fills a pair budget with the others in admission order.  A job admitted
-// while a step runs joins the next one, so its work overlaps the work already
-// on the device instead of waiting for it.  Up to two steps are queued on the
-// device; the finalize (overflow = pair total - sum of the other entries) and
-// the copy of a job's histograms follow its last step on the same stream, and
-// the estimator runs on the host.  Every item of a job is counted exactly
-// once, whichever steps it lands in, so a job's histograms are those of a lone
-// call.  Jobs whose histograms do not fit the step kernel's shared memory are
-// counted alone by their preparation worker.
+// sequence of steps.  A step holds either the whole work of several small jobs,
+// one launch each on streams of their own (a job of a few thousand points
+// leaves most SMs free: the blocks of the others fill them), or a preemptible
+// launch over a large job's remaining items.  A job admitted while a step runs
+// joins the next one, so its work overlaps the work already on the device
+// instead of waiting for it.  Up to two steps are queued on the device; the
+// finalize (overflow = pair total - sum of the other entries) and the copy of a
+// job's histograms follow its last launch on the same stream, and the
+// estimator runs on the host.  Every item of a job is counted exactly once,
+// whichever steps it lands in, so a job's histograms are those of a lone call.
+// Jobs whose histograms fit neither counting kernel of the steps are counted
+// alone by their preparation worker.
 //
 // Paper: the three histograms of Eq. 1 for each job (Section 1), counted as in
 // Section 3; admission, batching and scheduling have no counterpart in the
@@ -53,6 +53,7 @@ double ms_since(std::chrono::steady_clock::time_point t0) {
 constexpr double kSmallJobPairs = 2e10;
 constexpr double kStepPairs = 1.5e11;
 constexpr int kStepsInFlight = 2;
+constexpr int kJobStreams = 8;  // streams that the small jobs of a step are spread over
 constexpr int kDefaultSlots = 32;
 constexpr int kPrepWorkers = 4;
 
@@ -79,12 +80,11 @@ struct Job {
     void* dev = nullptr;                  // accumulators, pair totals, work description
     unsigned long long* acc = nullptr;    // RR | DR | DD, ne + 1 words each
     unsigned long long* dtot = nullptr;   // their pair totals
-    WorkDesc* dwd = nullptr;              // its work description on the device (step slices point here)
-    WorkDesc hwd{};                       // and on the host (steps that hold only this job)
+    WorkDesc hwd{};                       // its work description
     Shape sh{};                           // the shape the description was built for
     uint64_t n_items = 0, next = 0;       // items of the job / scheduled so far
     double pairs_per_item = 0;
-    int inflight = 0;                     // steps with slices of the job that have not finished
+    int inflight = 0;                     // steps with work of the job that have not finished
     bool solo = false;                    // counted alone (outside the steps)
     // a large job runs in preemptible one-job steps: one draw order over all of its
     // items, laid out for draw_warps warps, positions [0, pos_end) of which pos_next
@@ -97,9 +97,10 @@ struct Job {
     bool work_left() const { return big ? pos_next < pos_end : next < n_items; }
 };
 
-// One step on the device: its slices, the jobs it holds, those it completes.
+// One step on the device: the jobs it holds, those it completes.
 struct Step {
-    int buf = 0;                          // index of its slice / statistics buffers and stream
+    int buf = 0;                          // index of its statistics buffers and streams
+    int launches = 0;                     // blocks of statistics words in use (one per launch)
     cudaEvent_t t0 = nullptr, t1 = nullptr;
     cudaEvent_t kdone = nullptr;          // its counting launch has finished
     std::vector<std::shared_ptr<Job>> jobs, finals;
@@ -130,15 +131,16 @@ class JobServer {
         for (int k = 0; k < kStepsInFlight; ++k)
             ok_ = ok_ && cudaEventCreateWithFlags(&yield_ev_[k], cudaEventDisableTiming) == cudaSuccess;
         // pinned result buffers (one per slot: 3 histograms of up to TPCF_MAX_EDGES + 1 words) and
-        // per-step-buffer slices and statistics words
+        // per step buffer the job streams and a block of statistics words per launch
         const size_t res_words = 3 * (size_t)(TPCF_MAX_EDGES + 1);
         ok_ = ok_ && cudaHostAlloc((void**)&h_res_, (size_t)slots * res_words * 8, cudaHostAllocDefault) == cudaSuccess;
         for (int k = 0; k < kStepsInFlight && ok_; ++k) {
-            ok_ = cudaHostAlloc((void**)&h_slices_[k], (size_t)slots * sizeof(StepSlice), cudaHostAllocDefault) ==
-                      cudaSuccess &&
-                  cudaHostAlloc((void**)&h_stats_[k], kStatWords * 8, cudaHostAllocDefault) == cudaSuccess &&
-                  dev_malloc((void**)&d_slices_[k], (size_t)slots * sizeof(StepSlice)) == cudaSuccess &&
-                  dev_malloc((void**)&d_stats_[k], (kStatWords + (size_t)slots) * 8) == cudaSuccess;
+            ok_ = cudaHostAlloc((void**)&h_stats_[k], (size_t)slots * kStatWords * 8, cudaHostAllocDefault) == cudaSuccess &&
+                  dev_malloc((void**)&d_stats_[k], (size_t)slots * kStatWords * 8) == cudaSuccess &&
+                  cudaEventCreateWithFlags(&fork_ev_[k], cudaEventDisableTiming) == cudaSuccess;
+            for (int q = 0; q < kJobStreams && ok_; ++q)
+                ok_ = cudaStreamCreateWithFlags(&job_streams_[k][q], cudaStreamNonBlocking) == cudaSuccess &&
+                      cudaEventCreateWithFlags(&join_ev_[k][q], cudaEventDisableTiming) == cudaSuccess;
         }
         for (int k = 0; k < slots; ++k) free_slots_.push_back(k);
         // preparation streams at the highest priority: a new job's preparation kernels run as
@@ -178,9 +180,15 @@ class JobServer {
             if (yield_ev_[k]) cudaEventDestroy(yield_ev_[k]);
         if (h_one_) cudaFreeHost(h_one_);
         for (int k = 0; k < kStepsInFlight; ++k) {
-            if (d_slices_[k]) cudaFree(d_slices_[k]);
+            for (int q = 0; q < kJobStreams; ++q) {
+                if (job_streams_[k][q]) {
+                    cudaStreamSynchronize(job_streams_[k][q]);
+                    cudaStreamDestroy(job_streams_[k][q]);
+                }
+                if (join_ev_[k][q]) cudaEventDestroy(join_ev_[k][q]);
+            }
+            if (fork_ev_[k]) cudaEventDestroy(fork_ev_[k]);
             if (d_stats_[k]) cudaFree(d_stats_[k]);
-            if (h_slices_[k]) cudaFreeHost(h_slices_[k]);
             if (h_stats_[k]) cudaFreeHost(h_stats_[k]);
         }
         if (h_res_) cudaFreeHost(h_res_);
@@ -403,14 +411,13 @@ class JobServer {
         if (rc != TPCF_OK) return rc;
         uint64_t totals[3] = {0, 0, 0};
         Shape sh;
-        j.solo = !serving_shape(ctx_, ne, &sh);
+        const uint64_t nd = j.nd, nr = j.nr;
+        j.solo = !serving_shape(ctx_, ne, nd * (nd ? nd - 1 : 0) / 2 + nd * nr + nr * (nr ? nr - 1 : 0) / 2, &sh);
         if (!j.solo) {
             const size_t acc_b = 3ull * (ne + 1) * 8, tot_b = 3 * 8;
-            const size_t off_wd = (acc_b + tot_b + 255) / 256 * 256;
-            if (dev_malloc_async(&j.dev, off_wd + sizeof(WorkDesc), st) != cudaSuccess) return TPCF_ENOMEM;
+            if (dev_malloc_async(&j.dev, acc_b + tot_b, st) != cudaSuccess) return TPCF_ENOMEM;
             j.acc = (unsigned long long*)j.dev;
             j.dtot = j.acc + 3 * (ne + 1);
-            j.dwd = (WorkDesc*)((char*)j.dev + off_wd);
             WorkDesc wd;
             rc = serving_job_desc(ctx_, j.cd, j.cr, j.b, sh, j.acc, &wd, &j.n_items, totals);
             if (rc != TPCF_OK) return rc;
@@ -418,7 +425,6 @@ class JobServer {
             j.sh = sh;
             if (cudaMemsetAsync(j.acc, 0, acc_b, st) != cudaSuccess ||
                 cudaMemcpyAsync(j.dtot, totals, tot_b, cudaMemcpyHostToDevice, st) != cudaSuccess ||
-                cudaMemcpyAsync(j.dwd, &wd, sizeof wd, cudaMemcpyHostToDevice, st) != cudaSuccess ||
                 cudaStreamSynchronize(st) != cudaSuccess)
                 return TPCF_ECUDA;
             j.pairs = totals[0] + totals[1] + totals[2];
@@ -427,7 +433,7 @@ class JobServer {
             j.big = (double)j.pairs > kSmallJobPairs;
             if (j.big) {
                 j.draw_warps = (uint32_t)sh.blocks * (uint32_t)(sh.threads / 32);
-                j.pos_end = serving_positions(j.n_items, j.draw_warps);
+                j.pos_end = serving_positions(sh, j.n_items, j.draw_warps);
             }
             // a job without items (every histogram empty) needs no step
             if (j.n_items == 0) {
@@ -456,8 +462,8 @@ class JobServer {
     //  1. the finalize of large jobs whose draw positions are all taken (a step
     //     without a counting launch);
     //  2. the small jobs with work left, all of it, in admission order, up to
-    //     kStepPairs pairs and the slots: the multi-job kernel (the one-job kernel
-    //     for a single job); a large job's step in flight is told to yield, so
+    //     kStepPairs pairs and the slots: a launch per job, the largest first, on
+    //     the step's job streams; a large job's step in flight is told to yield, so
     //     that this step's blocks get the SMs;
     //  3. when no large job's step is in flight: a preemptible step of the oldest
     //     large job over all of its remaining draw positions (the one-job kernel,
@@ -504,39 +510,35 @@ class JobServer {
         int rc = TPCF_OK;
         // (a yield copy into this buffer's words lands before they are cleared)
         if (cudaStreamWaitEvent(ss, yield_ev_[step.buf], 0) != cudaSuccess ||
-            cudaMemsetAsync(d_stats_[step.buf], 0, (kStatWords + pick.size()) * 8, ss) != cudaSuccess)
+            cudaMemsetAsync(d_stats_[step.buf], 0, std::max<size_t>(1, pick.size()) * kStatWords * 8, ss) != cudaSuccess)
             rc = TPCF_ECUDA;
+        step.launches = (int)std::max<size_t>(1, pick.size());
         if (small) {
-            StepSlice* hs = h_slices_[step.buf];
-            uint32_t pos = 0;
-            int ne_max = 2;
-            for (size_t k = 0; k < pick.size(); ++k) {
-                Job& j = *pick[k];
-                hs[k].job = j.dwd;
-                hs[k].q_begin = (uint32_t)j.next;
-                hs[k].pos_begin = pos;
-                pos += (uint32_t)take[k];
-                hs[k].pos_end = pos;
-                hs[k].pad = 0;
-                j.next += take[k];
+            std::vector<size_t> order(pick.size());
+            for (size_t k = 0; k < order.size(); ++k) order[k] = k;
+            std::stable_sort(order.begin(), order.end(), [&](size_t x, size_t y) {
+                return (double)take[x] * pick[x]->pairs_per_item > (double)take[y] * pick[y]->pairs_per_item;
+            });
+            if (rc == TPCF_OK && cudaEventRecord(fork_ev_[step.buf], ss) != cudaSuccess) rc = TPCF_ECUDA;
+            const int used = (int)std::min<size_t>(kJobStreams, order.size());
+            for (int q = 0; q < used && rc == TPCF_OK; ++q)
+                if (cudaStreamWaitEvent(job_streams_[step.buf][q], fork_ev_[step.buf], 0) != cudaSuccess) rc = TPCF_ECUDA;
+            for (size_t k = 0; k < order.size(); ++k) {
+                Job& j = *pick[order[k]];
+                cudaStream_t js = job_streams_[step.buf][k % kJobStreams];
+                unsigned long long* st = d_stats_[step.buf] + k * kStatWords;
+                if (rc == TPCF_OK)
+                    rc = serving_launch_one(ctx_, j.sh, j.hwd, (uint32_t)j.next, (uint32_t)take[order[k]], 0, 0, st, js);
+                if (rc == TPCF_OK) rc = finalize_job(j, st + kStatError, js);
+                j.next += take[order[k]];
                 ++j.inflight;
-                ne_max = std::max(ne_max, (int)j.edges.size());
-                step.jobs.push_back(pick[k]);
-                step.finals.push_back(pick[k]);  // all of a small job's work is in its step
+                j.finalized = true;
+                step.jobs.push_back(pick[order[k]]);  // all of a small job's work is in its step
             }
-            Shape sh;
-            if (rc == TPCF_OK && !serving_shape(ctx_, ne_max, &sh)) rc = TPCF_EINVAL;
-            if (rc == TPCF_OK && pick.size() == 1) {
-                rc = serving_launch_one(ctx_, pick[0]->sh, pick[0]->hwd, hs[0].q_begin, pos, 0, 0, d_stats_[step.buf],
-                                        ss);
-            } else if (rc == TPCF_OK) {
-                if (cudaMemcpyAsync(d_slices_[step.buf], hs, pick.size() * sizeof(StepSlice), cudaMemcpyHostToDevice,
-                                    ss) != cudaSuccess)
+            for (int q = 0; q < used; ++q)  // (also after an error: what was launched is waited for)
+                if (cudaEventRecord(join_ev_[step.buf][q], job_streams_[step.buf][q]) != cudaSuccess ||
+                    cudaStreamWaitEvent(ss, join_ev_[step.buf][q], 0) != cudaSuccess)
                     rc = TPCF_ECUDA;
-                else
-                    rc = serving_launch(ctx_, sh, ne_max, d_slices_[step.buf], (int)pick.size(),
-                                        d_stats_[step.buf] + kStatWords, pos, d_stats_[step.buf], ss);
-            }
             yield_big_step();
         } else if (step.big) {
             Job& j = *step.big;
@@ -552,26 +554,30 @@ class JobServer {
             }
         }
         cudaEventRecord(step.kdone, ss);
-        // the jobs this step completes: overflow from the pair totals, histograms to the host
+        // the large jobs this step completes
         for (auto& jp : step.finals) {
-            Job& j = *jp;
-            j.finalized = true;
-            const int ne = (int)j.edges.size();
-            if (rc == TPCF_OK &&
-                (launch_finalize_batch(j.acc, ne + 1, ne, j.acc, ne + 1, j.dtot, 3,
-                                       (ctx_->cfg.flags & TPCF_F_CHECK_OVERFLOW) ? 1 : 0,
-                                       d_stats_[step.buf] + kStatError, ss) != cudaSuccess ||
-                 cudaMemcpyAsync(res_buf(j), j.acc, 3ull * (ne + 1) * 8, cudaMemcpyDeviceToHost, ss) != cudaSuccess))
-                rc = TPCF_ECUDA;
+            jp->finalized = true;
+            if (rc == TPCF_OK) rc = finalize_job(*jp, d_stats_[step.buf] + kStatError, ss);
         }
         if (rc == TPCF_OK &&
-            cudaMemcpyAsync(h_stats_[step.buf], d_stats_[step.buf], kStatWords * 8, cudaMemcpyDeviceToHost, ss) !=
+            cudaMemcpyAsync(h_stats_[step.buf], d_stats_[step.buf], (size_t)step.launches * kStatWords * 8,
+                            cudaMemcpyDeviceToHost, ss) !=
                 cudaSuccess)
             rc = TPCF_ECUDA;
         cudaEventRecord(step.t1, ss);
         step_rc_.push_back(rc);
         steps_.push_back(std::move(step));
         return true;
+    }
+
+    // Overflow from the pair totals, then the job's histograms to its result buffer.
+    int finalize_job(Job& j, unsigned long long* err_word, cudaStream_t st) {
+        const int ne = (int)j.edges.size();
+        if (launch_finalize_batch(j.acc, ne + 1, ne, j.acc, ne + 1, j.dtot, 3,
+                                  (ctx_->cfg.flags & TPCF_F_CHECK_OVERFLOW) ? 1 : 0, err_word, st) != cudaSuccess ||
+            cudaMemcpyAsync(res_buf(j), j.acc, 3ull * (ne + 1) * 8, cudaMemcpyDeviceToHost, st) != cudaSuccess)
+            return TPCF_ECUDA;
+        return TPCF_OK;
     }
 
     bool big_in_flight() const {
@@ -600,7 +606,8 @@ class JobServer {
         step_rc_.pop_front();
         float ms = 0.f;
         cudaEventElapsedTime(&ms, step.t0, step.t1);
-        const unsigned long long err = h_stats_[step.buf][kStatError];
+        unsigned long long err = 0;
+        for (int k = 0; k < step.launches; ++k) err |= h_stats_[step.buf][(size_t)k * kStatWords + kStatError];
         if (rc == TPCF_OK && (err & kErrWaitTimeout)) rc = TPCF_ETIMEOUT;
         else if (rc == TPCF_OK && err) rc = TPCF_ECUDA;
         // a large job's step: the positions it took (a yielded step stops early;
@@ -700,8 +707,9 @@ class JobServer {
     unsigned long long* h_one_ = nullptr;  // pinned: the yield word's value
     cudaEvent_t yield_ev_[kStepsInFlight] = {nullptr, nullptr};
     uint64_t* h_res_ = nullptr;
-    StepSlice* h_slices_[kStepsInFlight] = {nullptr, nullptr};
-    StepSlice* d_slices_[kStepsInFlight] = {nullptr, nullptr};
+    cudaStream_t job_streams_[kStepsInFlight][kJobStreams] = {};  // the small jobs of a step
+    cudaEvent_t join_ev_[kStepsInFlight][kJobStreams] = {};
+    cudaEvent_t fork_ev_[kStepsInFlight] = {};
     unsigned long long* h_stats_[kStepsInFlight] = {nullptr, nullptr};
     unsigned long long* d_stats_[kStepsInFlight] = {nullptr, nullptr};
     std::chrono::steady_clock::time_point t0_;
