@@ -208,12 +208,14 @@ static __device__ int find_sub(const WorkDesc& wd, uint64_t q) {
     return lo;
 }
 
+template <bool BY_ROOT = true>
 static __device__ bool load_item(const WorkDesc& wd, uint32_t q, Cursor& c) {
     c.q = q;
     c.sub = find_sub(wd, q);
     const SubProblem& sp = sub_of(wd, c.sub);
-    const uint64_t local = walk_item(q - sp.item_begin, sp.n_items, sp.walk_mult);
-    c.g = item_geom(local, sp.na, sp.nb, sp.n_iblk, sp.n_jchunk, sp.auto_mode != 0, wd.I, wd.Jc, wd.J);
+    const uint64_t local = walk_item_inv(q - sp.item_begin, sp.n_items, sp.walk_mult, sp.walk_inv);
+    c.g = item_geom(local, sp.na, sp.nb, sp.n_iblk, sp.n_jchunk, sp.auto_mode != 0, wd.I, wd.Jc, wd.J,
+                    BY_ROOT);
     c.t = c.g.t_first;
     return c.t < c.g.t_end;
 }
@@ -243,6 +245,7 @@ __device__ void load_bins(const BinsDev* bd, const WorkDesc& wd, bool plain) {
         // Shared copy of the LUT as 16-bit entries (see lut_code).
         const bool count_over = (wd.flags & TPCF_F_CHECK_OVERFLOW) != 0;
         unsigned short* lut = sptr<unsigned short>(wd.off_lut);
+#pragma unroll 8
         for (int k = threadIdx.x; k < kLutCells; k += T) {
             const uint32_t e = bd->lut[k];
             lut[k] = lut_code(e & 0xffffu, e >> 16, (uint32_t)ne, count_over);
@@ -290,17 +293,27 @@ __device__ __forceinline__ void hist_inc(const HistCol& hc, int h) {
 // kernel derives overflow from the pair total.  Each thread takes its own
 // half out of the shared word with an atomic subtract, since the partner warp
 // may be adding to the other half at the same time.
+// Eight rows at a time: their loads, sums and atomics overlap (row by row a
+// merge of 66 rows took 25000 cycles).
 template <int T>
 __device__ void warp_flush_hist(const HistCol& hc, int nedges, bool count_over, unsigned long long* out) {
     const int lane = threadIdx.x & 31;
     const uint32_t sh = hc.inc == 1u ? 0u : 16u;
-    for (int h = 0; h <= nedges; ++h) {
-        const uint32_t a = hc.addr + ((uint32_t)h << row_shift<T>());
-        uint32_t mine = (ld_shared_u32(a) >> sh) & 0xffffu;
-        if (mine) red_add_shared(a, 0u - (mine << sh));
-        if (h == nedges && !count_over) break;
-        mine = __reduce_add_sync(0xffffffffu, mine);
-        if (lane == 0 && mine != 0) atomicAdd(out + h, (unsigned long long)mine);
+    for (int h0 = 0; h0 <= nedges; h0 += 8) {
+        uint32_t v[8], sum = 0;
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            v[k] = h0 + k <= nedges ? (ld_shared_u32(hc.addr + ((uint32_t)(h0 + k) << row_shift<T>())) >> sh) & 0xffffu : 0u;
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            if (v[k]) red_add_shared(hc.addr + ((uint32_t)(h0 + k) << row_shift<T>()), 0u - (v[k] << sh));
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+            const uint32_t t = __reduce_add_sync(0xffffffffu, v[k]);
+            if (lane == k) sum = t;
+        }
+        const int h = h0 + lane;  // lane k merges row h0 + k
+        if (lane < 8 && sum != 0u && (h < nedges || (h == nedges && count_over))) atomicAdd(out + h, (unsigned long long)sum);
     }
 }
 

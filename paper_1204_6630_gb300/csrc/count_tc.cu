@@ -56,10 +56,10 @@ constexpr int kQueueCodes = 64;                   // per-warp queue of unsettled
 // a wait is bounded by the time without progress.
 enum TcCtl { kTcAbort = 0, kTcTmem = 1, kTcBeat = 2, kTcCtlWords = 32 };
 
-// A staged tile: first i of the item, first j of the tile, and what to do with it.
-struct TcMeta {
-    uint32_t i0, jbase;
+// A staged tile: what to do with it, first j of the tile, first i of the item.
+struct __align__(16) TcMeta {
     uint32_t info;   // kInfo* below, sub-problem in bits 16..31
+    uint32_t jbase, i0;
     uint32_t pad;
 };
 enum : uint32_t {
@@ -118,6 +118,17 @@ __device__ __forceinline__ void tc_alloc(uint32_t dst) {
 }
 __device__ __forceinline__ void tc_dealloc(uint32_t tmem) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)kTmemCols));
+}
+// A tile record (16-byte aligned shared address).
+__device__ __forceinline__ void rec_load(uint32_t a, uint32_t& info, uint32_t& jbase, uint32_t& i0) {
+    [[maybe_unused]] uint32_t unused;
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(info), "=r"(jbase), "=r"(i0), "=r"(unused)
+                 : "r"(a)
+                 : "memory");
+}
+__device__ __forceinline__ void rec_store(uint32_t a, uint32_t info, uint32_t jbase, uint32_t i0) {
+    asm volatile("st.shared.v4.u32 [%0], {%1, %2, %3, %3};" ::"r"(a), "r"(info), "r"(jbase), "r"(i0) : "memory");
 }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
@@ -282,6 +293,12 @@ __device__ __forceinline__ void tc_drain(const WorkDesc& wd, const SubProblem& s
     }
 }
 
+// Merges the warp's counters (out of line: inlined three times it made the
+// loop below spill).
+static __device__ __noinline__ void tc_merge(HistCol hc, int ne, bool check, unsigned long long* out) {
+    warp_flush_hist<kWorkThreads>(hc, ne, check, out);
+}
+
 // ============================================================== the kernel
 // PREEMPT: draws start at wd.pos_lo and stop once stats[kStatYield] is set
 // (the job server's steps of one large job).  PRUNE: tiles and groups whose
@@ -300,7 +317,7 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
     uint64_t* const a_empty = a_full + 2;
     uint64_t* const d_full = a_full + 4;
     uint64_t* const d_free = d_full + kGroups;
-    TcMeta* const meta = sptr<TcMeta>(wd.off_meta);
+    const uint32_t meta = smem_addr(dyn_smem) + wd.off_meta;
     const bool check = (wd.flags & TPCF_F_CHECK_OVERFLOW) != 0;
     const uint64_t limit = wd.wait_limit_ns;
 
@@ -353,7 +370,7 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
         bool aborted = false;
 
         auto flush = [&]() {
-            warp_flush_hist<kWorkThreads>(hc, wd.ne, check, cur_hist);
+            tc_merge(hc, wd.ne, check, cur_hist);
             if (check) {
                 const unsigned long long o = warp_sum(over);
                 if (lane == 0 && o) atomicAdd(cur_hist + wd.ne, o);
@@ -367,14 +384,13 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                 aborted = true;
                 break;
             }
-            const volatile TcMeta* vm = meta + stage;
-            const uint32_t info = vm->info;
+            uint32_t info, jbase, i0;
+            rec_load(meta + stage * (uint32_t)sizeof(TcMeta), info, jbase, i0);
             if (info & kInfoStop) {
                 __syncwarp();
                 if (lane == 0) mbar_arrive(empty + stage);
                 break;
             }
-            const uint32_t jbase = vm->jbase;
             // other i-points: a new item's, or (PRUNE) another 128 of the item's
             bool turn = (info & kInfoNew) != 0u;
             uint32_t gi = (uint32_t)g;
@@ -396,7 +412,7 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                 }
                 const int sub = (int)(info >> 16);
                 const SubProblem& sp = sub_of(wd, sub);
-                iw = vm->i0 + kBlk * gi + 32u * (uint32_t)(warp & 3);
+                iw = i0 + kBlk * gi + 32u * (uint32_t)(warp & 3);
                 jq0 = jbase;
                 unsigned long long* tgt = sp.hist;
                 if (sp.row_seg) tgt += (size_t)__ldg(sp.row_seg + iw / kSegAlign) * sp.row_stride;
@@ -411,9 +427,6 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                 ay = pack2(p.y, p.y);
                 az = pack2(p.z, p.z);
             }
-            uint32_t nbatch = 0, kept = 0;
-            // a lane's counter gains at most one per pair of the tile and one per queue batch
-            if (inc_bound + 2u * kBlk + 2u > 0xffffu || over > 0x40000000u) flush();
             if ((info >> g) & 1u) {
                 // ---- the group's accumulators: one maximum per 32 x 32 pairs
                 if (!tc_wait(d_full + g, dphase, limit, ctl, wd.stats)) {
@@ -422,9 +435,11 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                 }
                 dphase ^= 1u;
                 tc_fence_after();
+                // (votes after each pair of loads: without them four loads are in flight and their
+                // registers spill)
                 float m0 = tc_row_max32(d_addr), m1 = tc_row_max32(d_addr + 32u);
                 tc_wait_ld(m0, m1);
-                kept = __any_sync(0xffffffffu, m0 >= thr) ? 1u : 0u;
+                uint32_t kept = __any_sync(0xffffffffu, m0 >= thr) ? 1u : 0u;
                 kept |= __any_sync(0xffffffffu, m1 >= thr) ? 2u : 0u;
                 float m2 = tc_row_max32(d_addr + 64u), m3 = tc_row_max32(d_addr + 96u);
                 tc_wait_ld(m2, m3);
@@ -432,50 +447,57 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                 if (lane == 0) mbar_arrive(d_free + g);
                 kept |= __any_sync(0xffffffffu, m2 >= thr) ? 4u : 0u;
                 kept |= __any_sync(0xffffffffu, m3 >= thr) ? 8u : 0u;
-                const SubProblem& sp = sub_of(wd, cur_sub);
-                // blocks at or below the diagonal (j-block and i-block of 32 coincide or do not overlap)
-                uint32_t todo = check ? 0xfu : kept;
-                if (rule == 1u && jbase < iw) todo &= ~0u << ((iw - jbase) >> 5 < 4u ? (iw - jbase) >> 5 : 4u);
-                // (a counted block's overflow needs its pair mask; otherwise a mask is needed on the
-                // diagonal and, where padding could look in range, at the catalogs' ends)
-                const bool ends = (wd.need_idx || check) && (jbase + kBlk > nb || iw + 32u > na);
-                const float* sx = sptr<const float>(wd.off_stage + stage * kStageBytes + kBlkX);
-                while (todo) {
-                    const uint32_t b = (uint32_t)__ffs((int)todo) - 1u;
-                    todo &= todo - 1u;
-                    const uint32_t jb = jbase + 32u * b;
-                    const bool diag = rule != 0u && jb == iw;
-                    uint32_t valid = ~0u;
-                    if (diag || ends) {
-                        const uint32_t left = nb > jb ? nb - jb : 0u;
-                        if (left < 32u) valid = (1u << left) - 1u;
-                        if (iw + (uint32_t)lane >= na) valid = 0u;
-                        if (diag) valid &= rule == 1u ? (0xfffffffeu << lane) : ~(1u << lane);
-                    }
-                    if (!((kept >> b) & 1u)) {  // (only with a counted overflow row)
-                        over += (uint32_t)__popc(valid);
-                        continue;
-                    }
-                    uint32_t um = (diag || ends) ? tc_block<true>(wd, ax, ay, az, sx + 32 * b, valid, hc)
-                                                 : tc_block<false>(wd, ax, ay, az, sx + 32 * b, valid, hc);
-                    // ---- queue the unsettled pairs; a full batch of 32 is classified at once
-                    uint32_t act = __ballot_sync(0xffffffffu, um != 0u);
-                    while (act) {
-                        if (um) {
-                            const int k = __clz((int)um);
-                            um &= ~(0x80000000u >> k);
-                            uq[qn + (uint32_t)__popc(act & ((1u << lane) - 1u))] =
-                                (uint32_t)lane | ((jb + (uint32_t)k - jq0) << 5);
+                // most tiles hold nothing within the range: on to the next
+                if (kept != 0u || check) {
+                    // a lane's counter gains at most one per pair of the tile and one per queue batch
+                    // (one batch more when the queue is emptied at the item's end)
+                    if (inc_bound + 2u * kBlk + 2u > 0xffffu || over > 0x40000000u) flush();
+                    inc_bound += 32u * (uint32_t)__popc(kept);
+                    const SubProblem& sp = sub_of(wd, cur_sub);
+                    // blocks at or below the diagonal (j-block and i-block of 32 coincide or do not overlap)
+                    uint32_t todo = check ? 0xfu : kept;
+                    if (rule == 1u && jbase < iw) todo &= ~0u << ((iw - jbase) >> 5 < 4u ? (iw - jbase) >> 5 : 4u);
+                    // (a counted block's overflow needs its pair mask; otherwise a mask is needed on the
+                    // diagonal and, where padding could look in range, at the catalogs' ends)
+                    const bool ends = (wd.need_idx || check) && (jbase + kBlk > nb || iw + 32u > na);
+                    const float* sx = sptr<const float>(wd.off_stage + stage * kStageBytes + kBlkX);
+                    while (todo) {
+                        const uint32_t b = (uint32_t)__ffs((int)todo) - 1u;
+                        todo &= todo - 1u;
+                        const uint32_t jb = jbase + 32u * b;
+                        const bool diag = rule != 0u && jb == iw;
+                        uint32_t valid = ~0u;
+                        if (diag || ends) {
+                            const uint32_t left = nb > jb ? nb - jb : 0u;
+                            if (left < 32u) valid = (1u << left) - 1u;
+                            if (iw + (uint32_t)lane >= na) valid = 0u;
+                            if (diag) valid &= rule == 1u ? (0xfffffffeu << lane) : ~(1u << lane);
                         }
-                        qn += (uint32_t)__popc(act);
-                        if (qn >= 32u) {
-                            __syncwarp();
-                            qn -= 32u;
-                            tc_drain(wd, sp, uq + qn, 32u, ax, ay, az, iw, jq0, hc, band, mism);
-                            ++nbatch;
-                            __syncwarp();  // the batch is read before later codes overwrite it
+                        if (!((kept >> b) & 1u)) {  // (only with a counted overflow row)
+                            over += (uint32_t)__popc(valid);
+                            continue;
                         }
-                        act = __ballot_sync(0xffffffffu, um != 0u);
+                        uint32_t um = (diag || ends) ? tc_block<true>(wd, ax, ay, az, sx + 32 * b, valid, hc)
+                                                     : tc_block<false>(wd, ax, ay, az, sx + 32 * b, valid, hc);
+                        // ---- queue the unsettled pairs; a full batch of 32 is classified at once
+                        uint32_t act = __ballot_sync(0xffffffffu, um != 0u);
+                        while (act) {
+                            if (um) {
+                                const int k = __clz((int)um);
+                                um &= ~(0x80000000u >> k);
+                                uq[qn + (uint32_t)__popc(act & ((1u << lane) - 1u))] =
+                                    (uint32_t)lane | ((jb + (uint32_t)k - jq0) << 5);
+                            }
+                            qn += (uint32_t)__popc(act);
+                            if (qn >= 32u) {
+                                __syncwarp();
+                                qn -= 32u;
+                                tc_drain(wd, sp, uq + qn, 32u, ax, ay, az, iw, jq0, hc, band, mism);
+                                ++inc_bound;
+                                __syncwarp();  // the batch is read before later codes overwrite it
+                            }
+                            act = __ballot_sync(0xffffffffu, um != 0u);
+                        }
                     }
                 }
             }
@@ -484,11 +506,10 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                 if (qn) {
                     __syncwarp();
                     tc_drain(wd, sub_of(wd, cur_sub), uq, qn, ax, ay, az, iw, jq0, hc, band, mism);
-                    ++nbatch;
+                    ++inc_bound;
                     qn = 0;
                 }
             }
-            inc_bound += 32u * (uint32_t)__popc(kept) + nbatch;
             __syncwarp();
             if (lane == 0) mbar_arrive(empty + stage);
             if (++stage == S) {
@@ -509,8 +530,8 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
         bool any = false;
         while (true) {
             if (!tc_wait(full + stage, phase, limit, ctl, wd.stats)) break;
-            const volatile TcMeta* vm = meta + stage;
-            const uint32_t info = vm->info;
+            uint32_t info, jbase, i0;
+            rec_load(meta + stage * (uint32_t)sizeof(TcMeta), info, jbase, i0);
             if (info & kInfoStop) {
                 __syncwarp();
                 if (lane == 0) mbar_arrive(empty + stage);
@@ -559,7 +580,8 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
         // 2 degrees: 145 ms with one item per draw, 40 ms with 32, 37 ms with the
         // chunk spheres, 26 ms with tiles given to the groups of warps in turn).
         const uint32_t batch = wd.draw_batch;
-        while (ok) {
+        // (lane 0's result counts; it is asked for a batch ahead, while the current one is issued)
+        auto draw = [&]() {
             unsigned long long p = ~0ull;
             if (lane == 0) {
                 if constexpr (PREEMPT) {
@@ -568,17 +590,22 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                 } else {
                     p = atomicAdd(counter, (unsigned long long)batch);
                 }
-                ctl[kTcBeat] = ctl[kTcBeat] + 1;
             }
-            p = __shfl_sync(0xffffffffu, p, 0);
+            return p;
+        };
+        unsigned long long next = draw();
+        while (ok) {
+            const unsigned long long p = __shfl_sync(0xffffffffu, next, 0);
             if (p >= n || ctl[kTcAbort]) break;
+            next = draw();
+            if (lane == 0) ctl[kTcBeat] = ctl[kTcBeat] + 1;
             Cursor c;
             c.sub = 0;
             c.g = ItemGeom{0u, 0u, 0u, 0u};
             uint32_t gm[kGroups] = {0u, 0u, 0u, 0u};
             unsigned long long pairs = 0;
             if ((uint32_t)lane < batch && p + (uint32_t)lane < n &&
-                load_item(wd, (uint32_t)(wd.item_lo + p + (uint32_t)lane), c)) {
+                load_item<!PRUNE>(wd, (uint32_t)(wd.item_lo + p + (uint32_t)lane), c)) {
                 const SubProblem& sp = sub_of(wd, c.sub);
                 pairs = span_pairs(c.g.i0, wd.I, (uint64_t)c.g.j0 + (uint64_t)c.t * wd.J,
                                    (uint64_t)c.g.j0 + (uint64_t)c.g.t_end * wd.J, sp.na, sp.nb, sp.auto_mode != 0);
@@ -643,15 +670,16 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                 {
                     const unsigned char* src = sp.a_blk + (size_t)(i0 / kBlk) * kBlkBytes;
                     uint4* const dst = sptr<uint4>(wd.off_atile + buf * kABytes);
-#pragma unroll 2
-                    for (int gg = 0; gg < kGroups; ++gg) {
-                        uint4 x[4];
+#pragma unroll 1
+                    for (int gg = 0; gg < kGroups; gg += 2) {  // (eight loads in flight)
+                        uint4 x[8];
 #pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            x[k] = __ldg(reinterpret_cast<const uint4*>(src + (size_t)gg * kBlkBytes) + 32 * k + lane);
+                        for (int k = 0; k < 8; ++k)
+                            x[k] = __ldg(reinterpret_cast<const uint4*>(src + (size_t)(gg + k / 4) * kBlkBytes) +
+                                         32 * (k % 4) + lane);
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            uint4* const p = dst + gg * (kABlock / 16) + 32 * k + lane;
+                        for (int k = 0; k < 8; ++k) {
+                            uint4* const p = dst + (gg + k / 4) * (kABlock / 16) + 32 * (k % 4) + lane;
                             p[0] = x[k];
                             // Y: the halves' two triples exchanged
                             p[kBlk] = make_uint4((x[k].y >> 16) | (x[k].z << 16), (x[k].z >> 16) | (x[k].x << 16),
@@ -685,11 +713,9 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                     }
                     if (lane == 0) {
                         const uint32_t jt = j0 + t * kBlk;
-                        volatile TcMeta* vm = meta + stage;
-                        vm->i0 = i0;
-                        vm->jbase = jt;
-                        vm->info = who | (buf ? kInfoABuf : 0u) | first | (tiles ? 0u : kInfoLast) |
-                                   ((uint32_t)sub << 16);
+                        rec_store(meta + stage * (uint32_t)sizeof(TcMeta),
+                                  who | (buf ? kInfoABuf : 0u) | first | (tiles ? 0u : kInfoLast) | ((uint32_t)sub << 16),
+                                  jt, i0);
                         fence_proxy_async_smem();  // the group's reads of the stage's previous tile come first
                         if (!(hook && issued == 0)) {  // (test hook: the first copy is never issued)
                             const unsigned char* src = sp.b_blk + (size_t)(jt / kBlk) * kBlkBytes;
@@ -709,8 +735,7 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
             }
         }
         if (ok && !ctl[kTcAbort] && tc_wait(empty + stage, phase ^ 1u, limit, ctl, wd.stats) && lane == 0) {
-            volatile TcMeta* vm = meta + stage;
-            vm->info = kInfoStop;
+            rec_store(meta + stage * (uint32_t)sizeof(TcMeta), kInfoStop, 0u, 0u);
             mbar_arrive(full + stage);
         }
         __syncwarp();

@@ -5,6 +5,7 @@
 #pragma once
 
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 
 namespace tpcf {
@@ -53,25 +54,54 @@ __host__ __device__ inline uint64_t items_of(uint32_t n_iblk, uint32_t n_jchunk,
     return (uint64_t)n_iblk * n_jchunk - first_chunk_prefix(n_iblk, I, Jc);
 }
 
+// Auto mode: items before row ib, S(ib) = ib * n_jchunk - F(ib), and the row of
+// item `local`: the largest ib with S(ib) <= local.
+__host__ __device__ inline uint64_t row_start(uint64_t ib, uint32_t n_jchunk, uint32_t I, uint32_t Jc) {
+    return ib * (uint64_t)n_jchunk - first_chunk_prefix(ib, I, Jc);
+}
+
+// A single-precision root of S's quadratic (F(ib) is near k ib (ib - 1) / 2, k =
+// I / Jc), then exact steps, one or two: the shorter way for one item (20,011
+// points: 119 us against 127 with the search).
+__host__ __device__ inline uint64_t row_by_root(uint64_t local, uint32_t n_iblk, uint32_t n_jchunk, uint32_t I,
+                                                uint32_t Jc) {
+    const float k = (float)I / (float)Jc, h = (float)n_jchunk + 0.5f * k;
+    const float disc = h * h - 2.0f * k * (float)local;
+    const float est = (h - sqrtf(disc > 0.f ? disc : 0.f)) / k;
+    uint64_t ib = est > 0.f ? (uint64_t)est : 0ull;
+    if (ib > (uint64_t)n_iblk - 1) ib = (uint64_t)n_iblk - 1;
+    while (row_start(ib, n_jchunk, I, Jc) > local) --ib;
+    while (ib + 1 < n_iblk && row_start(ib + 1, n_jchunk, I, Jc) <= local) ++ib;
+    return ib;
+}
+
+// Bisection: the same number of steps in every lane, which a warp that looks up
+// 32 items at once needs (pruned full sphere: 26.4 ms against 29.3 with the root).
+__host__ __device__ inline uint64_t row_by_search(uint64_t local, uint32_t n_iblk, uint32_t n_jchunk, uint32_t I,
+                                                  uint32_t Jc) {
+    uint64_t lo = 0, hi = n_iblk;  // S(lo) <= local < S(hi)
+    while (hi - lo > 1) {
+        const uint64_t mid = (lo + hi) / 2;
+        if (row_start(mid, n_jchunk, I, Jc) <= local) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+
 // Local item index -> geometry.  Auto mode: row ib has n_jchunk - floor(ib I / Jc)
 // items, starting at chunk floor(ib I / Jc), the chunk holding j = ib * I.
 __host__ __device__ inline ItemGeom item_geom(uint64_t local, uint32_t na, uint32_t nb,
                                               uint32_t n_iblk, uint32_t n_jchunk, bool auto_mode,
-                                              uint32_t I, uint32_t Jc, uint32_t J) {
+                                              uint32_t I, uint32_t Jc, uint32_t J, bool by_root = true) {
     uint64_t ib, jc;
-    if (!auto_mode) {
+    if (!auto_mode && local <= 0xffffffffull) {
+        ib = (uint32_t)local / n_jchunk;
+        jc = (uint32_t)local % n_jchunk;
+    } else if (!auto_mode) {
         ib = local / n_jchunk;
         jc = local % n_jchunk;
     } else {
-        // largest ib with S(ib) <= local, S(ib) = ib * n_jchunk - F(ib)
-        uint64_t lo = 0, hi = n_iblk;  // S(lo) <= local < S(hi)
-        while (hi - lo > 1) {
-            uint64_t mid = (lo + hi) / 2;
-            uint64_t s = mid * (uint64_t)n_jchunk - first_chunk_prefix(mid, I, Jc);
-            if (s <= local) lo = mid; else hi = mid;
-        }
-        ib = lo;
-        uint64_t s = ib * (uint64_t)n_jchunk - first_chunk_prefix(ib, I, Jc);
+        ib = by_root ? row_by_root(local, n_iblk, n_jchunk, I, Jc) : row_by_search(local, n_iblk, n_jchunk, I, Jc);
+        const uint64_t s = row_start(ib, n_jchunk, I, Jc);
         jc = first_chunk(ib, I, Jc) + (local - s);
     }
     ItemGeom g;
@@ -142,6 +172,21 @@ __host__ __device__ inline uint64_t walk_multiplier(uint64_t n) {
 
 __host__ __device__ inline uint64_t walk_item(uint64_t k, uint64_t n, uint64_t m) {
     return n ? (k * m) % n : 0;
+}
+
+// The same with inv = floor((2^64 - 1) / n) in place of the 64-bit division
+// (k, m < n < 2^32, so that k m < 2^64): the quotient estimate is at most two short.
+__host__ __device__ inline uint64_t walk_item_inv(uint64_t k, uint64_t n, uint64_t m, uint64_t inv) {
+    if (n == 0) return 0;
+    const uint64_t x = k * m;
+#ifdef __CUDA_ARCH__
+    const uint64_t q = __umul64hi(x, inv);
+#else
+    const uint64_t q = (uint64_t)(((unsigned __int128)x * inv) >> 64);
+#endif
+    uint64_t r = x - q * n;
+    while (r >= n) r -= n;
+    return r;
 }
 
 }  // namespace tpcf

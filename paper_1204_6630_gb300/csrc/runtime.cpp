@@ -902,7 +902,7 @@ bool shape_for(tpcf_ctx* ctx, int mode, int nedges, int T, int R, int Jreq, int 
 // down to one tile (512 x 128 pairs) per item.  False when the histograms do
 // not leave shared memory for a ring of four stages.
 bool tc_shape_for(tpcf_ctx* ctx, int nedges, uint64_t total_pairs, Shape* sh) {
-    constexpr uint64_t kTcItemsPerSm = 16;
+    constexpr uint64_t kTcItemsPerSm = 8;
     int S = 8;
     while (S >= 4 && count_tc_smem_bytes(S, nedges) > ctx->smem_optin) S -= 2;
     if (S < 4) return false;
@@ -991,6 +991,7 @@ uint64_t build_work(tpcf_ctx* ctx, const SubSpec* specs, int nsub, const BinsDev
         sp.item_begin = items;
         sp.n_items = (p.na == 0 || p.nb == 0) ? 0 : items_of(sp.n_iblk, sp.n_jchunk, p.auto_mode, I, Jc);
         sp.walk_mult = walk_multiplier(sp.n_items);
+        sp.walk_inv = sp.n_items ? ~0ull / sp.n_items : 0ull;
         sp.hist = acc + hist_base * acc_stride;
         sp.bins = bins_dev;
         sp.row_seg = p.row_seg ? p.row_seg + p.a_off / kSegAlign : nullptr;

@@ -88,6 +88,7 @@ struct SubProblem {
     uint64_t item_begin;  // global walk position of this sub-problem's first item
     uint64_t n_items;
     uint64_t walk_mult;   // position item_begin + k visits local item (k * walk_mult) mod n_items
+    uint64_t walk_inv;          // floor((2^64 - 1) / n_items)
     unsigned long long* hist;   // B + 2 accumulators (device)
     const BinsDev* bins;        // device pointer to this sub-problem's bins
     // Row attribution (leave-one-out jackknife): pairs go to histogram
