@@ -20,6 +20,18 @@
 // of 16 additions of partial sums below 1.002).  A block is rejected when
 // every D < tc_thr = RD(C_B - 64u), which proves d < C_B for all its pairs.
 //
+// 3-D counts (EUCLID) reject on D = a.b - |b|^2 / 2: d^2 >= S_B is D <= (|a|^2 -
+// S_B) / 2, a threshold of the lane that holds a.  The operands hold the points
+// scaled by powers of two to norm <= 1 (2^-ka, 2^-kb, one per catalog); the two
+// spare places of X hold n1 + n2 = -|b|^2 / 2, which the i-side meets with 0 in X
+// and with s = 2^(kb - ka) in Y, so that D comes out in units of 2^(ka + kb).
+// Error with t = max(s, 1/s): 2u and 9.8u as above, 5u s from |b|^2 / 2 (three
+// roundings, the copies, the split), 16 additions of partial sums below 2t at 2u t,
+// 8u t from the threshold (three roundings of |a|^2 / 2s, the copies, the last
+// addition where the screen rejects anything): 57u t in all, kTcGuard3d = 128u.
+// 300,000 + 300,000 points, distances to 0.05 of the box: 12.2 ms (FP32
+// differences on the CUDA cores: 33.5 ms, bound by their nine operations a pair).
+//
 // One CTA per SM, 21 warps:
 //   * warps 0..15, four groups of four: group g reads the accumulators of
 //     i-points 128 g .. 128 g + 127 of the CTA's 512 (tcgen05.ld with a maximum
@@ -237,10 +249,11 @@ __device__ __forceinline__ float4 union_sphere(const float4 (&g)[kGroups]) {
 // path of count.cu (the codes of a group of four j are read before the
 // increments of the group before it).  `valid` (MASKED) names the lane's pairs
 // that may be counted.  Returns the unsettled pairs: pair j at bit 31 - j.
-template <bool MASKED>
+template <bool EUCLID, bool MASKED>
 __device__ __forceinline__ uint32_t tc_block(const WorkDesc& wd, u64 ax, u64 ay, u64 az, const float* sx,
                                              uint32_t valid, const HistCol& hc) {
-    const uint32_t lut_adj = smem_addr(dyn_smem) + wd.off_lut - 0x4B000000u * 2u;
+    const uint32_t lut_base = smem_addr(dyn_smem) + wd.off_lut;
+    const uint32_t lut_adj = lut_base - 0x4B000000u * 2u;
     const u64 nt2 = wd.neg_fast_t2;
     uint32_t ent[2][4];
     uint32_t um = 0;
@@ -250,14 +263,26 @@ __device__ __forceinline__ uint32_t tc_block(const WorkDesc& wd, u64 ax, u64 ay,
             const ulonglong2 bx = *reinterpret_cast<const ulonglong2*>(sx + 4 * k);
             const ulonglong2 by = *reinterpret_cast<const ulonglong2*>(sx + kBlk + 4 * k);
             const ulonglong2 bz = *reinterpret_cast<const ulonglong2*>(sx + 2 * kBlk + 4 * k);
-            const u64 v0 = ffma2(az, bz.x, ffma2(ay, by.x, ffma2(ax, bx.x, nt2)));
-            const u64 v1 = ffma2(az, bz.y, ffma2(ay, by.y, ffma2(ax, bx.y, nt2)));
+            u64 v0, v1;
+            if constexpr (EUCLID) {  // z as euclid_z rounds it
+                const u64 dx0 = fsub2(ax, bx.x), dy0 = fsub2(ay, by.x), dz0 = fsub2(az, bz.x);
+                const u64 dx1 = fsub2(ax, bx.y), dy1 = fsub2(ay, by.y), dz1 = fsub2(az, bz.y);
+                v0 = ffma2(dz0, dz0, ffma2(dy0, dy0, ffma2(dx0, dx0, 0ull)));
+                v1 = ffma2(dz1, dz1, ffma2(dy1, dy1, ffma2(dx1, dx1, 0ull)));
+            } else {
+                v0 = ffma2(az, bz.x, ffma2(ay, by.x, ffma2(ax, bx.x, nt2)));
+                v1 = ffma2(az, bz.y, ffma2(ay, by.y, ffma2(ax, bx.y, nt2)));
+            }
             const float e[4] = {lo_of(v0), hi_of(v0), lo_of(v1), hi_of(v1)};
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                const float v = __saturatef(e[u] * wd.lut_scale);
-                const float f = fmaf(v, (float)(1 << kLutBits), 8388608.0f);
-                ent[k & 1][u] = (uint32_t)ld_shared_s16(__float_as_uint(f) * 2u + lut_adj);
+                if constexpr (EUCLID) {
+                    ent[k & 1][u] = (uint32_t)ld_shared_s16(euclid_cell_addr(wd, e[u], lut_base));
+                } else {
+                    const float v = __saturatef(e[u] * wd.lut_scale);
+                    const float f = fmaf(v, (float)(1 << kLutBits), 8388608.0f);
+                    ent[k & 1][u] = (uint32_t)ld_shared_s16(__float_as_uint(f) * 2u + lut_adj);
+                }
             }
         }
         if (k >= 1) {
@@ -275,6 +300,7 @@ __device__ __forceinline__ uint32_t tc_block(const WorkDesc& wd, u64 ax, u64 ay,
 
 // Classifies the n <= 32 queued pairs at q, one per lane: code = lane holding
 // the i-point | j-offset from jq0 << 5.
+template <bool EUCLID>
 __device__ __forceinline__ void tc_drain(const WorkDesc& wd, const SubProblem& sp, const uint32_t* q, uint32_t n,
                                          u64 ax, u64 ay, u64 az, uint32_t iw, uint32_t jq0, const HistCol& hc,
                                          uint32_t& band, uint32_t& mism) {
@@ -288,7 +314,7 @@ __device__ __forceinline__ void tc_drain(const WorkDesc& wd, const SubProblem& s
     const float z = __shfl_sync(0xffffffffu, lo_of(az), l);
     if (has) {
         const float3 b = ldg_point32(sp.b_blk, jg);
-        hist_inc<kWorkThreads>(hc, classify_unsettled<false>(wd, sp, x, y, z, b.x, b.y, b.z, iw + (uint32_t)l, jg,
+        hist_inc<kWorkThreads>(hc, classify_unsettled<EUCLID>(wd, sp, x, y, z, b.x, b.y, b.z, iw + (uint32_t)l, jg,
                                                              band, mism));
     }
 }
@@ -305,7 +331,7 @@ static __device__ __noinline__ void tc_merge(HistCol hc, int ne, bool check, uns
 // bounding spheres are too far apart are left out, and a tile's i-groups go to
 // the groups of warps in turn (without pruning group g always takes i-points
 // 128 g .. of the item, and its loop is the shorter for it).
-template <bool PREEMPT, bool PRUNE>
+template <bool PREEMPT, bool PRUNE, bool EUCLID>
 __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_constant__ WorkDesc wd) {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const uint32_t S = wd.stages;
@@ -358,7 +384,7 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
         const uint32_t d_addr = tmem + (uint32_t)(g * 128) + ((uint32_t)(warp & 3) << 21);  // lane (w % 4) * 32
         const HistCol hc = hist_col<kWorkThreads>(wd);
         uint32_t* const uq = sptr<uint32_t>(wd.off_queue) + (uint32_t)warp * kQueueCodes;
-        const float thr = wd.tc_thr;
+        float thr = wd.tc_thr;  // (3-D: the i-point's own threshold)
         uint32_t stage = 0, phase = 0, dphase = 0;
         uint32_t iw = 0, qn = 0, jq0 = 0;  // first i of the warp, queue length, j origin of the queue's codes
         uint32_t na = 0, nb = 0, rule = 0;
@@ -403,7 +429,7 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                 if constexpr (PRUNE) {
                     if (qn) {
                         __syncwarp();
-                        tc_drain(wd, sub_of(wd, cur_sub), uq, qn, ax, ay, az, iw, jq0, hc, band, mism);
+                        tc_drain<EUCLID>(wd, sub_of(wd, cur_sub), uq, qn, ax, ay, az, iw, jq0, hc, band, mism);
                         ++inc_bound;
                         qn = 0;
                         __syncwarp();
@@ -423,6 +449,10 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                 nb = sp.nb;
                 rule = sp.auto_mode ? 1u : (sp.no_self ? 2u : 0u);
                 const float3 p = ldg_point32(sp.a_blk, iw + (uint32_t)lane);
+                if constexpr (EUCLID) {
+                    const float ux = p.x * sp.tc_scale, uy = p.y * sp.tc_scale, uz = p.z * sp.tc_scale;
+                    thr = fmaf(fmaf(uz, uz, fmaf(uy, uy, ux * ux)), sp.tc_qmul, sp.tc_qadd);
+                }
                 ax = pack2(p.x, p.x);
                 ay = pack2(p.y, p.y);
                 az = pack2(p.z, p.z);
@@ -477,8 +507,8 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                             over += (uint32_t)__popc(valid);
                             continue;
                         }
-                        uint32_t um = (diag || ends) ? tc_block<true>(wd, ax, ay, az, sx + 32 * b, valid, hc)
-                                                     : tc_block<false>(wd, ax, ay, az, sx + 32 * b, valid, hc);
+                        uint32_t um = (diag || ends) ? tc_block<EUCLID, true>(wd, ax, ay, az, sx + 32 * b, valid, hc)
+                                                     : tc_block<EUCLID, false>(wd, ax, ay, az, sx + 32 * b, valid, hc);
                         // ---- queue the unsettled pairs; a full batch of 32 is classified at once
                         uint32_t act = __ballot_sync(0xffffffffu, um != 0u);
                         while (act) {
@@ -492,7 +522,7 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                             if (qn >= 32u) {
                                 __syncwarp();
                                 qn -= 32u;
-                                tc_drain(wd, sp, uq + qn, 32u, ax, ay, az, iw, jq0, hc, band, mism);
+                                tc_drain<EUCLID>(wd, sp, uq + qn, 32u, ax, ay, az, iw, jq0, hc, band, mism);
                                 ++inc_bound;
                                 __syncwarp();  // the batch is read before later codes overwrite it
                             }
@@ -505,7 +535,7 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                 if (lane == 0) mbar_arrive(a_empty + ((info & kInfoABuf) ? 1 : 0));
                 if (qn) {
                     __syncwarp();
-                    tc_drain(wd, sub_of(wd, cur_sub), uq, qn, ax, ay, az, iw, jq0, hc, band, mism);
+                    tc_drain<EUCLID>(wd, sub_of(wd, cur_sub), uq, qn, ax, ay, az, iw, jq0, hc, band, mism);
                     ++inc_bound;
                     qn = 0;
                 }
@@ -680,10 +710,10 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
 #pragma unroll
                         for (int k = 0; k < 8; ++k) {
                             uint4* const p = dst + (gg + k / 4) * (kABlock / 16) + 32 * (k % 4) + lane;
-                            p[0] = x[k];
+                            p[0] = EUCLID ? make_uint4(x[k].x, x[k].y, x[k].z, 0u) : x[k];
                             // Y: the halves' two triples exchanged
                             p[kBlk] = make_uint4((x[k].y >> 16) | (x[k].z << 16), (x[k].z >> 16) | (x[k].x << 16),
-                                                 (x[k].x >> 16) | (x[k].y << 16), 0u);
+                                                 (x[k].x >> 16) | (x[k].y << 16), EUCLID ? sp.tc_pad : 0u);
                         }
                     }
                     fence_proxy_async_smem();  // the products read it through the asynchronous proxy
@@ -756,7 +786,7 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
     if (warp == kIssueWarp) tc_dealloc(tmem);
 }
 
-template <bool PREEMPT, bool PRUNE>
+template <bool PREEMPT, bool PRUNE, bool EUCLID>
 cudaError_t launch_tc_t(const WorkDesc& wd_in, const Shape& sh, cudaStream_t stream) {
     WorkDesc wd = wd_in;
     const TcLayout L = tc_layout((int)wd.stages, wd.nedges_max);
@@ -777,7 +807,7 @@ cudaError_t launch_tc_t(const WorkDesc& wd_in, const Shape& sh, cudaStream_t str
     wd.stage_bytes = kStageBytes;
     if (L.total > sh.smem || wd.I != 128u * kGroups || wd.J != kBlk || wd.Jc > 32u * kBlk)
         return cudaErrorInvalidValue;
-    count_tc_kernel<PREEMPT, PRUNE><<<sh.blocks, kThreads, sh.smem, stream>>>(wd);
+    count_tc_kernel<PREEMPT, PRUNE, EUCLID><<<sh.blocks, kThreads, sh.smem, stream>>>(wd);
     return cudaGetLastError();
 }
 
@@ -790,16 +820,23 @@ cudaError_t count_tc_set_smem_limit() {
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     // (the opt-in maximum: the attribute belongs to the kernel, not to a launch)
-    const void* kernels[4] = {(const void*)count_tc_kernel<false, false>, (const void*)count_tc_kernel<true, false>,
-                              (const void*)count_tc_kernel<false, true>, (const void*)count_tc_kernel<true, true>};
+    const void* kernels[6] = {
+        (const void*)count_tc_kernel<false, false, false>, (const void*)count_tc_kernel<true, false, false>,
+        (const void*)count_tc_kernel<false, true, false>,  (const void*)count_tc_kernel<true, true, false>,
+        (const void*)count_tc_kernel<false, false, true>,  (const void*)count_tc_kernel<false, true, true>};
     for (const void* k : kernels)
         if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
     return e;
 }
 
 cudaError_t launch_count_tc(const WorkDesc& wd, const Shape& sh, bool preempt, cudaStream_t stream) {
-    if (wd.prune) return preempt ? launch_tc_t<true, true>(wd, sh, stream) : launch_tc_t<false, true>(wd, sh, stream);
-    return preempt ? launch_tc_t<true, false>(wd, sh, stream) : launch_tc_t<false, false>(wd, sh, stream);
+    if (wd.euclid) {  // (the job server, whose steps preempt, counts angles)
+        if (preempt) return cudaErrorInvalidValue;
+        return wd.prune ? launch_tc_t<false, true, true>(wd, sh, stream) : launch_tc_t<false, false, true>(wd, sh, stream);
+    }
+    if (wd.prune)
+        return preempt ? launch_tc_t<true, true, false>(wd, sh, stream) : launch_tc_t<false, true, false>(wd, sh, stream);
+    return preempt ? launch_tc_t<true, false, false>(wd, sh, stream) : launch_tc_t<false, false, false>(wd, sh, stream);
 }
 
 }  // namespace tpcf

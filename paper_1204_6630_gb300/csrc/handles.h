@@ -76,6 +76,7 @@ struct tpcf_catalog {
     uint32_t* seg_of_block = nullptr;  // device: segment of each kSegAlign-point block (segmented only)
     double eps_max = 0.0;           // bound on | |v|^2 - 1 | over the points (unit-vector catalogs)
     bool euclid = false;            // 3-D catalog: arbitrary finite points (distances, not angles)
+    int tc_exp = 0;                 // 3-D: operand records hold the points times 2^-tc_exp
     double norm_max = 0.0;          // bound on |v| over the points (3-D catalogs)
     cudaStream_t free_stream = nullptr;  // stream-ordered buffers: freed in this stream's order
     bool stream_ordered = false;

@@ -200,15 +200,28 @@ __device__ __forceinline__ uint32_t split16(float v) {  // hi | lo << 16
     return (uint32_t)__half_as_ushort(h) | ((uint32_t)__half_as_ushort(l) << 16);
 }
 
-// Writes point q's FP32 coordinates and operand record into its block.
-__device__ __forceinline__ void put_block(unsigned char* blk, uint32_t q, float x, float y, float z, bool operand) {
+// Writes point q's FP32 coordinates and operand record into its block (3-D: the
+// record of the point times `scale`).
+__device__ __forceinline__ void put_block(unsigned char* blk, uint32_t q, float x, float y, float z, int euclid,
+                                          float scale) {
     unsigned char* b = blk + (size_t)(q / kBlk) * kBlkBytes;
     const uint32_t o = q % kBlk;
-    if (operand) {
-        const uint32_t sx = split16(x), sy = split16(y), sz = split16(z);
-        reinterpret_cast<uint4*>(b)[o] =
-            make_uint4(__byte_perm(sx, sy, 0x5410), __byte_perm(sz, sx, 0x7610), __byte_perm(sy, sz, 0x7632), 0u);
+    uint32_t norm = 0u;
+    float ux = x, uy = y, uz = z;
+    if (euclid) {
+        if (isfinite(x)) {
+            ux *= scale;
+            uy *= scale;
+            uz *= scale;
+            norm = split16(-0.5f * fmaf(uz, uz, fmaf(uy, uy, ux * ux)));
+        } else {  // padding: below every threshold (the screen need not reject it: its pairs are overflow)
+            ux = uy = uz = 0.f;
+            norm = 0xfbffu;  // -65504
+        }
     }
+    const uint32_t sx = split16(ux), sy = split16(uy), sz = split16(uz);
+    reinterpret_cast<uint4*>(b)[o] =
+        make_uint4(__byte_perm(sx, sy, 0x5410), __byte_perm(sz, sx, 0x7610), __byte_perm(sy, sz, 0x7632), norm);
     float* f = reinterpret_cast<float*>(b + kBlkX);
     f[o] = x;
     f[kBlk + o] = y;
@@ -222,7 +235,7 @@ __device__ __forceinline__ void put_block(unsigned char* blk, uint32_t q, float 
 __global__ void prep_gather_kernel(const double* __restrict__ xyz, uint32_t n,
                                    const uint32_t* __restrict__ order, const uint32_t* __restrict__ seg_of_point,
                                    const uint32_t* __restrict__ seg_delta, Point64* out64,
-                                   unsigned char* blk, int euclid) {
+                                   unsigned char* blk, int euclid, const unsigned long long* __restrict__ norm2) {
     const uint32_t p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p >= n) return;
     const uint32_t s = order ? order[p] : p;
@@ -230,7 +243,7 @@ __global__ void prep_gather_kernel(const double* __restrict__ xyz, uint32_t n,
     const double x = xyz[3ull * s], y = xyz[3ull * s + 1], z = xyz[3ull * s + 2];
     const float fx = __double2float_rn(x), fy = __double2float_rn(y), fz = __double2float_rn(z);
     out64[q] = Point64{x, y, z, 0.0};
-    put_block(blk, q, fx, fy, fz, !euclid);
+    put_block(blk, q, fx, fy, fz, euclid, euclid ? ldexpf(1.f, -tc_exponent(*norm2)) : 1.f);
 }
 
 // Padding of 3-D catalogs: (+inf, +inf, +inf).  A pair with a real point has
@@ -244,7 +257,7 @@ __global__ void prep_fill_kernel(Point64* out64, unsigned char* blk, uint32_t n_
     if (p >= n_pad) return;
     const float f = (float)v;
     out64[p] = Point64{v, v, v, 0.0};
-    put_block(blk, p, f, f, f, false);
+    put_block(blk, p, f, f, f, 1, 1.f);
 }
 
 // Bounding sphere of each kCapPoints-point group of a prepared catalog (one
@@ -380,7 +393,7 @@ cudaError_t launch_prepare(const double* xyz_in, uint32_t n, const uint32_t* seg
     }
     if (n > 0) {
         prep_gather_kernel<<<(n + 255) / 256, 256, 0, stream>>>(xyz_in, n, do_sort ? vals : nullptr, seg_of_point,
-                                                               seg_delta, out64, blk, euclid);
+                                                               seg_delta, out64, blk, euclid, eps_word);
         ++nl;
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }

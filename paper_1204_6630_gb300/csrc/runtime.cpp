@@ -793,6 +793,7 @@ int tpcf::catalog_create_impl(tpcf_ctx* ctx, const double* xyz, uint64_t n, int 
     if (euclid) {
         c->eps_max = INFINITY;  // not unit vectors: no chord refinement of angular counts
         c->norm_max = std::sqrt(word * (1.0 + 1e-15)) * (1.0 + 1e-15);  // the device |v|^2 is within 3.4e-16 relative
+        c->tc_exp = tc_exponent(hw[1]);
     } else {
         c->eps_max = word + 4e-16;  // the device sum of squares is within 3.4e-16 of |v|^2
         c->norm_max = 1.0 + 1e-6;
@@ -919,6 +920,30 @@ bool tc_shape_for(tpcf_ctx* ctx, int nedges, uint64_t total_pairs, Shape* sh) {
     return true;
 }
 
+// The tensor-core screen of a 3-D sub-problem: a.b - |b|^2 / 2 in units of
+// 2^(ka + kb) (the operands hold a 2^-ka and b 2^-kb) against the lane's (|a|^2 -
+// S_B) / 2; s = 2^(kb - ka) brings |b|^2 / 2 to those units.  False when the
+// screen could reject next to nothing: its error band is not small beside the
+// range (points far from the origin for their separations) or the catalogs'
+// scales differ too much.  The FP32 kernel, whose value is a difference of
+// coordinates, has no such band (300,000 + 300,000 points in a box of 1000,
+// distances to 50, band 0.03 of the range: 12.2 ms here, 33.5 ms there).
+bool tc_screen_3d(const SubSpec& p, double S_B, SubProblem* sp) {
+    if (p.na == 0 || p.nb == 0) return true;
+    const int ka = p.a->tc_exp, kb = p.b->tc_exp, r = kb - ka;
+    if (r < -kTcMaxRatio || r > kTcMaxRatio) return false;
+    const double guard = std::ldexp(kTcGuard3d, r < 0 ? -r : r), h = std::ldexp(S_B, -(ka + kb) - 1);
+    if (!(8.0 * guard <= h)) return false;
+    if (sp) {
+        sp->tc_scale = (float)std::ldexp(1.0, -ka);
+        sp->tc_qmul = (float)std::ldexp(0.5, -r);
+        sp->tc_qadd = round_down_f32(-(h + guard));
+        const uint32_t f16 = (uint32_t)(15 + r) << 10;  // binary16 2^r
+        sp->tc_pad = f16 | f16 << 16;
+    }
+    return true;
+}
+
 // Items per draw of the tensor-core kernel: one, unless most are pruned away
 // (then up to 32, as long as every SM still draws some 16 times).
 uint32_t tc_draw_batch(tpcf_ctx* ctx, bool prune, uint64_t items) {
@@ -928,11 +953,11 @@ uint32_t tc_draw_batch(tpcf_ctx* ctx, bool prune, uint64_t items) {
 
 // Default shape: 512 x 8 for large problems, smaller i-blocks when the
 // catalogs (or sub-ranges) are small or the per-thread histograms do not fit.
-bool choose_shape(tpcf_ctx* ctx, int mode, int nedges, uint64_t total_pairs, uint64_t max_n, Shape* sh) {
+bool choose_shape(tpcf_ctx* ctx, int mode, bool tc, int nedges, uint64_t total_pairs, uint64_t max_n, Shape* sh) {
     const tpcf_config& cfg = ctx->cfg;
     if (cfg.threads != 0 && cfg.ipt != 0)
         return shape_for(ctx, mode, nedges, cfg.threads, cfg.ipt, cfg.jtile, cfg.stages, sh);
-    if (mode == kModeScreenScalar && cfg.threads == 0 && cfg.ipt == 0 && cfg.jtile == 0 && cfg.stages == 0 &&
+    if (tc && cfg.threads == 0 && cfg.ipt == 0 && cfg.jtile == 0 && cfg.stages == 0 &&
         tc_shape_for(ctx, nedges, total_pairs, sh))
         return true;
     const double per_sm = (double)total_pairs / std::max(1, ctx->num_sms);
@@ -966,7 +991,8 @@ uint64_t range_pairs(const SubProblem& sp, uint64_t lo, uint64_t hi, uint32_t I,
 // caller); acc is the accumulator array (stride acc_stride words per
 // histogram); returns the number of items.
 uint64_t build_work(tpcf_ctx* ctx, const SubSpec* specs, int nsub, const BinsDev* bins_dev, const Shape& sh,
-                    unsigned long long* acc, size_t acc_stride, std::vector<SubProblem>& subs) {
+                    unsigned long long* acc, size_t acc_stride, std::vector<SubProblem>& subs,
+                    const BinsDev* bins_3d = nullptr) {
     const uint32_t I = 32u * (uint32_t)sh.ipt, Jc = (uint32_t)sh.jchunk;
     subs.assign(nsub, SubProblem());
     uint64_t items = 0;
@@ -997,6 +1023,7 @@ uint64_t build_work(tpcf_ctx* ctx, const SubSpec* specs, int nsub, const BinsDev
         sp.row_seg = p.row_seg ? p.row_seg + p.a_off / kSegAlign : nullptr;
         sp.row_stride = (uint32_t)acc_stride;
         sp.no_self = p.no_self ? 1u : 0u;
+        if (bins_3d && sh.tc) (void)tc_screen_3d(p, bins_3d->cos_last, &sp);
         hist_base += (size_t)p.nhist;
         items += sp.n_items;
     }
@@ -1135,7 +1162,9 @@ int run_counts(tpcf_ctx* ctx, const SubSpec* specs, int nsub, const tpcf_bins* b
         max_n = std::max<uint64_t>(max_n, std::max(specs[s].na, specs[s].nb));
     }
     Shape sh;
-    const bool fits = choose_shape(ctx, mode, ne, all_pairs, max_n, &sh);
+    bool tc = mode == kModeScreenScalar || mode == kModeEuclidScreen;
+    for (int s = 0; s < nsub && tc && bins->euclid; ++s) tc = tc_screen_3d(specs[s], bh->cos_last, nullptr);
+    const bool fits = choose_shape(ctx, mode, tc, ne, all_pairs, max_n, &sh);
     if (!fits)
         return ctx->fail(TPCF_EINVAL, "no kernel shape fits (threads=%d ipt=%d jtile=%d)",
                          ctx->cfg.threads, ctx->cfg.ipt, ctx->cfg.jtile);
@@ -1191,7 +1220,8 @@ int run_counts(tpcf_ctx* ctx, const SubSpec* specs, int nsub, const tpcf_bins* b
     memset(&wd, 0, sizeof wd);
     std::vector<SubProblem> subs;
     auto setup = [&](const Shape& shp) -> int {
-        const uint64_t items = build_work(ctx, specs, nsub, bdev, shp, acc, acc_stride, subs);
+        const uint64_t items = build_work(ctx, specs, nsub, bdev, shp, acc, acc_stride, subs,
+                                          bins->euclid ? bh : nullptr);
         if (items > 0xffff0000ull) return TPCF_EOVERFLOW;
         if (use_slot) {
             for (int s2 = 0; s2 < nsub; ++s2) wd.sub[s2] = subs[s2];

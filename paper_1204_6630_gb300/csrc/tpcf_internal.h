@@ -20,14 +20,29 @@ constexpr uint32_t kSegAlign = 256;
 constexpr uint32_t kCapPoints = 128;
 // A catalog's FP32 points and tensor-core operands, in blocks of kBlk points:
 // plane X (16 bytes a point), then the FP32 coordinates as x | y | z arrays.
-// X = (x1, y1, z1, x2, y2, z2, 0, 0) is the binary16 split x = x1 + x2
-// (likewise y, z); zero in 3-D catalogs.
+// X = (x1, y1, z1, x2, y2, z2, n1, n2) is the binary16 split x = x1 + x2
+// (likewise y, z).  Angular catalogs: n1 = n2 = 0.  3-D catalogs: of the point
+// scaled by 2^-k to norm <= 1 (k from the largest norm, tc_exponent), and n1 +
+// n2 splits -|v|^2 / 2; padding has a large negative n1.
 constexpr uint32_t kBlk = 128;
 constexpr uint32_t kBlkX = kBlk * 16;
 constexpr uint32_t kBlkBytes = kBlkX + kBlk * 12;
 // Bound on the distance of the tensor-core screen value from the binary64 dot
 // product (44u, derived in count_tc.cu) with a margin.
 constexpr double kTcGuard = 64.0 * 5.9604644775390625e-08;
+// The same for 3-D counts: bound on the distance of the products' value from
+// (a.b - |b|^2 / 2) scaled, plus that of the lane's threshold, per unit of
+// max(s, 1/s), s the ratio of the catalogs' scales (57u, derived in count_tc.cu).
+constexpr double kTcGuard3d = 128.0 * 5.9604644775390625e-08;
+constexpr int kTcMaxRatio = 10;  // |log2 s| at most: s is a binary16 operand
+
+// Smallest k with 2^k >= sqrt(norm2) (at least -100: its scale is an FP32 number).
+__host__ __device__ inline int tc_exponent(unsigned long long norm2_bits) {
+    const int e = (int)((norm2_bits >> 52) & 0x7ffu) - 1023;  // norm2 < 2^(e + 1)
+    if (norm2_bits == 0ull) return 0;
+    const int k = (e + 2) >> 1;
+    return k < -100 ? -100 : k;
+}
 // 3-D catalogs store their spheres scaled by 2^-64 (exact), so that FP32
 // squares of separations up to 2e28 stay finite.
 constexpr double kCapScale3d = 5.421010862427522e-20;
@@ -103,6 +118,10 @@ struct SubProblem {
     const float4* a_caps;
     const float4* b_caps;
     const float4* b_caps2;  // spheres of B's kPad-point blocks; NULL: the sub-range does not start on one
+    // Tensor-core screen of 3-D counts: a block is kept where a lane's value reaches
+    // fma(|tc_scale a|^2, tc_qmul, tc_qadd); tc_pad: the scales' ratio twice, binary16.
+    float tc_scale, tc_qmul, tc_qadd;
+    uint32_t tc_pad;
 };
 
 constexpr int kMaxInlineSub = 3;
