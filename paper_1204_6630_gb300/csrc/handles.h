@@ -15,6 +15,8 @@
 #include "tpcf.h"
 #include "tpcf_internal.h"
 
+struct tpcf_ctx;
+
 namespace tpcf {
 
 constexpr int kSlots = 16;
@@ -33,8 +35,11 @@ constexpr uint32_t kDefaultWaitUs = 2000000;
 
 // Device allocations of the library; the test hook can make them fail.
 extern std::atomic<int> g_alloc_fail_countdown;
-cudaError_t dev_malloc(void** p, size_t bytes);
-cudaError_t dev_malloc_async(void** p, size_t bytes, cudaStream_t st);
+cudaError_t dev_malloc(tpcf_ctx* ctx, void** p, size_t bytes);
+cudaError_t dev_malloc_async(tpcf_ctx* ctx, void** p, size_t bytes, cudaStream_t st);
+// Stream-ordered scratch from the context's pool.
+cudaError_t pool_malloc(tpcf_ctx* ctx, void** p, size_t bytes, cudaStream_t st);
+constexpr unsigned long long kPoolKeep = 64ull << 20;  // unused bytes the pool keeps
 
 class JobServer;
 
@@ -44,6 +49,7 @@ struct tpcf_ctx {
     tpcf_config cfg;
     int num_sms = 0;
     size_t smem_optin = 0;
+    cudaMemPool_t pool = nullptr;   // stream-ordered allocations (null: the device's default pool)
     std::mutex err_mu;
     std::string last_error;
     struct Slot {

@@ -31,22 +31,31 @@ using namespace tpcf;
 
 std::atomic<int> tpcf::g_alloc_fail_countdown{-1};
 
-cudaError_t tpcf::dev_malloc(void** p, size_t bytes) {
+cudaError_t tpcf::dev_malloc(tpcf_ctx* ctx, void** p, size_t bytes) {
     int c = g_alloc_fail_countdown.load();
     if (c >= 0) {
         if (c == 0) { *p = nullptr; return cudaErrorMemoryAllocation; }
         g_alloc_fail_countdown.fetch_sub(1);
     }
-    return cudaMalloc(p, bytes);
+    cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation && ctx->pool && cudaMemPoolTrimTo(ctx->pool, 0) == cudaSuccess) {
+        e = cudaMalloc(p, bytes);  // with what the pool had kept
+        if (e == cudaSuccess) (void)cudaGetLastError();
+    }
+    return e;
 }
 
-cudaError_t tpcf::dev_malloc_async(void** p, size_t bytes, cudaStream_t st) {
+cudaError_t tpcf::pool_malloc(tpcf_ctx* ctx, void** p, size_t bytes, cudaStream_t st) {
+    return ctx->pool ? cudaMallocFromPoolAsync(p, bytes, ctx->pool, st) : cudaMallocAsync(p, bytes, st);
+}
+
+cudaError_t tpcf::dev_malloc_async(tpcf_ctx* ctx, void** p, size_t bytes, cudaStream_t st) {
     int c = g_alloc_fail_countdown.load();
     if (c >= 0) {
         if (c == 0) { *p = nullptr; return cudaErrorMemoryAllocation; }
         g_alloc_fail_countdown.fetch_sub(1);
     }
-    return cudaMallocAsync(p, bytes, st);
+    return pool_malloc(ctx, p, bytes, st);
 }
 
 int tpcf_ctx::fail(int code, const char* fmt, ...) {
@@ -120,8 +129,24 @@ extern "C" int tpcf_create(tpcf_ctx** out, const tpcf_config* cfg_in) {
     if (cudaGetDeviceProperties(&prop, cfg.device) != cudaSuccess) { delete ctx; return TPCF_ECUDA; }
     ctx->num_sms = prop.multiProcessorCount;
     ctx->smem_optin = prop.sharedMemPerBlockOptin;
+    // Stream-ordered allocations come from a pool of the context's own that keeps up
+    // to kPoolKeep unused bytes mapped: the device's default pool unmaps what is free
+    // at every synchronisation, and mapping it again took 25 us an allocation (4 us
+    // from this pool).
+    cudaMemPoolProps pp;
+    memset(&pp, 0, sizeof pp);
+    pp.allocType = cudaMemAllocationTypePinned;
+    pp.location.type = cudaMemLocationTypeDevice;
+    pp.location.id = cfg.device;
+    unsigned long long keep = kPoolKeep;
+    if (cudaMemPoolCreate(&ctx->pool, &pp) != cudaSuccess) {
+        (void)cudaGetLastError();
+        ctx->pool = nullptr;  // the default pool serves as well
+    } else {
+        (void)cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    }
     for (auto& s : ctx->slots) {
-        if (dev_malloc((void**)&s.dev, kSlotWords * 8) != cudaSuccess ||
+        if (dev_malloc(ctx, (void**)&s.dev, kSlotWords * 8) != cudaSuccess ||
             cudaEventCreateWithFlags(&s.ev, cudaEventDisableTiming) != cudaSuccess) {
             tpcf_destroy(ctx);
             return TPCF_ENOMEM;
@@ -140,6 +165,7 @@ extern "C" int tpcf_destroy(tpcf_ctx* ctx) {
         if (s.dev) cudaFree(s.dev);
         if (s.ev) cudaEventDestroy(s.ev);
     }
+    if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
     delete ctx;
     return TPCF_OK;
 }
@@ -186,9 +212,14 @@ float round_up_f32(double x) {
 double derive_threshold(double t, int* verified) {
     if (t <= 0.0) { *verified = 1; return INFINITY; }
     int64_t lo = dkey(-1.0), hi = dkey(1.0);  // pred(lo) true (t <= pi), pred(hi) false (t > 0)
+    // (further than `sure` from cos t the angle differs from t by 16 ulps and more, at
+    // least: the predicate is known there, and 9 of 10 arc cosines are saved)
+    const double near = cos(t), sure = 32.0 * ((nextafter(t, INFINITY) - t) + 2.3e-16 * fabs(near));
     while (hi - lo > 1) {
         int64_t mid = lo + (hi - lo) / 2;
-        if (angle_at_least(dfromkey(mid), t)) lo = mid; else hi = mid;
+        const double d = dfromkey(mid);
+        const bool at_least = d < near - sure ? true : (d > near + sure ? false : angle_at_least(d, t));
+        if (at_least) lo = mid; else hi = mid;
     }
     const double C = dfromkey(lo);
     const double ulp_t = nextafter(t, INFINITY) - t;
@@ -399,14 +430,14 @@ void build_lut(const std::vector<float>& elo, const std::vector<float>& ehi, int
     const int ne = (int)elo.size();
     const double w = std::ldexp(1.0, q - kLutBits);
     lut.assign(kLutCells, 0);
+    // (elo and ehi do not increase with m, so both sets are the first P or Q edges, and
+    // they only lose edges as e grows)
+    uint32_t P = (uint32_t)ne, Q = (uint32_t)ne;
     for (int k = 0; k < kLutCells; ++k) {
         const double e_min = k == 0 ? -INFINITY : (k - 0.5) * w;
         const double e_max = k == kLutCells - 1 ? INFINITY : (k + 0.5) * w;
-        uint32_t P = 0, Q = 0;
-        for (int m = 0; m < ne; ++m) {
-            P += (e_max < (double)elo[m]);
-            Q += (e_min <= (double)ehi[m]);
-        }
+        while (P > 0 && !(e_max < (double)elo[P - 1])) --P;
+        while (Q > 0 && !(e_min <= (double)ehi[Q - 1])) --Q;
         lut[k] = P | (Q << 16);
     }
 }
@@ -485,7 +516,7 @@ int tpcf::bins_create_impl(tpcf_ctx* ctx, const double* edges, int nedges, cudaS
         bins_destroy_impl(b);
         return ctx->fail(code, "bins: device allocation or copy failed");
     };
-    if ((stream_ordered ? dev_malloc_async(&b->dev_buf, total, st) : dev_malloc(&b->dev_buf, total)) != cudaSuccess)
+    if ((stream_ordered ? dev_malloc_async(ctx, &b->dev_buf, total, st) : dev_malloc(ctx, &b->dev_buf, total)) != cudaSuccess)
         return cleanup(TPCF_ENOMEM);
     unsigned char* base = (unsigned char*)b->dev_buf;
     b->host.cos_thr = (const double*)base;
@@ -586,7 +617,7 @@ static int euclid_set(tpcf_ctx* ctx, tpcf_bins* b, int key, const tpcf::BinsDev*
                      off_zlo = off_c32 + nf16, off_zhi = off_zlo + nf16, off_lut = off_zhi + nf16,
                      off_desc = (off_lut + nl + 255) / 256 * 256, total = off_desc + sizeof(BinsDev);
         tpcf_bins::Set set;
-        if (dev_malloc(&set.dev_buf, total) != cudaSuccess) return ctx->fail(TPCF_ENOMEM, "bins: allocation failed");
+        if (dev_malloc(ctx, &set.dev_buf, total) != cudaSuccess) return ctx->fail(TPCF_ENOMEM, "bins: allocation failed");
         unsigned char* base = (unsigned char*)set.dev_buf;
         memset(&set.host, 0, sizeof set.host);
         set.host.cos_thr = (const double*)base;
@@ -665,10 +696,38 @@ size_t tpcf::catalog_bytes(uint64_t n) {
     return (size_t)n_pad * sizeof(Point64) + (size_t)(n_pad / kBlk) * kBlkBytes;
 }
 
-int tpcf::catalog_create_impl(tpcf_ctx* ctx, const double* xyz, uint64_t n, int where, const uint64_t* offsets,
-                              int nseg, cudaStream_t st, bool stream_ordered, tpcf_catalog** out, bool euclid) {
-    if (!ctx || !out) return TPCF_EINVAL;
-    *out = nullptr;
+// A catalog in preparation: its kernels are queued, their results not yet read.
+struct CatalogPrep {
+    tpcf_catalog* c = nullptr;
+    void* tmp_in = nullptr;
+    unsigned long long* keys = nullptr;
+    uint32_t* vals = nullptr;
+    uint32_t* seg = nullptr;
+    uint32_t* seg_delta = nullptr;
+    unsigned long long* err = nullptr;
+
+    void release(cudaStream_t st) {
+        if (tmp_in) cudaFreeAsync(tmp_in, st);
+        if (keys) cudaFreeAsync(keys, st);
+        if (vals) cudaFreeAsync(vals, st);
+        if (seg) cudaFreeAsync(seg, st);
+        if (seg_delta) cudaFreeAsync(seg_delta, st);
+        if (err) cudaFreeAsync(err, st);
+        cudaStreamSynchronize(st);
+    }
+    int fail(int code, const char* what) {
+        tpcf_ctx* ctx = c->ctx;
+        release(c->free_stream);
+        catalog_destroy_impl(c);
+        c = nullptr;
+        return ctx->fail(code, "catalog: %s", what);
+    }
+};
+
+// First half of a creation: allocation, upload and the preparation kernels.
+// Device inputs are read, and host inputs may be, until catalog_finish.
+static int catalog_begin(tpcf_ctx* ctx, const double* xyz, uint64_t n, int where, const uint64_t* offsets, int nseg,
+                         cudaStream_t st, bool stream_ordered, bool euclid, CatalogPrep& p) {
     if (n > TPCF_MAX_POINTS) return ctx->fail(TPCF_EOVERFLOW, "catalog: %llu points > limit",
                                               (unsigned long long)n);
     if (n > 0 && !xyz) return ctx->fail(TPCF_EINVAL, "catalog: NULL coordinates");
@@ -708,29 +767,14 @@ int tpcf::catalog_create_impl(tpcf_ctx* ctx, const double* xyz, uint64_t n, int 
     uint32_t n_pow2 = 2048;
     while (n_pow2 < n) n_pow2 <<= 1;
 
-    void* tmp_in = nullptr;
-    unsigned long long* keys = nullptr;
-    uint32_t* vals = nullptr;
-    uint32_t* seg = nullptr;
-    uint32_t* seg_delta = nullptr;
-    unsigned long long* err = nullptr;
-    int rc = TPCF_OK;
-    auto release = [&]() {
-        if (tmp_in) cudaFreeAsync(tmp_in, st);
-        if (keys) cudaFreeAsync(keys, st);
-        if (vals) cudaFreeAsync(vals, st);
-        if (seg) cudaFreeAsync(seg, st);
-        if (seg_delta) cudaFreeAsync(seg_delta, st);
-        if (err) cudaFreeAsync(err, st);
-        cudaStreamSynchronize(st);
-    };
-    auto fail_with = [&](int code, const char* what) {
-        release();
-        catalog_destroy_impl(c);
-        return ctx->fail(code, "catalog: %s", what);
-    };
-    auto alloc = [&](void** p, size_t bytes) {
-        return stream_ordered ? dev_malloc_async(p, bytes, st) : dev_malloc(p, bytes);
+    p.c = c;
+    auto fail_with = [&](int code, const char* what) { return p.fail(code, what); };
+    auto pool = [&](void** q, size_t bytes) { return pool_malloc(ctx, q, bytes, st); };
+    void*& tmp_in = p.tmp_in;
+    unsigned long long *&keys = p.keys, *&err = p.err;
+    uint32_t *&vals = p.vals, *&seg = p.seg, *&seg_delta = p.seg_delta;
+    auto alloc = [&](void** q, size_t bytes) {
+        return stream_ordered ? dev_malloc_async(ctx, q, bytes, st) : dev_malloc(ctx, q, bytes);
     };
     // one allocation: binary64 points, blocks, spheres
     const size_t b64 = (size_t)c->n_pad * sizeof(Point64), bblk = (size_t)(c->n_pad / kBlk) * kBlkBytes;
@@ -742,16 +786,15 @@ int tpcf::catalog_create_impl(tpcf_ctx* ctx, const double* xyz, uint64_t n, int 
     c->caps2 = c->caps + c->n_pad / kCapPoints;
     const double* in = xyz;
     if (n > 0 && where == TPCF_HOST) {
-        if (cudaMallocAsync(&tmp_in, n * 24, st) != cudaSuccess)
+        if (pool(&tmp_in, n * 24) != cudaSuccess)
             return fail_with(TPCF_ENOMEM, "staging allocation failed");
         if (cudaMemcpyAsync(tmp_in, xyz, n * 24, cudaMemcpyHostToDevice, st) != cudaSuccess)
             return fail_with(TPCF_ECUDA, "host-to-device copy failed");
         in = (const double*)tmp_in;
     }
     // err: error word, largest |v|^2 or | |v|^2 - 1 |, then the bounding box (3 min, 3 max keys)
-    if (cudaMallocAsync((void**)&err, 64, st) != cudaSuccess ||
-        cudaMallocAsync((void**)&keys, (size_t)n_pow2 * 8, st) != cudaSuccess ||
-        cudaMallocAsync((void**)&vals, (size_t)n_pow2 * 4, st) != cudaSuccess)
+    if (pool((void**)&err, 64) != cudaSuccess || pool((void**)&keys, (size_t)n_pow2 * 8) != cudaSuccess ||
+        pool((void**)&vals, (size_t)n_pow2 * 4) != cudaSuccess)
         return fail_with(TPCF_ENOMEM, "scratch allocation failed");
     if (cudaMemsetAsync(err, 0, 64, st) != cudaSuccess || cudaMemsetAsync(err + 2, 0xff, 24, st) != cudaSuccess)
         return fail_with(TPCF_ECUDA, "memset failed");
@@ -769,8 +812,8 @@ int tpcf::catalog_create_impl(tpcf_ctx* ctx, const double* xyz, uint64_t n, int 
         for (int s = 0; s < nseg; ++s)
             for (uint64_t b = c->seg_start[s] / kSegAlign; b < c->seg_start[s + 1] / kSegAlign; ++b) hb[b] = (uint32_t)s;
         if (alloc((void**)&c->seg_of_block, (size_t)nblk * 4) != cudaSuccess ||
-            cudaMallocAsync((void**)&seg_delta, (size_t)nseg * 4, st) != cudaSuccess ||
-            (n > 0 && cudaMallocAsync((void**)&seg, n * 4, st) != cudaSuccess))
+            pool((void**)&seg_delta, (size_t)nseg * 4) != cudaSuccess ||
+            (n > 0 && pool((void**)&seg, n * 4) != cudaSuccess))
             return fail_with(TPCF_ENOMEM, "segment allocation failed");
         if ((n > 0 && cudaMemcpyAsync(seg, hs.data(), n * 4, cudaMemcpyHostToDevice, st) != cudaSuccess) ||
             cudaMemcpyAsync(seg_delta, hd.data(), (size_t)nseg * 4, cudaMemcpyHostToDevice, st) != cudaSuccess ||
@@ -783,14 +826,21 @@ int tpcf::catalog_create_impl(tpcf_ctx* ctx, const double* xyz, uint64_t n, int 
                                    c->blk, c->caps, c->caps2, c->n_pad, keys, vals, n_pow2, err, err + 1, st, &nl);
     ctx->launches.fetch_add(nl);
     if (e != cudaSuccess) return fail_with(TPCF_ECUDA, cudaGetErrorString(e));
+    return TPCF_OK;
+}
+
+// Second half: waits for the preparation, reads its results and frees its scratch.
+static int catalog_finish(CatalogPrep& p, tpcf_catalog** out) {
+    tpcf_catalog* c = p.c;
+    const cudaStream_t st = c->free_stream;
     unsigned long long hw[2] = {0, 0};
-    if (cudaMemcpyAsync(hw, err, 16, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+    if (cudaMemcpyAsync(hw, p.err, 16, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
         cudaStreamSynchronize(st) != cudaSuccess)
-        return fail_with(TPCF_ECUDA, "preparation failed");
+        return p.fail(TPCF_ECUDA, "preparation failed");
     const unsigned long long herr = hw[0];
     double word;
     memcpy(&word, &hw[1], 8);
-    if (euclid) {
+    if (c->euclid) {
         c->eps_max = INFINITY;  // not unit vectors: no chord refinement of angular counts
         c->norm_max = std::sqrt(word * (1.0 + 1e-15)) * (1.0 + 1e-15);  // the device |v|^2 is within 3.4e-16 relative
         c->tc_exp = tc_exponent(hw[1]);
@@ -799,13 +849,21 @@ int tpcf::catalog_create_impl(tpcf_ctx* ctx, const double* xyz, uint64_t n, int 
         c->norm_max = 1.0 + 1e-6;
     }
     if (herr & kErrBadPoint) {
-        rc = TPCF_EINVAL;
-        return fail_with(rc, euclid ? "a point is not finite"
+        return p.fail(TPCF_EINVAL, c->euclid ? "a point is not finite"
                                     : "a point is not finite or not a unit vector (| |v| - 1 | > 1e-6)");
     }
-    release();
+    p.release(st);
     *out = c;
     return TPCF_OK;
+}
+
+int tpcf::catalog_create_impl(tpcf_ctx* ctx, const double* xyz, uint64_t n, int where, const uint64_t* offsets,
+                              int nseg, cudaStream_t st, bool stream_ordered, tpcf_catalog** out, bool euclid) {
+    if (!ctx || !out) return TPCF_EINVAL;
+    *out = nullptr;
+    CatalogPrep p;
+    const int rc = catalog_begin(ctx, xyz, n, where, offsets, nseg, st, stream_ordered, euclid, p);
+    return rc == TPCF_OK ? catalog_finish(p, out) : rc;
 }
 
 extern "C" int tpcf_catalog_create_segmented(tpcf_ctx* ctx, const double* xyz, uint64_t n, int where,
@@ -1225,7 +1283,7 @@ int run_counts(tpcf_ctx* ctx, const SubSpec* specs, int nsub, const tpcf_bins* b
         acc_stride = (size_t)ne + 1;
         acc_words = (size_t)H * acc_stride + kStatWords;
         const size_t bytes = acc_words * 8 + sub_bytes + tot_bytes;
-        if ((capture ? dev_malloc(&call_buf, bytes) : cudaMallocAsync(&call_buf, bytes, st)) != cudaSuccess)
+        if ((capture ? dev_malloc(ctx, &call_buf, bytes) : pool_malloc(ctx, &call_buf, bytes, st)) != cudaSuccess)
             return ctx->fail(TPCF_ENOMEM, "accumulator allocation failed (%zu bytes)", bytes);
         acc = (unsigned long long*)call_buf;
         stat_w = acc + (size_t)H * acc_stride;
@@ -1861,9 +1919,24 @@ extern "C" int tpcf_correlate(tpcf_ctx* ctx, const double* d_xyz, uint64_t nd, c
     tpcf_catalog *cd = nullptr, *cr = nullptr;
     tpcf_bins* b = nullptr;
     std::vector<uint64_t> hdd(nedges + 1), hdr(nedges + 1), hrr(nedges + 1);
-    int rc = tpcf_catalog_create(ctx, d_xyz, nd, TPCF_HOST, stream, &cd);
-    if (rc == TPCF_OK) rc = tpcf_catalog_create(ctx, r_xyz, nr, TPCF_HOST, stream, &cr);
-    if (rc == TPCF_OK) rc = tpcf_bins_create(ctx, edges, nedges, &b);
+    // Both catalogs are queued before either is waited for, and the bins are derived
+    // on the host meanwhile (1,000 + 2,000 points, 20 bins: 790 us one after the
+    // other, 300 us so; 100,003 + 200,006 points, 50 bins: 6.2 ms, 5.3 ms).  Errors
+    // come in the order data, randoms, bins, as if each were made by itself.
+    const cudaStream_t st0 = (cudaStream_t)stream;
+    CatalogPrep pd, pr;
+    int rc = catalog_begin(ctx, d_xyz, nd, TPCF_HOST, nullptr, 0, st0, true, false, pd);
+    if (rc == TPCF_OK) {
+        int rc_r = catalog_begin(ctx, r_xyz, nr, TPCF_HOST, nullptr, 0, st0, true, false, pr);
+        int rc_b = rc_r == TPCF_OK ? bins_create_impl(ctx, edges, nedges, st0, true, &b) : TPCF_OK;
+        if (rc_r == TPCF_OK) rc_r = catalog_finish(pr, &cr);
+        rc = catalog_finish(pd, &cd);
+        if (rc == TPCF_OK && rc_r == TPCF_ENOMEM)  // (the data's scratch is free now)
+            rc_r = catalog_create_impl(ctx, r_xyz, nr, TPCF_HOST, nullptr, 0, st0, true, &cr);
+        if (rc == TPCF_OK) rc = rc_r;
+        if (rc == TPCF_OK && !b) rc_b = bins_create_impl(ctx, edges, nedges, st0, true, &b);
+        if (rc == TPCF_OK) rc = rc_b;
+    }
     if (rc == TPCF_OK)
         rc = tpcf_count_all(ctx, cd, cr, b, stream, hdd.data(), hdr.data(), hrr.data(), TPCF_HOST, st);
     if (rc == TPCF_OK && w)

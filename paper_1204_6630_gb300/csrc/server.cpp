@@ -136,7 +136,7 @@ class JobServer {
         ok_ = ok_ && cudaHostAlloc((void**)&h_res_, (size_t)slots * res_words * 8, cudaHostAllocDefault) == cudaSuccess;
         for (int k = 0; k < kStepsInFlight && ok_; ++k) {
             ok_ = cudaHostAlloc((void**)&h_stats_[k], (size_t)slots * kStatWords * 8, cudaHostAllocDefault) == cudaSuccess &&
-                  dev_malloc((void**)&d_stats_[k], (size_t)slots * kStatWords * 8) == cudaSuccess &&
+                  dev_malloc(ctx_, (void**)&d_stats_[k], (size_t)slots * kStatWords * 8) == cudaSuccess &&
                   cudaEventCreateWithFlags(&fork_ev_[k], cudaEventDisableTiming) == cudaSuccess;
             for (int q = 0; q < kJobStreams && ok_; ++q)
                 ok_ = cudaStreamCreateWithFlags(&job_streams_[k][q], cudaStreamNonBlocking) == cudaSuccess &&
@@ -415,7 +415,7 @@ class JobServer {
         j.solo = !serving_shape(ctx_, ne, nd * (nd ? nd - 1 : 0) / 2 + nd * nr + nr * (nr ? nr - 1 : 0) / 2, &sh);
         if (!j.solo) {
             const size_t acc_b = 3ull * (ne + 1) * 8, tot_b = 3 * 8;
-            if (dev_malloc_async(&j.dev, acc_b + tot_b, st) != cudaSuccess) return TPCF_ENOMEM;
+            if (dev_malloc_async(ctx_, &j.dev, acc_b + tot_b, st) != cudaSuccess) return TPCF_ENOMEM;
             j.acc = (unsigned long long*)j.dev;
             j.dtot = j.acc + 3 * (ne + 1);
             WorkDesc wd;
