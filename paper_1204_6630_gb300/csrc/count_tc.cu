@@ -29,7 +29,7 @@
 // roundings, the copies, the split), 16 additions of partial sums below 2t at 2u t,
 // 8u t from the threshold (three roundings of |a|^2 / 2s, the copies, the last
 // addition where the screen rejects anything): 57u t in all, kTcGuard3d = 128u.
-// 300,000 + 300,000 points, distances to 0.05 of the box: 12.2 ms (FP32
+// 300,000 + 300,000 points, distances to 0.05 of the box: 11.5 ms (FP32
 // differences on the CUDA cores: 33.5 ms, bound by their nine operations a pair).
 //
 // One CTA per SM, 21 warps:
@@ -120,6 +120,18 @@ __host__ __device__ inline TcLayout tc_layout(int S, int nedges) {
 // ============================================================== tcgen05 wrappers
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
+}
+
+__device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_addr(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
 }
 
 // Allocation of the tensor memory (whole warp; the address goes to the shared word at `dst`).
@@ -405,13 +417,18 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
             inc_bound = 0;
         };
 
+        uint32_t ninfo = 0, njbase = 0, ni0 = 0;
+        bool have = false;  // the stage's record has been read ahead
         while (true) {
-            if (!tc_wait(full + stage, phase, limit, ctl, wd.stats)) {
-                aborted = true;
-                break;
+            uint32_t info = ninfo, jbase = njbase, i0 = ni0;
+            if (!have) {
+                if (!tc_wait(full + stage, phase, limit, ctl, wd.stats)) {
+                    aborted = true;
+                    break;
+                }
+                rec_load(meta + stage * (uint32_t)sizeof(TcMeta), info, jbase, i0);
             }
-            uint32_t info, jbase, i0;
-            rec_load(meta + stage * (uint32_t)sizeof(TcMeta), info, jbase, i0);
+            have = false;
             if (info & kInfoStop) {
                 __syncwarp();
                 if (lane == 0) mbar_arrive(empty + stage);
@@ -472,11 +489,40 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                 uint32_t kept = __any_sync(0xffffffffu, m0 >= thr) ? 1u : 0u;
                 kept |= __any_sync(0xffffffffu, m1 >= thr) ? 2u : 0u;
                 float m2 = tc_row_max32(d_addr + 64u), m3 = tc_row_max32(d_addr + 96u);
+                // The next stage's record meanwhile, if it is there.  (A rejected tile is bound by
+                // this loop's chain of waits, not by a unit: with this and the step below 700,001 x
+                // 1,400,003 points on the sphere to 2 degrees 55.6 -> 50.4 ms, an octant of 1,000,000 +
+                // 1,000,000 to 10 degrees 216.7 -> 213.3 ms; patches where every tile is classified
+                // 49.3 -> 50.4 ms.  Most pruned tiles are classified: 26.2 -> 26.6 ms with both.)
+                if constexpr (!PRUNE) {
+                    const uint32_t ns = stage + 1u == S ? 0u : stage + 1u;
+                    if (__all_sync(0xffffffffu, mbar_test_wait(full + ns, ns ? phase : phase ^ 1u))) {
+                        rec_load(meta + ns * (uint32_t)sizeof(TcMeta), ninfo, njbase, ni0);
+                        have = true;
+                    }
+                }
                 tc_wait_ld(m2, m3);
                 tc_fence_before();
-                if (lane == 0) mbar_arrive(d_free + g);
+                if (PRUNE && lane == 0) mbar_arrive(d_free + g);
                 kept |= __any_sync(0xffffffffu, m2 >= thr) ? 4u : 0u;
                 kept |= __any_sync(0xffffffffu, m3 >= thr) ? 8u : 0u;
+                if constexpr (!PRUNE) {
+                    // a tile with nothing to classify is done: its accumulators and its stage
+                    // are given back in one step
+                    const bool done = kept == 0u && !check && !(info & kInfoLast);
+                    __syncwarp();
+                    if (lane == 0) {
+                        mbar_arrive(d_free + g);
+                        if (done) mbar_arrive(empty + stage);
+                    }
+                    if (done) {
+                        if (++stage == S) {
+                            stage = 0;
+                            phase ^= 1u;
+                        }
+                        continue;
+                    }
+                }
                 // most tiles hold nothing within the range: on to the next
                 if (kept != 0u || check) {
                     // a lane's counter gains at most one per pair of the tile and one per queue batch

@@ -985,7 +985,7 @@ bool tc_shape_for(tpcf_ctx* ctx, int nedges, uint64_t total_pairs, Shape* sh) {
 // range (points far from the origin for their separations) or the catalogs'
 // scales differ too much.  The FP32 kernel, whose value is a difference of
 // coordinates, has no such band (300,000 + 300,000 points in a box of 1000,
-// distances to 50, band 0.03 of the range: 12.2 ms here, 33.5 ms there).
+// distances to 50, band 0.03 of the range: 11.5 ms here, 33.5 ms there).
 bool tc_screen_3d(const SubSpec& p, double S_B, SubProblem* sp) {
     if (p.na == 0 || p.nb == 0) return true;
     const int ka = p.a->tc_exp, kb = p.b->tc_exp, r = kb - ka;
