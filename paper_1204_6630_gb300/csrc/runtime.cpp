@@ -958,7 +958,9 @@ bool shape_for(tpcf_ctx* ctx, int mode, int nedges, int T, int R, int Jreq, int 
 // Shape of the tensor-core kernel (angular screen): 512 i-points x Jc j-points
 // per item.  Jc is the largest that leaves every SM kTcItemsPerSm items, so
 // that the launch's last items are a small part of it; a small problem is cut
-// down to one tile (512 x 128 pairs) per item.  False when the histograms do
+// down to one tile (512 x 128 pairs) per item (auto count of 20,011 points: 147 us
+// with items of 1024, 123 us so; 8,192 + 8,192 points: 101 us, 600 us on the FP32
+// kernel's 128 x 8 shape).  False when the histograms do
 // not leave shared memory for a ring of four stages.
 bool tc_shape_for(tpcf_ctx* ctx, int nedges, uint64_t total_pairs, Shape* sh) {
     constexpr uint64_t kTcItemsPerSm = 8;
@@ -1032,7 +1034,10 @@ bool plain_shape(tpcf_ctx* ctx, int nedges, uint64_t total_pairs, Shape* sh) {
     return false;
 }
 
-// Default shape: 512 x 8 for large problems, smaller i-blocks when the
+// Default shape: the tensor-core kernel wherever its screen applies (octant of
+// 1,000,000 + 1,000,000 points: 213 ms, 296 ms on the FP32 kernel; 512 patches: 56
+// and 63 ms; 8,192 + 8,192 points: 0.10 and 0.60 ms); a caller's own shape is the
+// FP32 kernel's.  There 512 x 8 for large problems, smaller blocks when the
 // catalogs (or sub-ranges) are small or the per-thread histograms do not fit.
 bool choose_shape(tpcf_ctx* ctx, int mode, bool tc, int nedges, uint64_t total_pairs, uint64_t max_n, Shape* sh) {
     const tpcf_config& cfg = ctx->cfg;
@@ -1108,7 +1113,7 @@ uint64_t build_work(tpcf_ctx* ctx, const SubSpec* specs, int nsub, const BinsDev
         sp.row_seg = p.row_seg ? p.row_seg + p.a_off / kSegAlign : nullptr;
         sp.row_stride = (uint32_t)acc_stride;
         sp.no_self = p.no_self ? 1u : 0u;
-        if (bins_3d && sh.tc) (void)tc_screen_3d(p, bins_3d->cos_last, &sp);
+        if (bins_3d && sh.tc && !tc_screen_3d(p, bins_3d->cos_last, &sp)) return ~0ull;  // (never chosen: refused)
         hist_base += (size_t)p.nhist;
         items += sp.n_items;
     }
@@ -1348,7 +1353,8 @@ int run_counts(tpcf_ctx* ctx, const SubSpec* specs, int nsub, const tpcf_bins* b
     // work (about 4 items per warp, the same window of the walk for every shape),
     // keep the one with the least time per pair
     if ((ctx->cfg.flags & TPCF_F_AUTOTUNE) && ctx->cfg.threads == 0 && ctx->cfg.jtile == 0) {
-        const std::array<int, 5> key{mode, ne, nsub, ilog2_u64(all_pairs + 1), ilog2_u64(max_n + 1)};
+        // (tc: a shape of the tensor-core kernel is not for 3-D points that its screen refuses)
+        const std::array<int, 5> key{mode + (tc ? 16 : 0), ne, nsub, ilog2_u64(all_pairs + 1), ilog2_u64(max_n + 1)};
         std::lock_guard<std::mutex> tl(ctx->tune_mu);
         auto it = ctx->tuned.find(key);
         if (it != ctx->tuned.end()) {
@@ -1371,6 +1377,7 @@ int run_counts(tpcf_ctx* ctx, const SubSpec* specs, int nsub, const tpcf_bins* b
                     if (cand_t[ti] == 0 ? (!tc_fits || ji > 0)
                                         : !shape_for(ctx, mode, ne, cand_t[ti], 8, cand_j[ji], 0, &c))
                         continue;
+                    if (mode == kModePlainFP64) plain_chunk(all_pairs, &c);
                     if (setup(c) != TPCF_OK) continue;
                     const uint64_t window = (uint64_t)ctx->num_sms * (c.tc ? 1ull : (uint64_t)(c.threads / 32)) * 4;
                     if (wd.item_hi - wd.item_lo > window) wd.item_hi = wd.item_lo + window;

@@ -86,3 +86,19 @@ def test_range_ends(T, hi):
     d = synth.box_clustered(700, 8, 0.01, 1.0, 3) - 0.5
     r = np.concatenate([synth.box_points(600, 1.0, 4) - 0.5, d[:50], d[:50] + 1e-8])
     _check(T, d, r, np.linspace(0.0, hi, 8))
+
+
+@pytest.mark.gpu
+def test_autotuned_shapes(T):
+    """A shape tuned on points near the origin is not used for points the screen refuses."""
+    d, r = synth.box_clustered(3000, 8, 0.02, 1.0, 5), synth.box_points(3100, 1.0, 6)
+    edges = synth.log_edges_r(0.005, 0.3, 9)
+    with T.Context(flags=T.TPCF_F_AUTOTUNE) as ctx:
+        for offset in (0.0, 5e5, 0.0):
+            a, b = d + offset, r + offset
+            got = ctx.count_all(ctx.catalog3d(a), ctx.catalog3d(b), ctx.bins3d(edges))
+            want = (oracle.count_auto(a, edges, THREADS, euclid=True),
+                    oracle.count_cross(a, b, edges, THREADS, euclid=True),
+                    oracle.count_auto(b, edges, THREADS, euclid=True))
+            for g, o in zip(got, want):
+                np.testing.assert_array_equal(g, o)
