@@ -11,12 +11,13 @@ copies), bin thresholds, one fused DD/DR/RR counting launch, the finalize
 kernels, and the Landy-Szalay estimate.  `value` is pairs/s over the K timed
 steps (CUDA events, max over ranks).  `e2e` repeats the step through the
 host-array call tpcf_correlate with the catalogs in pinned host memory (copies
-included).  The roofline is that of the counting kernel: 3 FP32 pipe lane
-operations per pair (3 FFMA, the range offset folded into the first), counted
-as 6 flops, against the FP32 peak derived from the device's SM count x 128
-lanes x 2 flops x the maximum SM clock (nvidia-smi), with the fraction at the
-clock sampled under load and against the measured FMA-chain throughput
-(tpcf_fp32_peak) beside it.  The line also carries the all-binary64 kernel on
+included).  The roofline is that of the tensor-core screen, which evaluates
+every pair: a K = 16 product of binary16 splits, 32 flops, against the measured
+16-bit matrix throughput of MEASURED_PEAKS.json (1900 TFLOP/s if absent).
+Beside it stands the same rate as FP32 dot products (3 FMAs, 6 flops) against
+the FP32 peak derived from the device's SM count x 128 lanes x 2 flops x the
+maximum SM clock (nvidia-smi), at the clock sampled under load, and against
+the measured FMA-chain throughput (tpcf_fp32_peak).  The line also carries the all-binary64 kernel on
 the same catalogs (`fp64_plain`) and one launch with spatial pruning
 (`pruning`, the opt-in TPCF_F_PRUNE flag: same histograms, pairs covered per
 second); neither is the brute-force headline.  After the timed region, compact
@@ -66,7 +67,8 @@ sys.path.insert(0, ROOT)
 
 METRIC = "pairs/s (DD+DR+RR)"
 UNIT = "pairs/s"
-FLOPS_PER_PAIR = 6            # 3 FP32 pipe lane-ops (3 FFMA), FMA convention
+FLOPS_PER_PAIR = 6            # the dot product: 3 FMAs, FMA convention
+TENSOR_FLOPS_PER_PAIR = 32    # the screen's K = 16 product of binary16 splits
 L2_FLUSH_BYTES = 256 << 20
 
 
@@ -169,6 +171,19 @@ def roofline_peaks(local: int, clocks: dict):
     derived = sms * 128 * 2 * max_mhz * 1e6 / 1e12
     at_clock = sms * 128 * 2 * med_mhz * 1e6 / 1e12
     return sms, max_mhz, med_mhz, derived, at_clock
+
+
+def tensor_roofline(pairs: float, ms: float) -> dict:
+    """Rate of the tensor-core screen against the measured 16-bit matrix throughput."""
+    peak, src = 1900.0, "fallback (no MEASURED_PEAKS.json)"
+    try:
+        with open(os.path.join(ROOT, "MEASURED_PEAKS.json")) as fh:
+            peak, src = float(json.load(fh)["bf16_tflops"]), "MEASURED_PEAKS.json bf16_tflops"
+    except (OSError, ValueError, KeyError):
+        pass
+    achieved = pairs * TENSOR_FLOPS_PER_PAIR / (ms / 1e3) / 1e12
+    return {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
+            "peak_source": src}
 
 
 def run_reference(args):
@@ -382,7 +397,7 @@ def run_gpu(args):
         try:
             import hashlib
             rec = json.load(open(prof))
-            src = os.path.join(ROOT, "paper_1204_6630_gb300", "csrc", "count.cu")
+            src = os.path.join(ROOT, "paper_1204_6630_gb300", "csrc", "count_tc.cu")
             sha = hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
             if rec.get("kernel_source_sha256_16") == sha and args.n == 1_000_000:
                 traffic = rec.get("dram_bytes_per_launch")
@@ -399,17 +414,17 @@ def run_gpu(args):
         "metric": METRIC, "value": pairs * args.steps / (elapsed_ms / 1e3), "unit": UNIT,
         "n_gpus": world, "steps": args.steps, "warmup": args.warmup, "ms_per_step": elapsed_ms / args.steps,
         "higher_is_better": True, "scaling": "strong", "vs_baseline": None,
-        "dtype": "f32", "precision": "FP32 screen + binary64 guard-band recheck, uint64 counts",
+        "dtype": "f32", "precision": "binary16-split tensor-core rejection, FP32 screen, binary64 guard-band recheck, uint64 counts",
         "data": "synthetic", "config": cfg,
-        "roofline": {"bound": "alu", "achieved": achieved, "peak": peak_derived, "unit": "TFLOP/s",
-                     "frac": achieved / peak_derived, "traffic": traffic,
-                     "kernel": "count_kernel (screen, fused DD/DR/RR)",
-                     "kernel_ms": statistics.mean(kernel_ms),
-                     "peak_source": f"derived: {sms} SMs (device) x 128 FP32 lanes x 2 flops x {max_mhz:.0f} MHz "
-                                    "(maximum SM clock, nvidia-smi); MEASURED_PEAKS.json has no FP32 entry",
-                     "peak_at_sampled_clock": {"value": peak_clock, "sm_mhz": med_mhz,
-                                               "frac": achieved / peak_clock},
-                     "peak_measured": peak_meas},
+        "roofline": {**tensor_roofline(st["pairs"], kern_s * 1e3), "traffic": traffic,
+                     "kernel": "count_tc_kernel (fused DD/DR/RR)", "kernel_ms": statistics.mean(kernel_ms),
+                     "fp32_equivalent": {
+                         "achieved": achieved, "peak": peak_derived, "frac": achieved / peak_derived,
+                         "peak_source": f"derived: {sms} SMs (device) x 128 FP32 lanes x 2 flops x {max_mhz:.0f} MHz "
+                                        "(maximum SM clock, nvidia-smi); MEASURED_PEAKS.json has no FP32 entry",
+                         "peak_at_sampled_clock": {"value": peak_clock, "sm_mhz": med_mhz,
+                                                   "frac": achieved / peak_clock},
+                         "peak_measured": peak_meas}},
         "band": {"pairs": st["band_pairs"], "fraction": st["band_pairs"] / max(1, st["pairs"]),
                  "fp32_mismatch": st["band_mismatch"]},
         "fp64_plain": fp64,
@@ -440,7 +455,8 @@ def extras(peak_meas) -> dict:
     return {
         "large": {"workload": lg["config"]["workload"], "pairs": lg["config"]["pairs_per_step"],
                   "kernel_ms": lg["ms_per_step"], "pairs_per_s": lg["value"],
-                  "frac": lg["roofline"]["frac"], "frac_of_measured": lg["roofline"]["frac_of_measured"],
+                  "frac": lg["roofline"]["frac"],
+                  "fp32_equivalent_frac": lg["roofline"]["fp32_equivalent"]["frac"],
                   "band_pairs": lg["band"]["pairs"],
                   "subsample_points": lg["subsample_parity"]["points_per_catalog"],
                   "subsample_identical_to_oracle": lg["subsample_parity"]["identical_to_oracle"],
@@ -754,11 +770,11 @@ def large_record(steps: int, warmup: int, sub: int, prune: bool = True, peak_mea
         "config": {"workload": "sphere_large: N_D=4,000,000 (4096 clusters sigma 0.1 deg), N_R=8,000,000 uniform, "
                                "full sphere, 80 log bins 0.005-2 deg, seed 0", "pairs_per_step": pairs,
                    "timed": "fused DD/DR/RR counting launch + finalize on resident catalogs (CUDA events)"},
-        "roofline": {"bound": "alu", "achieved": ach, "peak": peak_derived, "unit": "TFLOP/s",
-                     "frac": ach / peak_derived,
-                     "peak_source": f"derived: {sms} SMs x 128 FP32 lanes x 2 flops x {max_mhz:.0f} MHz",
-                     "peak_measured": peak_meas,
-                     "frac_of_measured": ach / peak_meas if peak_meas else None},
+        "roofline": {**tensor_roofline(pairs, km),
+                     "fp32_equivalent": {"achieved": ach, "peak": peak_derived, "frac": ach / peak_derived,
+                                         "peak_source": f"derived: {sms} SMs x 128 FP32 lanes x 2 flops x {max_mhz:.0f} MHz",
+                                         "peak_measured": peak_meas,
+                                         "frac_of_measured": ach / peak_meas if peak_meas else None}},
         "band": {"pairs": st["band_pairs"], "fraction": st["band_pairs"] / pairs,
                  "fp32_mismatch": st["band_mismatch"]},
         "subsample_parity": {"points_per_catalog": sub, "identical_to_oracle": same,
@@ -807,16 +823,16 @@ def run_box3d(args):
             oracle.count_auto(rs, w.edges, cores, euclid=True))
     same = all(np.array_equal(a, c) for a, c in zip(sub, want))
     km = statistics.mean(kms)
-    lane_ops = 6  # 3 FADD + 3 FFMA per pair on the FP32 pipe
+    lane_ops = 6  # 3 FADD + 3 FFMA per pair, as on the FP32 pipe (the screen runs on the tensor cores)
     peak = 152 * 128 * 2.07e9
     print(json.dumps({
         "mode": "box3d", "metric": METRIC, "value": pairs / km * 1e3, "unit": UNIT, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": km, "higher_is_better": True, "dtype": "f32", "data": "synthetic",
         "config": {"workload": f"box: N_D={nd:,} clustered (4096 clusters sigma 2), N_R={nr:,} uniform, side 1000, "
                                "30 log distance bins 0.5-50, seed 0", "pairs_per_step": pairs},
-        "roofline": {"bound": "alu", "lane_ops_per_pair": lane_ops,
-                     "frac": pairs / (km / 1e3) * lane_ops / peak,
-                     "peak": "152 SMs x 128 FP32 lanes x 2.07 GHz lane-ops/s (derived)"},
+        "roofline": {**tensor_roofline(pairs, km),
+                     "fp32_equivalent": {"lane_ops_per_pair": lane_ops, "frac": pairs / (km / 1e3) * lane_ops / peak,
+                                         "peak": "152 SMs x 128 FP32 lanes x 2.07 GHz lane-ops/s (derived)"}},
         "band": {"pairs": st["band_pairs"], "fraction": st["band_pairs"] / pairs},
         "subsample_parity": {"points_per_catalog": args.sub, "identical_to_oracle": same},
         "clocks": clocks.summary()}))

@@ -91,7 +91,7 @@ extern "C" {
 #define TPCF_F_AUTOTUNE 0x8u         /* the first counting call of a workload class times every kernel
                                         shape that fits and the context keeps the fastest */
 #define TPCF_F_PRUNE 0x10u           /* spatial pruning: each counting launch skips the blocks of
-                                        (one warp's i-points x 128 j-points) whose bounding spheres
+                                        (128 or one warp's i-points x 128 j-points) whose bounding spheres
                                         are provably farther apart than the last edge (every pair
                                         in them is overflow); counts are unchanged, the skipped pair
                                         slots are reported in tpcf_stats.pruned_pairs.  Screen
@@ -132,7 +132,9 @@ typedef struct tpcf_config {
     uint64_t hbm_budget_bytes; /* device memory the job server may hold for catalogs; 0 -> 120 GB
                                   capped at 80% of free memory */
     uint32_t flags;            /* TPCF_F_* */
-    int threads;               /* kernel shape override: threads per block (0 = tuned default) */
+    int threads;               /* kernel shape override: threads per block of the FP32 kernel; any of
+                                  the four set selects that kernel (0 = tuned default: the
+                                  tensor-core kernel where its screen applies) */
     int ipt;                   /* kernel shape override: i-points per thread (0 = default) */
     int jtile;                 /* kernel shape override: j-points per shared-memory tile of a warp's
                                   ring, a multiple of 128 dividing 4096 (0 = default) */
@@ -154,8 +156,8 @@ typedef struct tpcf_stats {
     uint32_t device_error;  /* device error word of the call (0 = none) */
     uint32_t launches;      /* kernels launched by the call */
     double kernel_ms;       /* device time of the counting launch (CUDA events) */
-    uint64_t pruned_pairs;  /* pair slots skipped by TPCF_F_PRUNE (blocks of 32 * ipt i-points x
-                               128 j-points, padding and masked slots included; 0 without it) */
+    uint64_t pruned_pairs;  /* pair slots skipped by TPCF_F_PRUNE (blocks of 128, or 32 * ipt, i-points
+                               x 128 j-points, padding and masked slots included; 0 without it) */
 } tpcf_stats;
 
 /* ------------------------------------------------------------------ misc */
@@ -172,8 +174,8 @@ uint64_t tpcf_kernel_launches(const tpcf_ctx *ctx);
 
 /* ------------------------------------------------------------------ measurement
  * tpcf_fp32_peak: the measured FP32 fused multiply-add throughput of `device`
- * in TFLOP/s (2 flops per FMA), the denominator of the counting kernel's
- * roofline.  16 independent FMA chains per thread, 4 blocks of 512 threads per
+ * in TFLOP/s (2 flops per FMA), the unit in which the benchmark gives the pair
+ * rate.  16 independent FMA chains per thread, 4 blocks of 512 threads per
  * SM, best of 5 timed launches (CUDA events) after a warm-up launch; packed = 0
  * issues fma.rn.f32, packed = 1 fma.rn.f32x2 (two FMAs per instruction).
  * Synchronous (about 0.1 s); allocates nothing; changes no device setting.
@@ -383,15 +385,15 @@ int tpcf_correlate(tpcf_ctx *ctx, const double *d_xyz, uint64_t nd, const double
  * Continuous batching: the counting work of all admitted jobs runs as a
  * sequence of steps, two in flight on two streams, so that the blocks of one
  * start on the SMs the other's blocks leave.  Small jobs (at most 2e10 pairs)
- * share steps: one launch of a multi-job kernel over all of their work items,
- * each job with its own bins and histograms.  A large job runs in
- * preemptible steps of the one-job kernel over all of its remaining work; a
+ * share steps: a launch for each over all of its work items, side by side on
+ * several streams.  A large job runs in preemptible steps over all of its
+ * remaining work; a
  * small job that becomes ready makes the running large step stop drawing new
  * items (its warps finish the items they hold), runs, and the large job
  * continues where it stopped.  A job admitted while steps run joins the next
  * step.  Each job's histograms equal those of a lone tpcf_correlate
  * call (every pair is counted once, whatever step it lands in).  Jobs with
- * more edges than the multi-job kernel's shared memory holds are counted
+ * more edges than the serving shape's shared memory holds are counted
  * alone by their preparation worker.  Job buffers are allocated and freed in
  * stream order (no device-wide synchronization between jobs).
  * Validation as tpcf_submit returns: TPCF_EINVAL for NULL arrays, bad edges or
