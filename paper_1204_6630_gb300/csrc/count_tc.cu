@@ -380,7 +380,7 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
         }
         for (int k = 0; k < 2; ++k) {
             mbar_init(a_full + k, 1);
-            mbar_init(a_empty + k, kWorkWarps);
+            mbar_init(a_empty + k, kWorkWarps + kGroups);
         }
         for (int g = 0; g < kGroups; ++g) {
             mbar_init(d_full + g, 1);
@@ -644,7 +644,12 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                 any = true;
             }
             __syncwarp();
-            if (lane == 0) mbar_arrive(empty + stage);
+            if (lane == 0) {
+                // (an issuer whose group has no tile in the item gives the operand back too: it has
+                // waited for it, by parity, and must not see the buffer filled twice meanwhile)
+                if (info & kInfoLast) mbar_arrive(a_empty + buf);
+                mbar_arrive(empty + stage);
+            }
             if (++stage == S) {
                 stage = 0;
                 phase ^= 1u;
