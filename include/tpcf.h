@@ -142,7 +142,8 @@ typedef struct tpcf_config {
                                   2..16 (0 = default) */
     uint32_t shard_index;      /* multi-process split of the pair tiles: this process's index */
     uint32_t shard_count;      /* number of shards (0 or 1 = no split); histograms of all
-                                  shards sum to the unsplit result exactly */
+                                  shards sum to the unsplit result exactly (shards of one
+                                  configuration, counting the same catalogs and bins) */
     uint32_t wait_timeout_us;  /* limit of every device-side wait; 0 -> 2,000,000 us */
     int server_workers;        /* job server: jobs admitted at once (slots: catalogs resident on the
                                   device, work in the running steps) (0 -> 32) */

@@ -922,6 +922,13 @@ int kernel_mode(const tpcf_config& cfg, bool euclid) {
     return euclid ? kModeEuclidScreen : kModeScreenScalar;
 }
 
+// SMs that items are laid out for.  Shards take ranges of one list of items, which all
+// must cut alike whatever their GPUs: a fixed number stands for the SMs there.
+uint64_t plan_sms(const tpcf_ctx* ctx) {
+    constexpr uint64_t kShardSms = 152;
+    return ctx->cfg.shard_count > 1 ? kShardSms : (uint64_t)ctx->num_sms;
+}
+
 // Shape for T threads x R i-points, j-tile J (0: default) and S stages per
 // warp (0: default); false when it does not fit shared memory.  Every warp
 // works on items of its own 32 R i-points x Jc = 4096 j-points, streamed in
@@ -968,7 +975,7 @@ bool tc_shape_for(tpcf_ctx* ctx, int nedges, uint64_t total_pairs, Shape* sh) {
     while (S >= 4 && count_tc_smem_bytes(S, nedges) > ctx->smem_optin) S -= 2;
     if (S < 4) return false;
     int Jc = 32 * (int)kBlk;
-    while (Jc > (int)kBlk && total_pairs / (512ull * (uint64_t)Jc) < kTcItemsPerSm * (uint64_t)ctx->num_sms) Jc /= 2;
+    while (Jc > (int)kBlk && total_pairs / (512ull * (uint64_t)Jc) < kTcItemsPerSm * plan_sms(ctx)) Jc /= 2;
     sh->threads = 512;
     sh->ipt = 16;
     sh->jtile = (int)kBlk;
@@ -1017,18 +1024,18 @@ uint32_t tc_draw_batch(tpcf_ctx* ctx, bool prune, uint64_t items) {
 // eight.  30,011 + 30,011 points on an octant: 128 threads 26.0 ms with chunks of
 // 4096, 25.4 ms with small ones, 512 threads 17.5 ms; 2,000 + 2,000: 4.7 ms with
 // chunks of 4096, 1.0 ms (128 threads) and 1.1 ms (512) with small ones.
-void plain_chunk(uint64_t total_pairs, Shape* sh) {
+void plain_chunk(tpcf_ctx* ctx, uint64_t total_pairs, Shape* sh) {
     constexpr uint64_t kPlainItems = 8;
-    const uint64_t warps = (uint64_t)sh->blocks * (uint64_t)(sh->threads / 32), I = 32ull * (uint64_t)sh->ipt;
+    const uint64_t warps = plan_sms(ctx) * (uint64_t)(sh->threads / 32), I = 32ull * (uint64_t)sh->ipt;
     while (sh->jchunk > sh->jtile && total_pairs / (I * (uint64_t)sh->jchunk) < kPlainItems * warps) sh->jchunk /= 2;
 }
 bool plain_shape(tpcf_ctx* ctx, int nedges, uint64_t total_pairs, Shape* sh) {
     const tpcf_config& cfg = ctx->cfg;
     const uint64_t items = total_pairs / (256ull * 128ull);  // 8 i-points a thread, one tile of j-points
     for (int threads = 512; threads >= 128; threads /= 2) {
-        if (threads > 128 && items < (uint64_t)ctx->num_sms * (uint64_t)(threads / 32)) continue;
+        if (threads > 128 && items < plan_sms(ctx) * (uint64_t)(threads / 32)) continue;
         if (!shape_for(ctx, kModePlainFP64, nedges, threads, 8, cfg.jtile, cfg.stages, sh)) continue;
-        plain_chunk(total_pairs, sh);
+        plain_chunk(ctx, total_pairs, sh);
         return true;
     }
     return false;
@@ -1043,7 +1050,7 @@ bool choose_shape(tpcf_ctx* ctx, int mode, bool tc, int nedges, uint64_t total_p
     const tpcf_config& cfg = ctx->cfg;
     if (cfg.threads != 0 && cfg.ipt != 0) {
         const bool r = shape_for(ctx, mode, nedges, cfg.threads, cfg.ipt, cfg.jtile, cfg.stages, sh);
-        if (r && mode == kModePlainFP64) plain_chunk(total_pairs, sh);
+        if (r && mode == kModePlainFP64) plain_chunk(ctx, total_pairs, sh);
         return r;
     }
     if (tc && cfg.threads == 0 && cfg.ipt == 0 && cfg.jtile == 0 && cfg.stages == 0 &&
@@ -1351,14 +1358,23 @@ int run_counts(tpcf_ctx* ctx, const SubSpec* specs, int nsub, const tpcf_bins* b
 
     // ---- optional autotuning: time every fitting shape on a bounded window of the
     // work (about 4 items per warp, the same window of the walk for every shape),
-    // keep the one with the least time per pair
+    // keep the one with the least time per pair.  Shards of one count take ranges of the
+    // same items: there the timing chooses among threads and tiles, not among items.
+    const Shape cut = sh;
+    auto same_items = [&](Shape* c) {
+        if (ctx->cfg.shard_count <= 1) return true;
+        if (c->tc != cut.tc || c->ipt != cut.ipt || cut.jchunk % c->jtile != 0) return false;
+        c->jchunk = cut.jchunk;
+        return true;
+    };
     if ((ctx->cfg.flags & TPCF_F_AUTOTUNE) && ctx->cfg.threads == 0 && ctx->cfg.jtile == 0) {
         // (tc: a shape of the tensor-core kernel is not for 3-D points that its screen refuses)
         const std::array<int, 5> key{mode + (tc ? 16 : 0), ne, nsub, ilog2_u64(all_pairs + 1), ilog2_u64(max_n + 1)};
         std::lock_guard<std::mutex> tl(ctx->tune_mu);
         auto it = ctx->tuned.find(key);
         if (it != ctx->tuned.end()) {
-            sh = it->second;
+            Shape c = it->second;
+            if (same_items(&c)) sh = c;
         } else {
             // (the FP32 kernel's nine shapes; the tensor-core kernel where it can run)
             const int cand_t[4] = {128, 256, 512, 0};
@@ -1377,7 +1393,8 @@ int run_counts(tpcf_ctx* ctx, const SubSpec* specs, int nsub, const tpcf_bins* b
                     if (cand_t[ti] == 0 ? (!tc_fits || ji > 0)
                                         : !shape_for(ctx, mode, ne, cand_t[ti], 8, cand_j[ji], 0, &c))
                         continue;
-                    if (mode == kModePlainFP64) plain_chunk(all_pairs, &c);
+                    if (mode == kModePlainFP64) plain_chunk(ctx, all_pairs, &c);
+                    if (!same_items(&c)) continue;
                     if (setup(c) != TPCF_OK) continue;
                     const uint64_t window = (uint64_t)ctx->num_sms * (c.tc ? 1ull : (uint64_t)(c.threads / 32)) * 4;
                     if (wd.item_hi - wd.item_lo > window) wd.item_hi = wd.item_lo + window;

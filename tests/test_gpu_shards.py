@@ -50,3 +50,18 @@ def test_shards_against_the_oracle(T):
                      oracle.count_auto(w.rand, w.edges, THREADS)])
     parts = [_count(T, w.data, w.rand, w.edges, threads=128, ipt=8, shard_index=s, shard_count=3)[0] for s in range(3)]
     np.testing.assert_array_equal(np.sum(parts, axis=0, dtype=np.uint64), want)
+
+
+def test_shards_of_autotuned_contexts_cut_the_work_alike(T):
+    """A context that tuned a smaller problem of the same class first (whose items are
+    smaller) still takes the same items as the other shards' contexts."""
+    edges = synth.log_edges(0.02, 6.0, 30)
+    small, x = synth.randoms(17000, seed=23), synth.clustered(20000, 64, 0.3, seed=24)
+    parts = []
+    for s in range(2):
+        with T.Context(flags=T.TPCF_F_AUTOTUNE, shard_index=s, shard_count=2) as ctx:
+            b = ctx.bins(edges)
+            if s == 0:
+                ctx.count_auto(ctx.catalog(small), b)
+            parts.append(ctx.count_auto(ctx.catalog(x), b))
+    np.testing.assert_array_equal(parts[0] + parts[1], oracle.count_auto(x, edges, THREADS))
