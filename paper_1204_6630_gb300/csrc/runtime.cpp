@@ -1357,8 +1357,7 @@ int run_counts(tpcf_ctx* ctx, const SubSpec* specs, int nsub, const tpcf_bins* b
     };
 
     // ---- optional autotuning: time every fitting shape on a bounded window of the
-    // work (about 4 items per warp, the same window of the walk for every shape),
-    // keep the one with the least time per pair.  Shards of one count take ranges of the
+    // work (the first items of the walk, about 4 draws per drawing warp), keep the one with the least time per pair.  Shards of one count take ranges of the
     // same items: there the timing chooses among threads and tiles, not among items.
     const Shape cut = sh;
     auto same_items = [&](Shape* c) {
@@ -1396,7 +1395,9 @@ int run_counts(tpcf_ctx* ctx, const SubSpec* specs, int nsub, const tpcf_bins* b
                     if (mode == kModePlainFP64) plain_chunk(ctx, all_pairs, &c);
                     if (!same_items(&c)) continue;
                     if (setup(c) != TPCF_OK) continue;
-                    const uint64_t window = (uint64_t)ctx->num_sms * (c.tc ? 1ull : (uint64_t)(c.threads / 32)) * 4;
+                    // (tensor-core kernel: an SM draws draw_batch items at a time)
+                    const uint64_t per_sm = c.tc ? (uint64_t)wd.draw_batch : (uint64_t)(c.threads / 32);
+                    const uint64_t window = (uint64_t)ctx->num_sms * per_sm * 4;
                     if (wd.item_hi - wd.item_lo > window) wd.item_hi = wd.item_lo + window;
                     uint64_t wpairs = 0;
                     for (int s2 = 0; s2 < nsub; ++s2)

@@ -197,3 +197,18 @@ def test_server_jobs_with_pruning(T):
             np.testing.assert_array_equal(res["dd"], dd)
             np.testing.assert_array_equal(res["dr"], dr)
             np.testing.assert_array_equal(res["rr"], rr)
+
+
+def test_autotuning_times_pruned_launches_as_they_run(T):
+    """The tuned context keeps the default (tensor-core) kernel, several times faster here:
+    its candidate is timed on as many draws per SM as a real launch makes.  The kernels
+    differ in the size of the blocks they skip, so the skipped slots tell which one ran."""
+    d = synth.clustered(400_000, 64, 0.3, synth.Footprint("sphere"), seed=14)
+    r = synth.randoms(800_000, synth.Footprint("sphere"), seed=15)
+    edges = synth.log_edges(0.01, 2.0, 30)
+    want, st0 = run(T, d, r, edges, True)
+    with T.Context(flags=T.TPCF_F_PRUNE | T.TPCF_F_AUTOTUNE) as ctx:
+        got, st = ctx.count_all(ctx.catalog(d), ctx.catalog(r), ctx.bins(edges), stats=True)
+    for g, o in zip(got, want):
+        np.testing.assert_array_equal(g, o)
+    assert st["pruned_pairs"] == st0["pruned_pairs"]
