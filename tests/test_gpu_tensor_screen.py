@@ -82,3 +82,12 @@ def test_values_at_the_threshold(T):
     b = np.cos(ang)[:, None] * a + np.sin(ang)[:, None] * t
     b /= np.linalg.norm(b, axis=1)[:, None]
     _check(T, a, b, np.linspace(0.0, tb, 9))
+
+
+@pytest.mark.parametrize("nedges", [110, 111, 121, 122, 132, 133])
+def test_ring_depths(T, nedges):
+    """Histograms take shared memory from the ring of tiles: eight stages up to 110 edges, six up
+    to 121, four up to 132, beyond that the FP32 kernel; many more tiles than stages in each."""
+    d = synth.clustered(2003, 8, 0.5, seed=nedges)
+    r = synth.randoms(9001, seed=nedges + 1)
+    _check(T, d, r, synth.linear_edges(0.0, 20.0, nedges - 1))
