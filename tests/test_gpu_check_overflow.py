@@ -140,14 +140,16 @@ def test_a_histogram_that_does_not_add_up_fails_the_call(T):
         np.testing.assert_array_equal(ctx.count_auto(d, b), oracle.count_auto(w.data, w.edges, THREADS))
 
 
-def test_counted_overflow_at_1m_covers_every_draw_phase(T):
-    # 1.9e6 items against 64 x 2432 late items: the walk-order middle of the range runs too, so
-    # an item the draw order dropped or counted twice would make the checked call fail
+@pytest.mark.parametrize("shape", [{}, dict(threads=512, ipt=8)], ids=["default", "fp32"])
+def test_counted_overflow_at_1m_covers_every_draw_phase(T, shape):
+    # FP32 kernel: 1.9e6 items against 64 x 2432 late items, so the walk-order middle of the range
+    # runs too; an item that either kernel's draws dropped or counted twice would make the checked
+    # call fail
     w = synth.octant_precision(seed=0, n=1_000_000)
-    with T.Context() as ctx:
+    with T.Context(**shape) as ctx:
         d, r, b = ctx.catalog(w.data), ctx.catalog(w.rand), ctx.bins(w.edges)
         derived = ctx.count_all(d, r, b)
-    with T.Context(flags=T.TPCF_F_CHECK_OVERFLOW) as ctx:
+    with T.Context(flags=T.TPCF_F_CHECK_OVERFLOW, **shape) as ctx:
         d, r, b = ctx.catalog(w.data), ctx.catalog(w.rand), ctx.bins(w.edges)
         counted, st = ctx.count_all(d, r, b, stats=True)
     for a, c in zip(counted, derived):
@@ -156,7 +158,7 @@ def test_counted_overflow_at_1m_covers_every_draw_phase(T):
 
 
 def test_counted_overflow_through_the_job_server(T):
-    # small jobs share the multi-job kernel's steps, the largest runs in preemptible one-job steps
+    # small jobs share steps, a launch each; the largest runs in preemptible steps of its own
     specs = synth.serving_jobs(24, seed=5)
     jobs = [synth.materialise_job(s) for s in specs]
     with T.Context() as lone:

@@ -5,7 +5,7 @@ tpcf_correlate call (larger jobs), whatever else runs beside it; the
 device-memory budget must serialize jobs that do not fit together and refuse
 a job that alone exceeds it; cancel and poll follow their documented states; a
 step whose bounded waits expire fails its jobs with TPCF_ETIMEOUT and leaves the
-device usable; a job whose bins do not fit the multi-job kernel runs alone.
+device usable; a job whose bins fit neither kernel of the steps runs alone.
 """
 import os
 
@@ -203,9 +203,9 @@ def test_mixed_sizes_and_bin_sets(T):
 
 
 def test_a_step_that_times_out_fails_its_jobs_and_the_device_stays_usable(T):
-    """With the test hook that leaves each warp's first tile copy unissued, every
-    step's bounded waits expire: its jobs finish with TPCF_ETIMEOUT (multi-job
-    steps and one-job slices alike), and a fresh server then counts correctly."""
+    """With the test hook that leaves each block's first tile copy unissued, every
+    launch's bounded waits expire: the jobs of its step finish with TPCF_ETIMEOUT,
+    and a fresh server then counts correctly."""
     fp = synth.Footprint("octant")
     small = [octant_job(300 + 50 * k, 600 + 70 * k, 40 + k) for k in range(3)]
     edges = synth.linear_edges(0.0, 10.0, 20)
@@ -223,9 +223,9 @@ def test_a_step_that_times_out_fails_its_jobs_and_the_device_stays_usable(T):
 
 
 def test_a_job_with_too_many_edges_for_the_step_kernel_runs_alone(T):
-    """300 bins do not fit the multi-job kernel's shared-memory histograms: that
-    job is counted alone by its preparation worker while the others share steps;
-    all equal their lone calls."""
+    """300 bins fit the shared memory of neither kernel that steps run: that job is
+    counted alone by its preparation worker while the others share steps; all equal
+    their lone calls."""
     edges_wide = synth.linear_edges(0.0, 3.0, 300)
     edges = synth.linear_edges(0.0, 3.0, 40)
     jobs = [octant_job(4000 + 500 * k, 6000 + 300 * k, 60 + k) for k in range(4)]
@@ -258,5 +258,29 @@ def test_a_small_job_preempts_a_running_large_job(T):
         rb = ctx.poll(jb, len(edges))
     assert rs["submit_ms"] + rs["latency_ms"] < rb["submit_ms"] + rb["latency_ms"]
     for res, want in ((rb, want_big), (rs, want_small)):
+        for name, a in zip(("dd", "dr", "rr", "w"), want):
+            np.testing.assert_array_equal(res[name], a)
+
+
+@pytest.mark.parametrize("case", ["wide", "plain"])
+def test_steps_of_the_fp32_kernel(T, case):
+    """Jobs of 133 to 136 edges, whose histograms leave the tensor-core kernel too small a
+    ring, and all jobs of a binary64 context run in steps of the FP32 kernel: a large job in
+    preemptible ones (a start position within its draw order), which a small job interrupts."""
+    import time
+    edges = synth.linear_edges(0.0, 2.0, 133 if case == "wide" else 30)
+    big = octant_job(700_000, 1_400_000, seed=72)
+    small = octant_job(2000, 4000, seed=73)
+    with T.Context() as lone:
+        want_big = lone.correlate(*big, edges)
+        want_small = lone.correlate(*small, edges)
+    with T.Context(precision=T.TPCF_PLAIN_FP64 if case == "plain" else T.TPCF_SCREEN_RECHECK) as ctx:
+        jb = ctx.submit(*big, edges)
+        time.sleep(0.15)  # the large job is prepared and counting
+        js = [ctx.submit(*small, edges) for _ in range(2)]
+        rs = [ctx.poll(j, len(edges)) for j in js]
+        rb = ctx.poll(jb, len(edges))
+    assert rs[0]["submit_ms"] + rs[0]["latency_ms"] < rb["submit_ms"] + rb["latency_ms"]
+    for res, want in [(rb, want_big)] + [(r, want_small) for r in rs]:
         for name, a in zip(("dd", "dr", "rr", "w"), want):
             np.testing.assert_array_equal(res[name], a)
