@@ -61,9 +61,10 @@ def test_range_ends(T, hi):
     _check(T, d, r, synth.linear_edges(0.0, hi, 7))
 
 
-@pytest.mark.parametrize("flags", [0, 0x10])
+@pytest.mark.parametrize("flags", [0, 0x10, 0x20])
 def test_chunks_of_several_tiles(T, flags):
-    """Large enough for chunks of more than one tile and, with pruning, batched draws."""
+    """Large enough for chunks of more than one tile and, with pruning, batched draws; with a
+    counted overflow row most tiles are whole ones that hold nothing in range."""
     fp = synth.Footprint("sphere")
     d = synth.clustered(30011, 64, 0.5, fp, seed=8)
     r = synth.randoms(41001, fp, seed=9)
