@@ -148,6 +148,18 @@ __device__ __noinline__ bool heavy_item(const WorkDesc& wd, const SubProblem& sp
 // L = kLateRounds and tail = kTailRounds items per warp of the launch (at most
 // n; the constants and the order's length, draw_positions, are in plan.h).
 
+// Out of line, as the merge below: with both inlined at every use the loop over the
+// tiles outgrew the instruction cache, and pruned launches, which are mostly draws,
+// waited for instructions (200,000 + 200,000 points on the sphere to 2 degrees, 512 x 8:
+// 2.94 ms inline, 2.47 ms so; 600,000 + 600,000: 16.3 and 13.6 ms).
+__device__ __noinline__ bool load_item_ool(const WorkDesc& wd, uint32_t q, Cursor& c) {
+    return load_item<false>(wd, q, c);
+}
+template <int T>
+__device__ __noinline__ void merge_hist(HistCol hc, int ne, bool check, unsigned long long* out) {
+    warp_flush_hist<T>(hc, ne, check, out);
+}
+
 // The warp's next item (or part) with countable tiles, drawing again past
 // empty and skipped ones; called by every lane of the warp (lane 0 draws a
 // position from `counter`, the position is broadcast).  A preemptible launch
@@ -181,7 +193,7 @@ __device__ void draw_next(const WorkDesc& wd, Cursor& c, unsigned long long* cou
         else if (p < n) { k = p - L; test = 0; }
         else if (p < parts_at) { k = n - L + (p - n); test = 2; }
         else { k = n - tail + (p - parts_at) / kTailParts; test = 2; }
-        if (!load_item(wd, (uint32_t)(wd.item_lo + k), c)) continue;
+        if (!load_item_ool(wd, (uint32_t)(wd.item_lo + k), c)) continue;
         if (test != 0 && heavy_item(wd, sub_of(wd, c.sub), c.g.i0, c.g.j0) != (test == 1)) continue;
         if (p >= parts_at) {
             const uint32_t part = (uint32_t)((p - parts_at) % kTailParts), nt = c.g.t_end - c.g.t_first;
@@ -657,7 +669,7 @@ __global__ void __launch_bounds__(T, 1) count_kernel(const __grid_constant__ Wor
             if (sp.row_seg) tgt += (size_t)__ldg(sp.row_seg + g_i0 / kSegAlign) * sp.row_stride;
             if (c_sub != cur_sub || tgt != cur_hist) {
                 if (cur_sub >= 0 && tgt != cur_hist) {
-                    warp_flush_hist<T>(hc, wd.ne, check, cur_hist);
+                    merge_hist<T>(hc, wd.ne, check, cur_hist);
                     inc_bound = 0;
                 }
                 cur_sub = c_sub;
@@ -698,7 +710,7 @@ __global__ void __launch_bounds__(T, 1) count_kernel(const __grid_constant__ Wor
         // batches), so at most 2 R J + 1; after the tile, the R J and the
         // batches that actually ran are added to the bound
         if (inc_bound + 2u * R * wd.J + 1u > 0xffffu) {
-            warp_flush_hist<T>(hc, wd.ne, check, cur_hist);
+            merge_hist<T>(hc, wd.ne, check, cur_hist);
             inc_bound = 0;
         }
         uint32_t nbatch = 0;
@@ -858,7 +870,7 @@ __global__ void __launch_bounds__(T, 1) count_kernel(const __grid_constant__ Wor
     }
     // ---- merge this warp's columns (skipped after an abort: outputs are invalid)
     if (!aborted && cur_sub >= 0) {
-        warp_flush_hist<T>(hc, wd.ne, check, cur_hist);
+        merge_hist<T>(hc, wd.ne, check, cur_hist);
     }
     if constexpr (!PLAIN) {
         const unsigned long long b = warp_sum(band_cnt), mm = warp_sum(mism_cnt);

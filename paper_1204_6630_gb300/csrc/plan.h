@@ -35,15 +35,13 @@ __host__ __device__ inline uint64_t first_chunk_prefix(uint64_t ib, uint32_t I, 
     }
     const uint64_t m = Jc / I;
     uint64_t Q, Rm;
-    if ((m & (m - 1)) == 0) {  // (kernel shapes: shifts instead of 64-bit divisions)
-        int sh = 0;
-        while ((1ull << sh) < m) ++sh;
-        Q = ib >> sh;
-        Rm = ib & (m - 1);
-    } else {
-        Q = ib / m;
-        Rm = ib % m;
-    }
+#ifdef __CUDA_ARCH__  // (kernel shapes: I and Jc are powers of two)
+    Q = ib >> (31 - __clz((int)m));
+    Rm = ib & (m - 1);
+#else
+    Q = ib / m;
+    Rm = ib % m;
+#endif
     return m * (Q * (Q - 1) / 2) + Q * Rm;
 }
 
