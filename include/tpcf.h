@@ -493,12 +493,21 @@ int tpcf_count_auto_noalloc(const double *xyz_dev, uint64_t n, const double *edg
  *
  * tpcf_debug_noalloc_grid: caps the number of blocks of the counting launch of
  * tpcf_count_auto_noalloc (0 = the default, 8 per SM), so that a test can make
- * one block count more than 2^32 pairs. */
+ * one block count more than 2^32 pairs.
+ *
+ * tpcf_debug_screen_values (GPU): the values by which the tensor-core kernel
+ * rejects, of the 128 points of block a_block of one catalog against those of
+ * block b_block of another (of the same kind; in device order, the input's with
+ * TPCF_F_NO_SORT): values[128 * i + j], approximating a.b, or in 3-D (a.b -
+ * |b|^2 / 2) / 2^(ka + kb) with 2^ka, 2^kb the catalogs' scales, and
+ * maxima[4 * i + q] over j = 32 q .. 32 q + 31.  Host arrays. */
 int64_t tpcf_plan_coverage(uint32_t na, uint32_t nb, int auto_mode, uint32_t I, uint32_t Jc,
                            uint32_t J, uint32_t shard_index, uint32_t shard_count, uint32_t *counts,
                            uint64_t *pairs);
 void tpcf_debug_fail_alloc_after(int n);
 void tpcf_debug_noalloc_grid(int blocks);
+int tpcf_debug_screen_values(tpcf_ctx *ctx, const tpcf_catalog *a, const tpcf_catalog *b, uint32_t a_block,
+                             uint32_t b_block, float *values, float *maxima);
 
 #ifdef __cplusplus
 }

@@ -191,10 +191,8 @@ __device__ __forceinline__ void tc_commit(uint64_t* bar) {
                  : "memory");
 }
 
-// Maximum over 32 columns of the lane's accumulator row (the loaded values
-// themselves are not used).  The result is valid after tc_wait_ld.
-__device__ __forceinline__ float tc_row_max32(uint32_t addr) {
-    [[maybe_unused]] uint32_t r[32];
+// 32 columns of the lane's accumulator row and their maximum, valid after tc_wait_ld.
+__device__ __forceinline__ float tc_row_max32(uint32_t addr, uint32_t (&r)[32]) {
     float m;
     asm volatile(
         "tcgen05.ld.red.sync.aligned.32x32b.x32.max.f32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
@@ -207,9 +205,25 @@ __device__ __forceinline__ float tc_row_max32(uint32_t addr) {
         : "r"(addr));
     return m;
 }
-// Waits for the warp's tensor-memory loads; the operands tie the loaded maxima to the wait.
+// The maximum alone.
+__device__ __forceinline__ float tc_row_max32(uint32_t addr) {
+    [[maybe_unused]] uint32_t r[32];
+    return tc_row_max32(addr, r);
+}
+// Waits for the warp's tensor-memory loads; the operands tie the loaded values to the wait.
 __device__ __forceinline__ void tc_wait_ld(float& a, float& b) {
     asm volatile("tcgen05.wait::ld.sync.aligned;" : "+f"(a), "+f"(b)::"memory");
+}
+
+__device__ __forceinline__ void tc_wait_ld(float& m, uint32_t (&r)[32]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+f"(m), "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]),
+                   "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14])
+                 :: "memory");
+    asm volatile("" : "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]),
+                      "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]),
+                      "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
+                 :: "memory");
 }
 
 // Bounded wait of a whole warp for phase `parity` of `bar`: false (with the
@@ -239,6 +253,18 @@ __device__ __forceinline__ bool tc_wait(uint64_t* bar, uint32_t parity, uint64_t
                                         unsigned long long* stats) {
     if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
     return tc_wait_slow(bar, parity, limit_ns, ctl, stats);
+}
+
+// The i-side operand's planes X and Y of a catalog's operand record x: X (3-D: without
+// the norm), and the halves' two triples exchanged (3-D: then the scales' ratio).
+template <bool EUCLID>
+__device__ __forceinline__ uint4 plane_x(const uint4& x) {
+    return EUCLID ? make_uint4(x.x, x.y, x.z, 0u) : x;
+}
+template <bool EUCLID>
+__device__ __forceinline__ uint4 plane_y(const uint4& x, uint32_t pad) {
+    return make_uint4((x.y >> 16) | (x.z << 16), (x.z >> 16) | (x.x << 16), (x.x >> 16) | (x.y << 16),
+                      EUCLID ? pad : 0u);
 }
 
 // A sphere that holds the (non-empty) spheres of an item's groups: centre the
@@ -785,10 +811,8 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
 #pragma unroll
                         for (int k = 0; k < 8; ++k) {
                             uint4* const p = dst + (gg + k / 4) * (kABlock / 16) + 32 * (k % 4) + lane;
-                            p[0] = EUCLID ? make_uint4(x[k].x, x[k].y, x[k].z, 0u) : x[k];
-                            // Y: the halves' two triples exchanged
-                            p[kBlk] = make_uint4((x[k].y >> 16) | (x[k].z << 16), (x[k].z >> 16) | (x[k].x << 16),
-                                                 (x[k].x >> 16) | (x[k].y << 16), EUCLID ? sp.tc_pad : 0u);
+                            p[0] = plane_x<EUCLID>(x[k]);
+                            p[kBlk] = plane_y<EUCLID>(x[k], sp.tc_pad);
                         }
                     }
                     fence_proxy_async_smem();  // the products read it through the asynchronous proxy
@@ -861,6 +885,61 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
     if (warp == kIssueWarp) tc_dealloc(tmem);
 }
 
+// ============================================================== the screen's values
+// A self-check: the accumulators of one product of 128 i-points and 128 j-points (values: 128
+// rows of 128) and the maxima of 32 that the kernel above compares (maxima: 128 rows of 4), by its
+// instructions.  One block of four warps.
+template <bool EUCLID>
+__global__ void __launch_bounds__(128, 1) screen_values_kernel(const unsigned char* a, const unsigned char* b,
+                                                               uint32_t pad, uint64_t limit_ns, float* values,
+                                                               float* maxima, unsigned long long* err) {
+    __shared__ __align__(128) unsigned char op[kABlock + 2 * kBlkX];
+    __shared__ __align__(8) uint64_t bar;
+    __shared__ uint32_t tmem_word;
+    const uint32_t t = threadIdx.x, warp = t >> 5;
+    {
+        const uint4 x = __ldg(reinterpret_cast<const uint4*>(a) + t), y = __ldg(reinterpret_cast<const uint4*>(b) + t);
+        uint4* const p = reinterpret_cast<uint4*>(op) + t;
+        p[0] = plane_x<EUCLID>(x);
+        p[kBlk] = plane_y<EUCLID>(x, pad);
+        p[2 * kBlk] = y;
+        p[3 * kBlk] = y;
+        fence_proxy_async_smem();
+    }
+    if (t == 0) {
+        mbar_init(&bar, 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
+    if (warp == 0) tc_alloc(smem_addr(&tmem_word));
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&tmem_word);
+    if (t == 0) {
+        tc_mma(tmem, op_desc(smem_addr(op), kBlkX), op_desc(smem_addr(op) + kABlock, kBlkX));
+        tc_commit(&bar);
+    }
+    const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&bar, 0u, limit_ns));
+    if (ok) {
+        tc_fence_after();
+        for (uint32_t q = 0; q < 4; ++q) {
+            uint32_t r[32];
+            float m = tc_row_max32(tmem + (warp << 21) + 32u * q, r);
+            tc_wait_ld(m, r);
+            maxima[4u * t + q] = m;
+#pragma unroll
+            for (int k = 0; k < 32; ++k) values[128u * t + 32u * q + (uint32_t)k] = __uint_as_float(r[k]);
+        }
+        tc_fence_before();
+    } else if ((t & 31u) == 0u) {
+        atomicOr(err, (unsigned long long)kErrWaitTimeout);
+    }
+    __syncthreads();
+    tc_fence_after();
+    if (warp == 0) tc_dealloc(tmem);
+}
+
 template <bool PREEMPT, bool PRUNE, bool EUCLID, bool CHECK = false>
 cudaError_t launch_tc_t(const WorkDesc& wd_in, const Shape& sh, cudaStream_t stream) {
     WorkDesc wd = wd_in;
@@ -904,6 +983,14 @@ cudaError_t count_tc_set_smem_limit() {
     for (const void* k : kernels)
         if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, optin);
     return e;
+}
+
+cudaError_t launch_screen_values(const unsigned char* a_blk, const unsigned char* b_blk, bool euclid, uint32_t pad,
+                                 uint64_t limit_ns, float* values, float* maxima, unsigned long long* err,
+                                 cudaStream_t stream) {
+    if (euclid) screen_values_kernel<true><<<1, 128, 0, stream>>>(a_blk, b_blk, pad, limit_ns, values, maxima, err);
+    else screen_values_kernel<false><<<1, 128, 0, stream>>>(a_blk, b_blk, pad, limit_ns, values, maxima, err);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_count_tc(const WorkDesc& wd, const Shape& sh, bool preempt, cudaStream_t stream) {

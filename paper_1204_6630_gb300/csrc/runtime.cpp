@@ -1606,6 +1606,37 @@ uint64_t tpcf::serving_positions(const Shape& sh, uint64_t n, uint32_t warps) {
     return sh.tc ? n : draw_positions(n, warps);
 }
 
+// ====================================================================== self-check
+// Test hook: the tensor-core screen's values of one block of either catalog.
+extern "C" int tpcf_debug_screen_values(tpcf_ctx* ctx, const tpcf_catalog* a, const tpcf_catalog* b, uint32_t a_block,
+                                        uint32_t b_block, float* values, float* maxima) {
+    if (!ctx) return TPCF_EINVAL;
+    if (!a || !b || !values || !maxima || a->ctx != ctx || b->ctx != ctx || a->euclid != b->euclid ||
+        a_block >= a->n_pad / kBlk || b_block >= b->n_pad / kBlk)
+        return ctx->fail(TPCF_EINVAL, "screen values: bad argument");
+    SubProblem sp;
+    memset(&sp, 0, sizeof sp);
+    if (a->euclid && !tc_screen_3d(SubSpec{a, b, false, (uint32_t)a->n, (uint32_t)b->n, 0, 0}, INFINITY, &sp))
+        return ctx->fail(TPCF_EINVAL, "screen values: the catalogs' scales differ too much");
+    cudaSetDevice(ctx->cfg.device);
+    constexpr size_t kV = 128 * 128, kM = 128 * 4;
+    float* d = nullptr;
+    if (dev_malloc(ctx, (void**)&d, (kV + kM) * 4 + 8) != cudaSuccess)
+        return ctx->fail(TPCF_ENOMEM, "screen values: allocation failed");
+    unsigned long long* derr = (unsigned long long*)(d + kV + kM);
+    unsigned long long err = 0;
+    const bool ok = cudaMemset(derr, 0, 8) == cudaSuccess &&
+                    launch_screen_values(a->blk + (size_t)a_block * kBlkBytes, b->blk + (size_t)b_block * kBlkBytes,
+                                         a->euclid, sp.tc_pad, (uint64_t)ctx->cfg.wait_timeout_us * 1000ull, d, d + kV,
+                                         derr, 0) == cudaSuccess &&
+                    cudaMemcpy(values, d, kV * 4, cudaMemcpyDeviceToHost) == cudaSuccess &&
+                    cudaMemcpy(maxima, d + kV, kM * 4, cudaMemcpyDeviceToHost) == cudaSuccess &&
+                    cudaMemcpy(&err, derr, 8, cudaMemcpyDeviceToHost) == cudaSuccess;
+    cudaFree(d);
+    if (!ok) return ctx->fail(TPCF_ECUDA, "screen values: a CUDA call failed");
+    return err ? ctx->fail(TPCF_ETIMEOUT, "screen values: a bounded device wait timed out") : TPCF_OK;
+}
+
 // ====================================================================== counting ABI
 extern "C" int tpcf_count_auto(tpcf_ctx* ctx, const tpcf_catalog* cat, const tpcf_bins* bins,
                                void* stream, uint64_t* hist, int where, tpcf_stats* st) {

@@ -207,6 +207,11 @@ cudaError_t launch_count_preemptible(const WorkDesc& wd, const Shape& sh, cudaSt
 // of 512 i-points x Jc j-points in tiles of kBlk; preempt: draws from
 // wd.pos_lo on, stopping at the yield word.
 cudaError_t launch_count_tc(const WorkDesc& wd, const Shape& sh, bool preempt, cudaStream_t stream);
+// The screen's values of 128 x 128 pairs (one block of either catalog; pad: the scales' ratio of a
+// 3-D pair of catalogs twice, binary16) and their maxima of 32; err: device error word.
+cudaError_t launch_screen_values(const unsigned char* a_blk, const unsigned char* b_blk, bool euclid, uint32_t pad,
+                                 uint64_t limit_ns, float* values, float* maxima, unsigned long long* err,
+                                 cudaStream_t stream);
 size_t count_tc_smem_bytes(int stages, int nedges);
 cudaError_t count_tc_set_smem_limit();
 // count_over = 1: the kernel counted the overflow row (TPCF_F_CHECK_OVERFLOW);

@@ -126,6 +126,7 @@ _SIGS = {
                                             ctypes.POINTER(ctypes.c_uint32), _u64p]),
     "tpcf_debug_fail_alloc_after": (None, [ctypes.c_int]),
     "tpcf_debug_noalloc_grid": (None, [ctypes.c_int]),
+    "tpcf_debug_screen_values": (ctypes.c_int, [_vp, _vp, _vp, ctypes.c_uint32, ctypes.c_uint32, _vp, _vp]),
     "tpcf_fp32_peak": (ctypes.c_int, [ctypes.c_int, ctypes.c_int, _dp]),
     "tpcf_count_auto_noalloc": (ctypes.c_int, [_vp, _u64, _dp, ctypes.c_int, _vp, _vp]),
     "tpcf_jackknife": (ctypes.c_int, [_vp, _vp, _vp, _vp, _vp, ctypes.c_int, _u64p, _dp, _dp,
@@ -551,6 +552,14 @@ def tpcf_debug_fail_alloc_after(n: int) -> None:
 
 def tpcf_debug_noalloc_grid(blocks: int) -> None:
     load().tpcf_debug_noalloc_grid(blocks)
+
+
+def tpcf_debug_screen_values(ctx: int, a: int, b: int, a_block: int = 0, b_block: int = 0):
+    """(values, maxima) of the tensor-core screen for one block of either catalog (see include/tpcf.h)."""
+    values, maxima = np.empty((128, 128), np.float32), np.empty((128, 4), np.float32)
+    _check(load().tpcf_debug_screen_values(ctx, a, b, a_block, b_block, values.ctypes.data, maxima.ctypes.data),
+           "tpcf_debug_screen_values", ctx)
+    return values, maxima
 
 
 def tpcf_fp32_peak(device: int = 0, packed: bool = False) -> float:
