@@ -144,7 +144,8 @@ typedef struct tpcf_config {
     uint32_t shard_count;      /* number of shards (0 or 1 = no split); histograms of all
                                   shards sum to the unsplit result exactly (shards of one
                                   configuration, counting the same catalogs and bins) */
-    uint32_t wait_timeout_us;  /* limit of every device-side wait; 0 -> 2,000,000 us */
+    uint32_t wait_timeout_us;  /* limit of every device-side wait (of time in which its block makes no
+                                  progress); 0 -> 2,000,000 us */
     int server_workers;        /* job server: jobs admitted at once (slots: catalogs resident on the
                                   device, work in the running steps) (0 -> 32) */
 } tpcf_config;

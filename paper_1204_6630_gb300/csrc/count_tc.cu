@@ -76,8 +76,8 @@ constexpr uint32_t kStageX2 = kBlkBytes;          // a stage: the tile's block (
 constexpr uint32_t kStageBytes = kBlkBytes + kBlkX;
 constexpr int kQueueCodes = 64;                   // per-warp queue of unsettled pairs
 
-// Control words.  kTcBeat changes with every batch of items the loader draws:
-// a wait is bounded by the time without progress.
+// Control words.  kTcBeat changes with every batch of items the loader draws and with
+// whatever the warps classify (tc_beat): a wait is bounded by the time without progress.
 enum TcCtl { kTcAbort = 0, kTcTmem = 1, kTcBeat = 2, kTcCtlWords = 32 };
 
 // A staged tile: what to do with it, first j of the tile, first i of the item.
@@ -226,9 +226,14 @@ __device__ __forceinline__ void tc_wait_ld(float& m, uint32_t (&r)[32]) {
                  :: "memory");
 }
 
+// Says that the block makes progress (a clock: any other value than before will do).
+__device__ __forceinline__ void tc_beat(const WorkDesc& wd) {
+    sptr<volatile int>(wd.off_ctl)[kTcBeat] = (int)clock();
+}
+
 // Bounded wait of a whole warp for phase `parity` of `bar`: false (with the
-// block's abort word and the call's error word set) after limit_ns in which the
-// loader drew nothing, and false as soon as another warp has aborted.
+// block's abort word and the call's error word set) after limit_ns in which
+// nothing was drawn or classified, and false as soon as another warp has aborted.
 __device__ __noinline__ bool tc_wait_slow(uint64_t* bar, uint32_t parity, uint64_t limit_ns, volatile int* ctl,
                                           unsigned long long* stats) {
     uint64_t t0 = global_ns();
@@ -354,6 +359,7 @@ template <bool EUCLID>
 __device__ __forceinline__ void tc_drain(const WorkDesc& wd, const SubProblem& sp, const uint32_t* q, uint32_t n,
                                          u64 ax, u64 ay, u64 az, uint32_t iw, uint32_t jq0, const HistCol& hc,
                                          uint32_t& band, uint32_t& mism) {
+    tc_beat(wd);
     const uint32_t lane = threadIdx.x & 31u;
     const bool has = lane < n;
     const uint32_t code = has ? q[lane] : 0u;
@@ -573,6 +579,7 @@ __global__ void __launch_bounds__(kThreads, 1) count_tc_kernel(const __grid_cons
                 }
                 // most tiles hold nothing within the range: on to the next
                 if (kept != 0u || check) {
+                    tc_beat(wd);
                     // a lane's counter gains at most one per pair of the tile and one per queue batch
                     // (one batch more when the queue is emptied at the item's end)
                     if (inc_bound + 2u * kBlk + 2u > 0xffffu || over > 0x40000000u) flush();

@@ -92,3 +92,17 @@ def test_ring_depths(T, nedges):
     d = synth.clustered(2003, 8, 0.5, seed=nedges)
     r = synth.randoms(9001, seed=nedges + 1)
     _check(T, d, r, synth.linear_edges(0.0, 20.0, nedges - 1))
+
+
+def test_a_short_wait_limit_outlasts_slow_tiles(T):
+    """Points a few arc seconds apart: nearly every pair goes to binary64 and a tile takes
+    milliseconds.  The limit of the device's waits counts time without progress, so one far
+    shorter than a tile still holds."""
+    d = synth.randoms(20000, synth.Footprint("sphere"), seed=5)
+    c = np.array([0.48, 0.6, 0.64])
+    d = c + 1e-5 * d
+    d /= np.linalg.norm(d, axis=1)[:, None]
+    edges = np.linspace(0.0, 2e-5, 100)
+    with T.Context(wait_timeout_us=300) as ctx:
+        got = ctx.count_auto(ctx.catalog(d), ctx.bins(edges))
+    np.testing.assert_array_equal(got, oracle.count_auto(d, edges, THREADS))
