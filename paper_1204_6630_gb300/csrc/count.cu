@@ -432,10 +432,11 @@ __device__ __forceinline__ uint32_t slow_group(const WorkDesc& wd, const u64 (&a
     return um;
 }
 
-// ---- all-binary64 mode: comparisons on the integer units.  order_key(a) <
-// order_key_thr(b) exactly when a < b, >= exactly when a >= b (no NaN): the bits
-// as a signed integer, the magnitude bits flipped below zero; a threshold of -0
-// counts as +0.
+// ---- all-binary64 mode: comparisons on the integer units.  order_key(a) >
+// order_key_thr(b) exactly when a > b, <= exactly when a <= b (no NaN); < and >=
+// likewise for an a that is not -0 (a squared distance): the bits as a signed
+// integer, the magnitude bits flipped below zero; a threshold of -0 counts as +0,
+// a value of -0 lies below it.
 // The binary64 unit is the bound, and a comparison there costs as much as a
 // product (six operations a pair with it, five without): 30,011 + 30,011 points
 // on an octant 28.7 -> 26.0 ms with four warps an SM, 17.5 ms with sixteen.
@@ -1007,8 +1008,9 @@ static cudaError_t set_smem_t(size_t bytes) {
                                 optin);
 }
 
-// The job server's jobs whose histograms do not fit the tensor-core kernel: the 512 x 8 screen kernel with preemptible
-// draws (a start position and the yield word).
+// The job server's steps of jobs whose histograms do not fit the tensor-core
+// kernel (133 to 136 edges) and of binary64 contexts: the 512 x 8 screen kernel
+// with preemptible draws (a start position and the yield word).
 cudaError_t launch_count_preemptible(const WorkDesc& wd, const Shape& sh, cudaStream_t stream) {
     if (sh.threads != 512 || sh.ipt != 8) return cudaErrorInvalidConfiguration;
     return launch_t<512, 8, kModeScreen, true>(wd, sh, stream);

@@ -17,7 +17,8 @@
 // binary16 values are exact in binary32; with accumulation in at least single
 // precision D is within 44u of the binary64 dot d (u = 2^-24: 2u from the FP32
 // copies, 9.8u from the split, at most one unit 2u in the last place for each
-// of 16 additions of partial sums below 1.002).  A block is rejected when
+// of 16 additions of partial sums below 1.002; measured, through
+// tpcf_debug_screen_values: at most 4.3u).  A block is rejected when
 // every D < tc_thr = RD(C_B - 64u), which proves d < C_B for all its pairs.
 //
 // 3-D counts (EUCLID) reject on D = a.b - |b|^2 / 2: d^2 >= S_B is D <= (|a|^2 -
@@ -28,9 +29,10 @@
 // Error with t = max(s, 1/s): 2u and 9.8u as above, 5u s from |b|^2 / 2 (three
 // roundings, the copies, the split), 16 additions of partial sums below 2t at 2u t,
 // 8u t from the threshold (three roundings of |a|^2 / 2s, the copies, the last
-// addition where the screen rejects anything): 57u t in all, kTcGuard3d = 128u.
-// 300,000 + 300,000 points, distances to 0.05 of the box: 11.5 ms (FP32
-// differences on the CUDA cores: 33.5 ms, bound by their nine operations a pair).
+// addition where the screen rejects anything): 57u t in all, kTcGuard3d = 128u
+// (measured without the threshold's part: at most 2.5u t).
+// 300,000 + 300,000 points, distances to 0.05 of the box: 11.2 ms (FP32
+// differences on the CUDA cores: 33.2 ms, bound by their nine operations a pair).
 //
 // One CTA per SM, 21 warps:
 //   * warps 0..15, four groups of four: group g reads the accumulators of
@@ -44,17 +46,18 @@
 // four groups; a group that is busy classifying holds back its own
 // accumulators only, and the others run up to the ring's depth ahead.
 //
-// What bounds it (octant of 1,000,000 + 1,000,000 points to 10 degrees 213 ms, the
-// FP32 screen of count.cu 296 ms; sphere of 700,001 x 1,400,003 to 2 degrees 50.4 ms,
-// there 110.8 ms):
+// What bounds it (octant of 1,000,000 + 1,000,000 points to 10 degrees 206 ms, the
+// FP32 screen of count.cu 284 ms; sphere of 700,001 x 1,400,003 to 2 degrees 50.4 ms,
+// there 108 ms):
 //   * a rejected tile of 512 x 128 pairs takes about 1050 cycles.  The tensor core
 //     needs 128 of them and reading the accumulators 344; the rest is the chain
 //     from one product of a group to the next (product, commit, wait, load, vote,
 //     arrival, wait): tensor memory holds one product of each group, so a group
 //     has nothing else to do meanwhile;
-//   * a kept 32 x 32 block takes about 2600 cycles of its warp and, with all warps
-//     at it, the shared-memory pipe: a lookup of 32 random cells is 3.9 wavefronts,
-//     with the counter 5.6 for 32 pairs.
+//   * a kept 32 x 32 block takes about 2800 cycles of its warp, its unsettled pairs
+//     500 (patches of close points: 1600), and, with all warps at it, the
+//     shared-memory pipe: a lookup of 32 random cells is 3.9 wavefronts, with the
+//     counter and the j-points 5.6 for 32 pairs.
 #include <stdint.h>
 
 #include "count_common.cuh"

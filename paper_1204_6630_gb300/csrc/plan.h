@@ -59,8 +59,9 @@ __host__ __device__ inline uint64_t row_start(uint64_t ib, uint32_t n_jchunk, ui
 }
 
 // A single-precision root of S's quadratic (F(ib) is near k ib (ib - 1) / 2, k =
-// I / Jc), then exact steps, one or two: the shorter way for one item (20,011
-// points: 119 us against 127 with the search).
+// I / Jc), then exact steps to the row: a few, but up to some hundred in the last
+// rows of the largest catalogs, where the discriminant cancels.  The shorter way
+// for one item (20,011 points: 119 us against 127 with the search).
 __host__ __device__ inline uint64_t row_by_root(uint64_t local, uint32_t n_iblk, uint32_t n_jchunk, uint32_t I,
                                                 uint32_t Jc) {
     const float k = (float)I / (float)Jc, h = (float)n_jchunk + 0.5f * k;

@@ -1,7 +1,8 @@
 // CUDA kernels (sm_103a) of catalog preparation: validation of the input
 // points, a space-filling-curve sort, and the device copies the counting
-// kernel reads (binary64 points, FP32 points as float4 and as x | y | z
-// arrays, bounding spheres per 128 points).
+// kernels read (binary64 points; blocks of 128 points that hold their
+// tensor-core operand records and FP32 x | y | z arrays; bounding spheres per
+// 128 and per 4096 points).
 //
 // Paper: Ponce et al., "Application of GPUs for the calculation of two point
 // correlation functions in cosmology", Section 3 (the pair angle follows from

@@ -967,8 +967,9 @@ bool shape_for(tpcf_ctx* ctx, int mode, int nedges, int T, int R, int Jreq, int 
 // that the launch's last items are a small part of it; a small problem is cut
 // down to one tile (512 x 128 pairs) per item (auto count of 20,011 points: 147 us
 // with items of 1024, 123 us so; 8,192 + 8,192 points: 101 us, 600 us on the FP32
-// kernel's 128 x 8 shape).  False when the histograms do
-// not leave shared memory for a ring of four stages.
+// kernel's 128 x 8 shape).  The ring has eight stages up to 110 edges, six up to 121
+// and four up to 132; false for more, whose histograms (1 KB an edge) leave too
+// little shared memory.
 bool tc_shape_for(tpcf_ctx* ctx, int nedges, uint64_t total_pairs, Shape* sh) {
     constexpr uint64_t kTcItemsPerSm = 8;
     int S = 8;
@@ -994,7 +995,7 @@ bool tc_shape_for(tpcf_ctx* ctx, int nedges, uint64_t total_pairs, Shape* sh) {
 // range (points far from the origin for their separations) or the catalogs'
 // scales differ too much.  The FP32 kernel, whose value is a difference of
 // coordinates, has no such band (300,000 + 300,000 points in a box of 1000,
-// distances to 50, band 0.03 of the range: 11.5 ms here, 33.5 ms there).
+// distances to 50, band 0.03 of the range: 11.2 ms here, 33.2 ms there).
 bool tc_screen_3d(const SubSpec& p, double S_B, SubProblem* sp) {
     if (p.na == 0 || p.nb == 0) return true;
     const int ka = p.a->tc_exp, kb = p.b->tc_exp, r = kb - ka;
@@ -1042,9 +1043,11 @@ bool plain_shape(tpcf_ctx* ctx, int nedges, uint64_t total_pairs, Shape* sh) {
 }
 
 // Default shape: the tensor-core kernel wherever its screen applies (octant of
-// 1,000,000 + 1,000,000 points: 213 ms, 296 ms on the FP32 kernel; 512 patches: 56
-// and 63 ms; 8,192 + 8,192 points: 0.10 and 0.60 ms); a caller's own shape is the
-// FP32 kernel's.  There 512 x 8 for large problems, smaller blocks when the
+// 1,000,000 + 1,000,000 points: 206 ms, 284 ms on the FP32 kernel; 512 patches of
+// 2,000,000 + 4,000,000: 44.6 and 47.7 ms; 8,192 + 8,192 points: 0.10 and 0.60 ms).
+// Where nearly every pair of large catalogs is in range the FP32 kernel is up to 7%
+// ahead (200,000 + 200,000 on the sphere to 180 degrees: 59.6 and 55.7 ms), which
+// neither sizes nor bins tell.  A caller's own shape is the FP32 kernel's.  There 512 x 8 for large problems, smaller blocks when the
 // catalogs (or sub-ranges) are small or the per-thread histograms do not fit.
 bool choose_shape(tpcf_ctx* ctx, int mode, bool tc, int nedges, uint64_t total_pairs, uint64_t max_n, Shape* sh) {
     const tpcf_config& cfg = ctx->cfg;

@@ -401,7 +401,7 @@ class JobServer {
     }
 
     // Catalogs, bins, accumulators and the work description of a job (its own
-    // stream, synchronously); a job whose histograms do not fit the step kernel
+    // stream, synchronously); a job whose histograms fit neither kernel of the steps
     // is counted here alone.
     int prepare(Job& j, cudaStream_t st) {
         const int ne = (int)j.edges.size();

@@ -36,7 +36,8 @@ constexpr double kTcGuard = 64.0 * 5.9604644775390625e-08;
 constexpr double kTcGuard3d = 128.0 * 5.9604644775390625e-08;
 constexpr int kTcMaxRatio = 10;  // |log2 s| at most: s is a binary16 operand
 
-// Smallest k with 2^k >= sqrt(norm2) (at least -100: its scale is an FP32 number).
+// A k with 2^k >= sqrt(norm2): the smallest, or one more where norm2 is an even power of
+// two (at least -100: its scale is an FP32 number).
 __host__ __device__ inline int tc_exponent(unsigned long long norm2_bits) {
     const int e = (int)((norm2_bits >> 52) & 0x7ffu) - 1023;  // norm2 < 2^(e + 1)
     if (norm2_bits == 0ull) return 0;
@@ -203,8 +204,8 @@ cudaError_t launch_count(const WorkDesc& wd, const Shape& sh, int mode, int nedg
 // A served job with histograms too large for the tensor-core kernel (FP32
 // screen of angles, shape 512 x 8): the kernel with preemptible draws (wd.pos_lo, stats[kStatYield]).
 cudaError_t launch_count_preemptible(const WorkDesc& wd, const Shape& sh, cudaStream_t stream);
-// The tensor-core counting kernel (count_tc.cu; FP32 screen of angles): items
-// of 512 i-points x Jc j-points in tiles of kBlk; preempt: draws from
+// The tensor-core counting kernel (count_tc.cu; angles, and distances where
+// its screen applies): items of 512 i-points x Jc j-points in tiles of kBlk; preempt: draws from
 // wd.pos_lo on, stopping at the yield word.
 cudaError_t launch_count_tc(const WorkDesc& wd, const Shape& sh, bool preempt, cudaStream_t stream);
 // The screen's values of 128 x 128 pairs (one block of either catalog; pad: the scales' ratio of a
