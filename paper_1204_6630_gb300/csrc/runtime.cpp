@@ -1047,8 +1047,9 @@ bool plain_shape(tpcf_ctx* ctx, int nedges, uint64_t total_pairs, Shape* sh) {
 // 2,000,000 + 4,000,000: 44.6 and 47.7 ms; 8,192 + 8,192 points: 0.10 and 0.60 ms).
 // Where nearly every pair of large catalogs is in range the FP32 kernel is up to 7%
 // ahead (200,000 + 200,000 on the sphere to 180 degrees: 59.6 and 55.7 ms), which
-// neither sizes nor bins tell.  A caller's own shape is the FP32 kernel's.  There 512 x 8 for large problems, smaller blocks when the
-// catalogs (or sub-ranges) are small or the per-thread histograms do not fit.
+// neither sizes nor bins tell.  A caller's own shape is the FP32 kernel's.  There
+// 512 x 8 for large problems, smaller blocks when the catalogs (or sub-ranges) are
+// small or the per-thread histograms do not fit.
 bool choose_shape(tpcf_ctx* ctx, int mode, bool tc, int nedges, uint64_t total_pairs, uint64_t max_n, Shape* sh) {
     const tpcf_config& cfg = ctx->cfg;
     if (cfg.threads != 0 && cfg.ipt != 0) {
