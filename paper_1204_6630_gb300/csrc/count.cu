@@ -432,11 +432,12 @@ __device__ __forceinline__ uint32_t slow_group(const WorkDesc& wd, const u64 (&a
     return um;
 }
 
-// ---- all-binary64 mode: comparisons on the integer units.  order_key(a) >
-// order_key_thr(b) exactly when a > b, <= exactly when a <= b (no NaN); < and >=
-// likewise for an a that is not -0 (a squared distance): the bits as a signed
-// integer, the magnitude bits flipped below zero; a threshold of -0 counts as +0,
-// a value of -0 lies below it.
+// ---- all-binary64 mode: comparisons on the integer units.  Dot products (finite):
+// order_key(a) > order_key_thr(b) exactly when a > b, <= exactly when a <= b: the
+// bits as a signed integer, the magnitude bits flipped below zero; a threshold of -0
+// counts as +0, a value of -0 lies below it.  Squared distances (+0 and up, or NaN
+// between two padding points of a jackknife's rows): the bits unsigned, in which a NaN
+// of either sign lies above every threshold.
 // The binary64 unit is the bound, and a comparison there costs as much as a
 // product (six operations a pair with it, five without): 30,011 + 30,011 points
 // on an octant 28.7 -> 26.0 ms with four warps an SM, 17.5 ms with sixteen.
@@ -447,6 +448,12 @@ __device__ __forceinline__ long long order_key(double a) {
 __device__ __forceinline__ long long order_key_thr(double a) {
     const long long b = __double_as_longlong(a);
     return (b << 1) == 0 ? 0 : b ^ (long long)((unsigned long long)(b >> 63) >> 1);
+}
+
+__device__ __forceinline__ u64 distance_key(double a) { return (u64)__double_as_longlong(a); }
+__device__ __forceinline__ u64 distance_key_thr(double a) {
+    const u64 b = (u64)__double_as_longlong(a);
+    return (b << 1) == 0ull ? 0ull : b;
 }
 
 // Slow path of the 3-D variant for a group of U j: z = fl32(|a' - b'|^2) is
@@ -737,6 +744,7 @@ __global__ void __launch_bounds__(T, 1) count_kernel(const __grid_constant__ Wor
             const double* cthr = sptr<const double>(wd.off_cthr);
             const int ne = wd.ne;
             const long long last = order_key_thr(wd.cos_last);
+            const u64 last2 = distance_key_thr(wd.cos_last);  // (3-D)
             for (int jj = 0; jj < J; ++jj) {
                 const Point64 b = sj[jj];
                 const uint32_t jg = jbase + (uint32_t)jj;
@@ -749,12 +757,12 @@ __global__ void __launch_bounds__(T, 1) count_kernel(const __grid_constant__ Wor
                         // 3-D: h = number of edges m with d^2 >= S_m (S increasing); d^2 >= S_B is overflow
                         const double ex = __dsub_rn(dx[r], b.x), ey = __dsub_rn(dy[r], b.y), ez = __dsub_rn(dz[r], b.z);
                         const double d2 = __dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)), __dmul_rn(ez, ez));
-                        const long long k2 = order_key(d2);  // (valid pairs are finite)
-                        if (k2 < last && valid) {
+                        const u64 k2 = distance_key(d2);
+                        if (k2 < last2 && valid) {
                             int lo = 0, hi = ne;
                             while (lo < hi) {
                                 const int mid = (lo + hi) >> 1;
-                                if (k2 >= order_key_thr(cthr[mid])) lo = mid + 1; else hi = mid;
+                                if (k2 >= distance_key_thr(cthr[mid])) lo = mid + 1; else hi = mid;
                             }
                             hist_inc<T>(hc, lo);
                         } else if (check && valid) {

@@ -144,3 +144,27 @@ def test_coordinates_near_the_limit(T, precision):
     assert st["device_error"] == 0
     for a, b in zip(got, o3(d, r, edges)):
         np.testing.assert_array_equal(a, b)
+
+
+def test_patches_and_jackknife_3d_in_binary64(T):
+    """The jackknife's rows run over the padding between segments: two padding points are NaN
+    apart, of whichever sign, and not a pair."""
+    sizes = [300, 0, 77, 1, 500, 256]
+    doff = np.concatenate([[0], np.cumsum(sizes)]).astype(np.uint64)
+    roff = 2 * doff
+    d = synth.box_clustered(int(doff[-1]), 20, 2.0, 60.0, 11)
+    r = synth.box_points(int(roff[-1]), 60.0, 12)
+    edges = np.linspace(0.0, 20.0, 13)
+    with T.Context(precision=PLAIN) as ctx:
+        cd, cr, b = ctx.catalog3d(d, offsets=doff), ctx.catalog3d(r, offsets=roff), ctx.bins3d(edges)
+        h = ctx.count_patches(cd, cr, b)
+        loo, w, cov = ctx.jackknife(cd, cr, b)
+    for p in range(len(sizes)):
+        dp, rp = d[int(doff[p]):int(doff[p + 1])], r[int(roff[p]):int(roff[p + 1])]
+        np.testing.assert_array_equal(h[p, 0], oracle.count_auto(dp, edges, THREADS, euclid=True))
+        np.testing.assert_array_equal(h[p, 1], oracle.count_cross(dp, rp, edges, THREADS, euclid=True))
+        np.testing.assert_array_equal(h[p, 2], oracle.count_auto(rp, edges, THREADS, euclid=True))
+    want_loo, want_w, want_cov = oracle.jackknife(d, r, doff, roff, edges, threads=THREADS, euclid=True)
+    np.testing.assert_array_equal(loo, want_loo)
+    np.testing.assert_array_equal(w, want_w)
+    np.testing.assert_array_equal(cov, want_cov)
