@@ -105,7 +105,9 @@ extern "C" {
                                         pair total fails (TPCF_ECUDA, "histogram does not add up";
                                         that histogram's overflow entry is UINT64_MAX), so a pair
                                         the kernel lost cannot hide in overflow.  Slower on tiles
-                                        that meet the diagonal or padding. */
+                                        that meet the diagonal or padding.  Not for tpcf_jackknife,
+                                        whose row totals leave out the alignment padding that the
+                                        kernels then count (TPCF_ECUDA). */
 #define TPCF_F_TEST_WAIT_TIMEOUT 0x100u /* test hook: the first j-tile copy of each counting
                                            launch is never issued, so its bounded wait expires
                                            and the call returns TPCF_ETIMEOUT */
